@@ -16,6 +16,7 @@ decode cases is formed here in fp64 from the code's coefficient matrix, so that 
 """
 import math
 
+import numpy as np
 import torch
 
 import paper_1803_09877_b200 as dr
@@ -215,3 +216,92 @@ def tolerance(case):
     if case["op"] in ("step", "host"):
         return {"rel": min(0.03, 2e-7 + 4e-8 * k), "max": min(1.0, 1e-6 + 2.5e-7 * k)}
     return {"rel": 1e-7 + 1e-16 * k, "max": 4e-7 + 1e-15 * k}
+
+
+def _code_matrix(n, s):
+    """W[j][k] = n^(-1/2) prod (w^k - w^m) over the n - 2 s - 1 columns m outside j .. j + 2 s, zero on those columns."""
+    w = np.exp(np.clongdouble(2j) * np.arccos(np.longdouble(-1)) * np.arange(n) / n)
+    W = np.zeros((n, n), dtype=np.clongdouble)
+    for j in range(n):
+        outside = [(j + t) % n for t in range(2 * s + 1, n)]
+        for k in [(j + t) % n for t in range(2 * s + 1)]:
+            W[j, k] = np.prod(w[k] - w[outside]) / np.sqrt(np.longdouble(n))
+    return W.astype(np.complex128)
+
+
+def _decode_vector(n, s, nodes):
+    """The minimum-norm b, zero on the adversaries, with [C_L] b = (0, .., 0, 1)."""
+    U = [j for j in range(n) if j not in nodes]
+    C = np.exp(2j * np.pi * (np.outer(np.arange(n - 2 * s), U) % n) / n) / math.sqrt(n)
+    last = np.zeros(n - 2 * s, dtype=np.complex128)
+    last[-1] = 1.0
+    b = np.zeros(n, dtype=np.complex128)
+    b[U] = np.linalg.lstsq(C, last, rcond=None)[0]
+    return b
+
+
+def exact(case, seed):
+    """The same in fp64: sums of the inputs by the code's definition, vectors combined with the decode vector of the true
+    adversary set.  Adversaries' Gaussian noise has no counterpart outside the library: no worker vectors then."""
+    n, s, d, v, op = case["n"], case["s"], case["d"], _vlen(case), case["op"]
+    cyc, packed = case["code"] != "rep", case["code"] == "cycp"
+    st = prepare(case, seed)
+    nodes, models, params = _adversaries(case, seed)
+    flags = torch.zeros(n, dtype=torch.uint8)
+    flags[nodes] = 1
+    r = 2 * s + 1
+    sizes = [n // (n // r) + (g < n % (n // r)) for g in range(n // r)]
+    first = [sum(sizes[:g]) for g in range(n // r)]
+    if op in ("decode", "update"):
+        R, u = st["R"], torch.empty(d, dtype=torch.float64, device="cuda")
+        if cyc:
+            honest = [j for j in range(n) if j not in nodes]
+            b = _decode_vector(n, s, nodes)[honest]
+            b = torch.from_numpy(np.stack([b.real, b.imag])).cuda()
+        else:
+            honest = [next(j for j in range(f, f + m) if j not in nodes) for f, m in zip(first, sizes)]
+        for c0 in range(0, v, 1 << 20):
+            c1 = min(v, c0 + (1 << 20))
+            if not cyc:
+                u[c0:c1] = R[honest, c0:c1].double().sum(0)
+                continue
+            x = R.view(n, v, 2)[honest, c0:c1].double()
+            u[c0:c1] = b[0] @ x[..., 0] - b[1] @ x[..., 1]
+            if packed:
+                c2 = min(c1, d - v)
+                u[v + c0:v + c2] = (b[0] @ x[..., 1] + b[1] @ x[..., 0])[: max(c2 - c0, 0)]
+        return flags, u if op == "decode" else st["w"].double() - UPDATE_SCALE * u
+    G = st["G"].cuda()
+    Z = None
+    if op == "encode" or not any(m == MODELS["gauss"][0] for m in models):
+        Z = torch.empty((n, 2 * v if cyc else v), dtype=torch.float64, device="cuda")
+        W = torch.from_numpy(_code_matrix(n, s)).cuda() if cyc else None
+        for c0 in range(0, v, 1 << 20):
+            c1 = min(v, c0 + (1 << 20))
+            g = G[:, c0:c1].double()
+            if not cyc:
+                for f, m in zip(first, sizes):
+                    Z[f:f + m, c0:c1] = g[f:f + m].sum(0)
+            else:
+                Wr, Wi, out = W.real.t().contiguous(), W.imag.t().contiguous(), Z.view(n, v, 2)[:, c0:c1]
+                zr, zi = Wr @ g, Wi @ g
+                if packed:
+                    h = torch.zeros_like(g)
+                    c2 = min(c1, d - v)
+                    h[:, : c2 - c0] = G[:, v + c0:v + c2]
+                    zr, zi = zr - Wi @ h, zi + Wr @ h
+                out[..., 0], out[..., 1] = zr, zi
+        if op != "encode":
+            for j, model, param in zip(nodes, models, params):
+                if model == MODELS["revgrad"][0]:
+                    Z[j] *= -param
+                else:
+                    Z[j] = param
+                    if cyc:
+                        Z[j, 1::2] = 0.0
+    if op == "encode":
+        return Z
+    u = torch.empty(d, dtype=torch.float64, device="cuda")
+    for c0 in range(0, d, 1 << 20):
+        u[c0:c0 + (1 << 20)] = G[:, c0:c0 + (1 << 20)].double().sum(0)
+    return Z, flags, u
