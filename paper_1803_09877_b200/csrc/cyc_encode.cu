@@ -277,7 +277,155 @@ cyc_encode_stream_kernel(const float* __restrict__ G, float2* __restrict__ Z, in
     cp_async_wait<0>();
 }
 
-// Any s, any length / alignment: one coordinate per thread, rows re-read through the caches,
+// Rows of any alignment and length, 1 <= s <= 7: the same walk with two coordinates kThreads apart (packed: one complex
+// coordinate) per thread, so that a warp's 4-byte loads and 8-byte stores are contiguous wherever a row starts, and everything
+// in fp64.  A thread keeps the last 2 s + 1 rows as fp64 in a register window and fetches each row 2 s + 1 steps ahead, into
+// the register that the step just freed; the first 2 s rows stay in shared memory for the end of the walk.
+//
+// Row j of Z starts anywhere relative to a 32-byte sector.  A block computes kAlign coordinates more than it writes and writes
+// of each row the run that starts on a sector, so that no sector is shared between blocks: shared ones left L2 half written
+// (n = 45, s = 1, d = 60.2 M + 1: 12.1 ms with plain strips, 8.3 ms so).  Two coordinates per thread instead of one take the
+// instructions per output from 61 to about 46 (s = 5: 8.3 -> 7.5 ms; s = 1: 8.3 -> 6.9 ms), and a barrier per 2 s + 1 rows
+// keeps a block's warps on neighbouring addresses (s = 5: 7.8 -> 7.5 ms).  What is left is latency: 16 to 24 warps per SM, fp64
+// pipe half busy.  Against the one-coordinate-per-thread kernel below, which re-reads every row 2 s + 1 times through the
+// caches: n = 45, s = 3, d = 3,000,017: 1130 -> 347 us (4.7 TB/s).
+template <int S, bool PACKED>
+struct FirCfg {
+    static constexpr int R = 2 * S + 1;
+    static constexpr int C = PACKED ? 1 : 2;                       // output coordinates per thread, kThreads apart
+    static constexpr int NI = 2;                                   // real inputs per thread and row
+    static constexpr int kThreads = 128;
+    static constexpr int kAlign = 4;                               // complex entries per 32-byte sector
+    static constexpr int kTile = kThreads * C - kAlign;            // coordinates that a block writes of every row
+    static constexpr int kBlocks = S <= 2 ? 6 : S <= 5 ? 4 : 3;    // per SM, what the registers allow
+};
+
+template <int S, bool PACKED>
+struct FirState {
+    float raw[FirCfg<S, PACKED>::R][FirCfg<S, PACKED>::NI];        // rows on their way
+    double win[FirCfg<S, PACKED>::R][FirCfg<S, PACKED>::NI];       // rows vv .. vv - 2 S, slot = vv mod R
+    const float* gp;                                               // next row to fetch
+    float2* zp;                                                    // next output row
+    int64_t off1;                                                  // from the first to the second input
+    int shift, dshift;                                             // entries of the next output row before its first sector
+    uint32_t mask[FirCfg<S, PACKED>::C];                           // bit k: this coordinate is written when shift = k
+    bool on1;
+};
+
+template <int S, bool PACKED>
+__device__ __forceinline__ void fir_fetch(FirState<S, PACKED>& w, int p, int64_t ldg) {
+    w.raw[p][0] = __ldcs(w.gp);
+    w.raw[p][1] = w.on1 ? __ldcs(w.gp + w.off1) : 0.0f;
+    w.gp += ldg;
+}
+
+// Step vv of the walk, slot P = vv mod R.  HEAD: the first R steps; TAIL: run-time guards.
+template <int S, int P, bool PACKED, bool HEAD, bool TAIL>
+__device__ __forceinline__ void fir_step(FirState<S, PACKED>& w, int vv, int n, int64_t ldg, int64_t ldz, float* stash,
+                                         const EncodeTaps64& taps, const EncodePhase64& ph) {
+    using Cfg = FirCfg<S, PACKED>;
+    constexpr int R = Cfg::R, NI = Cfg::NI, C = Cfg::C, kT = Cfg::kThreads;
+    if (TAIL && vv >= n + 2 * S) return;
+    if (TAIL && vv >= n) {
+#pragma unroll
+        for (int c = 0; c < NI; ++c) w.win[P][c] = (double)stash[((vv - n) * NI + c) * kT];
+    } else {
+#pragma unroll
+        for (int c = 0; c < NI; ++c) {
+            w.win[P][c] = (double)w.raw[P][c];
+            if (HEAD && P < 2 * S) stash[(P * NI + c) * kT] = w.raw[P][c];
+        }
+        if (vv + R < n) fir_fetch<S, PACKED>(w, P, ldg);
+    }
+    if (HEAD && P < 2 * S) return;
+    double ar[C], ai[C];
+#pragma unroll
+    for (int c = 0; c < C; ++c) ar[c] = ai[c] = 0.0;
+#pragma unroll
+    for (int k = 0; k < R; ++k) {
+        const int t = (k & 1) ? 2 * S - (k >> 1) : (k >> 1);       // small taps first
+        const double cr = taps.tap[t].x, ci = taps.tap[t].y;
+        const double(&x)[NI] = w.win[(P - t + 2 * R) % R];
+#pragma unroll
+        for (int c = 0; c < C; ++c) {
+            ar[c] = fma(cr, x[c], ar[c]);
+            ai[c] = fma(ci, x[c], ai[c]);
+        }
+        if constexpr (PACKED) {
+            ar[0] = fma(-ci, x[1], ar[0]);
+            ai[0] = fma(cr, x[1], ai[0]);
+        }
+    }
+    const double2 rot = ph.phase[TAIL && vv >= n ? vv - n : vv];
+#pragma unroll
+    for (int c = 0; c < C; ++c)
+        if ((w.mask[c] >> w.shift) & 1u)
+            __stcs(w.zp + c * kT, make_float2((float)fma(ar[c], rot.x, -ai[c] * rot.y), (float)fma(ar[c], rot.y, ai[c] * rot.x)));
+    w.zp += ldz;
+    w.shift = (w.shift - w.dshift) & (Cfg::kAlign - 1);
+    if (TAIL && vv == n - 1) {
+        w.zp -= (int64_t)n * ldz;
+        w.shift = (w.shift + n * w.dshift) & (Cfg::kAlign - 1);
+    }
+}
+
+template <int S, bool PACKED, bool HEAD, bool TAIL, int P = 0>
+__device__ __forceinline__ void fir_chunk(FirState<S, PACKED>& w, int v0, int n, int64_t ldg, int64_t ldz, float* stash,
+                                          const EncodeTaps64& taps, const EncodePhase64& ph) {
+    if constexpr (P < FirCfg<S, PACKED>::R) {
+        fir_step<S, P, PACKED, HEAD, TAIL>(w, v0 + P, n, ldg, ldz, stash, taps, ph);
+        fir_chunk<S, PACKED, HEAD, TAIL, P + 1>(w, v0, n, ldg, ldz, stash, taps, ph);
+    }
+}
+
+template <int S, bool PACKED>
+__global__ void __launch_bounds__(FirCfg<S, PACKED>::kThreads, FirCfg<S, PACKED>::kBlocks)
+cyc_encode_fir_kernel(const float* __restrict__ G, float2* __restrict__ Z, int64_t len, int64_t ldg, int64_t ldz,
+                      int64_t half, int64_t d_real, int n, const __grid_constant__ EncodeTaps64 taps,
+                      const __grid_constant__ EncodePhase64 ph) {
+    using Cfg = FirCfg<S, PACKED>;
+    constexpr int R = Cfg::R, C = Cfg::C, kT = Cfg::kThreads, kTile = Cfg::kTile, kAlign = Cfg::kAlign;
+    __shared__ float stash_all[2 * S * Cfg::NI * kT];
+    float* stash = stash_all + threadIdx.x;                        // this thread's column
+    const int64_t nstrips = (len + kTile - 1) / kTile;
+    for (int64_t strip = blockIdx.x; strip < nstrips; strip += gridDim.x) {
+        FirState<S, PACKED> w;
+        const int64_t c0 = strip * kTile, c = c0 + threadIdx.x;
+        w.gp = G + (c < len ? c : c0);                             // threads beyond the vector read their strip's first entry
+        w.off1 = PACKED ? half : kT;
+        w.on1 = PACKED ? (c < len && half + c < d_real) : (c + kT < len);
+        w.zp = Z + c + (int64_t)(2 * S) * ldz;
+        w.dshift = (int)(ldz & (kAlign - 1));
+        w.shift = (int)(-((int64_t)(reinterpret_cast<uintptr_t>(Z) >> 3) + c0 + (int64_t)(2 * S) * ldz)) & (kAlign - 1);
+#pragma unroll
+        for (int q = 0; q < C; ++q) {
+            const int i = threadIdx.x + q * kT;
+            uint32_t m = 0;
+#pragma unroll
+            for (int k = 0; k < kAlign; ++k)
+                if ((i >= k || strip == 0) && i < k + kTile && c0 + i < len) m |= 1u << k;
+            w.mask[q] = m;
+        }
+#pragma unroll
+        for (int p = 0; p < R; ++p) fir_fetch<S, PACKED>(w, p, ldg);       // n >= R
+        fir_chunk<S, PACKED, true, false>(w, 0, n, ldg, ldz, stash, taps, ph);
+        if (n == R) {                                              // the head ended at row n - 1: the next output is row 0
+            w.zp -= (int64_t)n * ldz;
+            w.shift = (w.shift + n * w.dshift) & (kAlign - 1);
+        }
+        int v0 = R;
+        for (; v0 + R < n; v0 += R) {
+            __syncthreads();
+            fir_chunk<S, PACKED, false, false>(w, v0, n, ldg, ldz, stash, taps, ph);
+        }
+        for (; v0 < n + 2 * S; v0 += R) {
+            __syncthreads();
+            fir_chunk<S, PACKED, false, true>(w, v0, n, ldg, ldz, stash, taps, ph);
+        }
+    }
+}
+
+// s = 0 off the streaming kernel's alignment, s > 7: one coordinate per thread, rows re-read through the caches,
 // fp64 taps and fp64 accumulation throughout (a tap rounded to fp32 is a fixed error of 2^-24 |tap| that
 // the decoder's cancellation amplifies like any other).  half > 0: packed mode (len complex coordinates; the imaginary
 // parts come from G[r][half + i], zero beyond d_real).
@@ -353,6 +501,33 @@ int launch_stream_any(const draco_plan* p, const float* G, float2* Z, int64_t le
     }
 }
 
+template <int S, bool PACKED>
+int launch_fir(const draco_plan* p, const float* G, float2* Z, int64_t len, int64_t ldg, int64_t ldz, int64_t half,
+               int64_t d_real, cudaStream_t st) {
+    using Cfg = FirCfg<S, PACKED>;
+    const int64_t nstrips = (len + Cfg::kTile - 1) / Cfg::kTile;
+    int64_t grid = (int64_t)p->sm_count * Cfg::kBlocks;
+    if (grid > nstrips) grid = nstrips;
+    cyc_encode_fir_kernel<S, PACKED><<<(int)grid, Cfg::kThreads, 0, st>>>(G, Z, len, ldg, ldz, half, d_real, p->n, p->taps64,
+                                                                          p->phase64);
+    DRACO_CUDA(cudaGetLastError());
+    return DRACO_OK;
+}
+
+template <bool PACKED>
+int launch_fir_any(const draco_plan* p, const float* G, float2* Z, int64_t len, int64_t ldg, int64_t ldz, int64_t half,
+                   int64_t d_real, cudaStream_t st) {
+    switch (p->s) {
+        case 1: return launch_fir<1, PACKED>(p, G, Z, len, ldg, ldz, half, d_real, st);
+        case 2: return launch_fir<2, PACKED>(p, G, Z, len, ldg, ldz, half, d_real, st);
+        case 3: return launch_fir<3, PACKED>(p, G, Z, len, ldg, ldz, half, d_real, st);
+        case 4: return launch_fir<4, PACKED>(p, G, Z, len, ldg, ldz, half, d_real, st);
+        case 5: return launch_fir<5, PACKED>(p, G, Z, len, ldg, ldz, half, d_real, st);
+        case 6: return launch_fir<6, PACKED>(p, G, Z, len, ldg, ldz, half, d_real, st);
+        default: return launch_fir<7, PACKED>(p, G, Z, len, ldg, ldz, half, d_real, st);
+    }
+}
+
 }  // namespace
 
 // half == 0: Z[j][i], i < len, from G[.][i].  half > 0 (packed): Z[j][i], i < len complex coordinates,
@@ -367,6 +542,9 @@ int launch_cyc_encode(const draco_plan* p, const float* G, float2* Z, int64_t le
     else fast = fast && (len % 4 == 0);
     if (fast) return packed ? launch_stream_any<true>(p, G, Z, len, ldg, ldz, half, st)
                             : launch_stream_any<false>(p, G, Z, len, ldg, ldz, 0, st);
+    if (p->s >= 1 && p->s <= 7)                            // the register window's sizes
+        return packed ? launch_fir_any<true>(p, G, Z, len, ldg, ldz, half, d_real, st)
+                      : launch_fir_any<false>(p, G, Z, len, ldg, ldz, 0, d_real, st);
     int64_t want = (len + kGenericThreads - 1) / kGenericThreads;
     const int64_t cap = (int64_t)p->sm_count * 16;
     if (want > cap) want = cap;
