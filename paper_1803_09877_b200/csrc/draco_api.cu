@@ -181,6 +181,8 @@ int draco_plan_create(int n, int s, int64_t d, int code, draco_plan** out) {
         DRACO_TRY(cudaMalloc(&p->partial_dev, partial_bytes));
         DRACO_TRY(cudaMemset(p->partial_dev, 0, partial_bytes));
     }
+    // the calls that use the plan may come on streams that do not wait for the default one
+    DRACO_TRY(cudaStreamSynchronize(nullptr));
 #undef DRACO_TRY
     *out = p;
     return DRACO_OK;
@@ -227,7 +229,7 @@ int draco_encode(const draco_plan* plan, const float* G, void* Z, void* stream) 
 
 int draco_rep_vote(draco_plan* plan, const void* R, float* u, float* maj, uint8_t* flags, void* stream) {
     if (!plan || plan->code != DRACO_REP || !R || !aligned16(R) || !aligned16(u) || !aligned16(maj)) return DRACO_EINVAL;
-    return launch_rep_vote(plan, (const float*)R, plan->d, plan->d, u, maj, flags, true, (cudaStream_t)stream);
+    return launch_rep_vote(plan, (const float*)R, plan->d, plan->d, u, maj, flags, (cudaStream_t)stream);
 }
 
 int draco_cyc_project(draco_plan* plan, const void* R, const float* f, double* e, void* stream) {
@@ -248,7 +250,7 @@ int draco_locate(draco_plan* plan, const void* R, const float* f, uint8_t* flags
     if (!plan || !R || !aligned16(R)) return DRACO_EINVAL;
     cudaStream_t st = (cudaStream_t)stream;
     if (plan->code == DRACO_REP)
-        return launch_rep_vote(plan, (const float*)R, plan->d, plan->d, nullptr, nullptr, flags, true, st);
+        return launch_rep_vote(plan, (const float*)R, plan->d, plan->d, nullptr, nullptr, flags, st);
     if (!f || !aligned16(f)) return DRACO_EINVAL;
     int rc = launch_cyc_project(plan, (const float2*)R, f, vec_len(plan), vec_len(plan), false, st);
     if (rc != DRACO_OK) return rc;
@@ -259,7 +261,7 @@ int draco_decode(draco_plan* plan, const void* R, const uint8_t* flags, float* u
     if (!plan || !R || !u || !aligned16(R) || !aligned16(u)) return DRACO_EINVAL;
     cudaStream_t st = (cudaStream_t)stream;
     if (plan->code == DRACO_REP)
-        return launch_rep_vote(plan, (const float*)R, plan->d, plan->d, u, nullptr, nullptr, true, st);
+        return launch_rep_vote(plan, (const float*)R, plan->d, plan->d, u, nullptr, nullptr, st);
     if (!flags) flags = plan->flags_dev;                 // the plan's own copy of its last locate's flags
     int rc = launch_cyc_decode_vector(plan, flags, st);
     if (rc != DRACO_OK) return rc;
@@ -270,7 +272,7 @@ int draco_decode_update(draco_plan* plan, const void* R, const uint8_t* flags, f
     if (!plan || !R || !w || !aligned16(R) || !aligned16(w)) return DRACO_EINVAL;
     cudaStream_t st = (cudaStream_t)stream;
     if (plan->code == DRACO_REP)
-        return launch_rep_vote(plan, (const float*)R, plan->d, plan->d, nullptr, nullptr, nullptr, true, st, w, scale);
+        return launch_rep_vote(plan, (const float*)R, plan->d, plan->d, nullptr, nullptr, nullptr, st, w, scale);
     if (!flags) flags = plan->flags_dev;
     int rc = launch_cyc_decode_vector(plan, flags, st);
     if (rc != DRACO_OK) return rc;
@@ -282,7 +284,7 @@ int draco_locate_decode(draco_plan* plan, const void* R, const float* f, uint8_t
     if (!plan || !R || !u || !flags || !aligned16(R) || !aligned16(u)) return DRACO_EINVAL;
     cudaStream_t st = (cudaStream_t)stream;
     if (plan->code == DRACO_REP)
-        return launch_rep_vote(plan, (const float*)R, plan->d, plan->d, u, nullptr, flags, true, st);
+        return launch_rep_vote(plan, (const float*)R, plan->d, plan->d, u, nullptr, flags, st);
     // projection, then syndromes / solve / support / decode vector in one launch, then the recovery
     if (!f || !aligned16(f)) return DRACO_EINVAL;
     int rc = launch_cyc_project(plan, (const float2*)R, f, vec_len(plan), vec_len(plan), false, st);
@@ -435,7 +437,7 @@ int draco_pipeline_host(draco_plan* plan, const float* G_host, const float* f_ho
         rc = launch_cyc_solve(plan, nullptr, nullptr, true, st);
         if (rc == DRACO_OK) rc = launch_cyc_recover(plan, (const float2*)Z, vlen, vlen, plan->u_dev, packed ? d : 0, st);
     } else {
-        rc = launch_rep_vote(plan, (const float*)Z, d, d, plan->u_dev, nullptr, nullptr, true, st);
+        rc = launch_rep_vote(plan, (const float*)Z, d, d, plan->u_dev, nullptr, nullptr, st);
     }
     if (rc != DRACO_OK) return rc;
     DRACO_CUDA(cudaMemcpyAsync(u_host, plan->u_dev, sizeof(float) * (size_t)d, cudaMemcpyDeviceToHost, st));

@@ -93,7 +93,7 @@ struct draco_plan {
     int project_grid;                 // capacity of partial_dev in blocks
     int project_used;                 // blocks whose partials the plan's last projection (all its chunks) filled
     uint8_t* flags_dev;               // [n] internal flags
-    uint32_t* mask_dev;               // repetition: disagreement bits, [n] words
+    uint32_t* mask_dev;               // repetition: the vote's scratch, zero between calls
     // host-buffer pipeline (allocated on its first call)
     float* stage_dev;                 // two [n][stage_chunk] slices of G (double buffer)
     cudaStream_t copy_stream, work_stream;
@@ -118,7 +118,7 @@ int cuda_fail(cudaError_t err, const char* what);
 int launch_rep_encode(const draco_plan* p, const float* G, float* Z, int64_t len, int64_t ldg, int64_t ldz,
                       cudaStream_t st);
 int launch_rep_vote(draco_plan* p, const float* R, int64_t len, int64_t ld, float* u, float* maj, uint8_t* flags,
-                    bool reset, cudaStream_t st, float* w = nullptr, float scale = 0.0f);
+                    cudaStream_t st, float* w = nullptr, float scale = 0.0f);
 int launch_cyc_encode(const draco_plan* p, const float* G, float2* Z, int64_t len, int64_t ldg, int64_t ldz,
                       int64_t half, int64_t d_real, cudaStream_t st);
 int launch_cyc_project(draco_plan* p, const float2* R, const float* f, int64_t len, int64_t ld, bool accumulate,

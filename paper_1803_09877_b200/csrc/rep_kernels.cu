@@ -4,8 +4,7 @@
 // streaming majority vote of Algorithm 2 on 32-bit patterns.
 //
 // Both kernels are single passes over an [n][len] fp32 matrix: a thread owns
-// VEC consecutive coordinates, walks the groups, and keeps one group's replicas
-// in registers (128-bit loads, one per replica).  HBM-bound: encode moves
+// four coordinates, walks the groups, and keeps one group's replicas in registers.  HBM-bound: encode moves
 // 8 n len bytes, vote 4 n len + 4 len bytes.
 #include "draco_internal.cuh"
 
@@ -15,105 +14,152 @@ namespace {
 
 constexpr int kThreads = 256;
 
-template <int VEC>
-struct Pack;
-template <>
-struct Pack<4> {
+// Four columns of one row, as bit patterns.
+struct Pack {
     uint4 v;
     __device__ __forceinline__ uint32_t get(int c) const { return c == 0 ? v.x : c == 1 ? v.y : c == 2 ? v.z : v.w; }
 };
-template <>
-struct Pack<2> {
-    uint2 v;
-    __device__ __forceinline__ uint32_t get(int c) const { return c == 0 ? v.x : v.y; }
+
+// The four columns of a thread.  ADJ: neighbours, one 128-bit access (every row starts on a 16-byte boundary and holds whole
+// vectors).  Otherwise blockDim.x apart, four 32-bit accesses, so that a warp's accesses are contiguous wherever a row starts;
+// `in` has bit c set for the columns inside the vector, the others read the first column again.  As many bytes in flight per
+// thread as with one 128-bit access; with one column per thread the vote ran at 2.6 - 3.9 TB/s on such rows (n = 45, s = 5,
+// d = 5,000,011: 348 us, now 150; n = 45, s = 3: 236, now 154; s = 1: 277, now 166; encode, s = 5: 427, now 344).
+template <bool ADJ>
+struct Columns {
+    int64_t col;
+    uint32_t in;
+    int o1, o2, o3;
+    __device__ __forceinline__ void open(int64_t c, int64_t len) {
+        col = c;
+        if constexpr (ADJ) {
+            in = 15u;
+        } else {
+            const int step = (int)blockDim.x;
+            in = 1u | (c + step < len ? 2u : 0u) | (c + 2 * step < len ? 4u : 0u) | (c + 3 * step < len ? 8u : 0u);
+            o1 = (in & 2u) ? step : 0;
+            o2 = (in & 4u) ? 2 * step : 0;
+            o3 = (in & 8u) ? 3 * step : 0;
+        }
+    }
+    __device__ __forceinline__ bool has(int c) const { return ADJ || ((in >> c) & 1u); }
+    __device__ __forceinline__ void load(Pack& p, const uint32_t* row) const {
+        const uint32_t* ptr = row + col;
+        if constexpr (ADJ) p.v = __ldcs(reinterpret_cast<const uint4*>(ptr));
+        else p.v = make_uint4(__ldcs(ptr), __ldcs(ptr + o1), __ldcs(ptr + o2), __ldcs(ptr + o3));
+    }
+    __device__ __forceinline__ void store(float* row, const float (&x)[4]) const {
+        float* ptr = row + col;
+        if constexpr (ADJ) {
+            __stcs(reinterpret_cast<float4*>(ptr), make_float4(x[0], x[1], x[2], x[3]));
+        } else {
+            const int off[4] = {0, o1, o2, o3};
+#pragma unroll
+            for (int c = 0; c < 4; ++c)
+                if (has(c)) __stcs(ptr + off[c], x[c]);
+        }
+    }
+    // w <- w - scale * x (the SGD step of Section 2 fused into the decoder's epilogue)
+    __device__ __forceinline__ void update(float* row, const float (&x)[4], float scale) const {
+        float* ptr = row + col;
+        if constexpr (ADJ) {
+            float4 w = *reinterpret_cast<const float4*>(ptr);
+            w.x = fmaf(-scale, x[0], w.x); w.y = fmaf(-scale, x[1], w.y); w.z = fmaf(-scale, x[2], w.z); w.w = fmaf(-scale, x[3], w.w);
+            *reinterpret_cast<float4*>(ptr) = w;
+        } else {
+            const int off[4] = {0, o1, o2, o3};
+#pragma unroll
+            for (int c = 0; c < 4; ++c)
+                if (has(c)) ptr[off[c]] = fmaf(-scale, x[c], ptr[off[c]]);
+        }
+    }
 };
-template <>
-struct Pack<1> {
-    uint32_t v;
-    __device__ __forceinline__ uint32_t get(int) const { return v; }
-};
-
-__device__ __forceinline__ void load_pack(Pack<4>& p, const uint32_t* ptr) {
-    p.v = __ldcs(reinterpret_cast<const uint4*>(ptr));
-}
-__device__ __forceinline__ void load_pack(Pack<2>& p, const uint32_t* ptr) {
-    p.v = __ldcs(reinterpret_cast<const uint2*>(ptr));
-}
-__device__ __forceinline__ void load_pack(Pack<1>& p, const uint32_t* ptr) { p.v = __ldcs(ptr); }
-
-__device__ __forceinline__ void store_vals(float* ptr, const float (&x)[4]) {
-    __stcs(reinterpret_cast<float4*>(ptr), make_float4(x[0], x[1], x[2], x[3]));
-}
-__device__ __forceinline__ void store_vals(float* ptr, const float (&x)[2]) {
-    __stcs(reinterpret_cast<float2*>(ptr), make_float2(x[0], x[1]));
-}
-__device__ __forceinline__ void store_vals(float* ptr, const float (&x)[1]) { __stcs(ptr, x[0]); }
-
-// w <- w - scale * x on VEC consecutive entries (the SGD step of Section 2 fused into the decoder's epilogue)
-__device__ __forceinline__ void update_vals(float* ptr, const float (&x)[4], float scale) {
-    float4 w = *reinterpret_cast<const float4*>(ptr);
-    w.x = fmaf(-scale, x[0], w.x); w.y = fmaf(-scale, x[1], w.y); w.z = fmaf(-scale, x[2], w.z); w.w = fmaf(-scale, x[3], w.w);
-    *reinterpret_cast<float4*>(ptr) = w;
-}
-__device__ __forceinline__ void update_vals(float* ptr, const float (&x)[2], float scale) {
-    float2 w = *reinterpret_cast<const float2*>(ptr);
-    w.x = fmaf(-scale, x[0], w.x); w.y = fmaf(-scale, x[1], w.y);
-    *reinterpret_cast<float2*>(ptr) = w;
-}
-__device__ __forceinline__ void update_vals(float* ptr, const float (&x)[1], float scale) { ptr[0] = fmaf(-scale, x[0], ptr[0]); }
 
 // ---------------------------------------------------------------- encode
 // MMAX > 0: groups of at most MMAX members, GB groups fetched together so that about 16 rows are in flight per
 // thread whatever the group size (as in the vote kernel); MMAX == 0: larger groups, members streamed.
-template <int MMAX, int VEC, int GB>
+// Rows off the 16-byte grid (ADJ false): a block reads kSector columns more than it writes and writes of each row the run that
+// starts on a 32-byte sector, so that no sector is shared between blocks (a shared one may go to memory half filled).
+constexpr int kSector = 8;                              // fp32 values
+template <int MMAX, bool ADJ, int GB>
 __global__ void __launch_bounds__(kThreads)
 rep_encode_kernel(const float* __restrict__ G, float* __restrict__ Z, int64_t len, int64_t ldg, int64_t ldz,
                   GroupTable gt) {
-    const int64_t nvec = len / VEC;
-    const int64_t stride = (int64_t)gridDim.x * kThreads;
-    for (int64_t v = (int64_t)blockIdx.x * kThreads + threadIdx.x; v < nvec; v += stride) {
-        const int64_t col = v * VEC;
+    const uint32_t* Gb = reinterpret_cast<const uint32_t*>(G);
+    const int span = 4 * (int)blockDim.x, tile = ADJ ? span : span - kSector;
+    const int64_t ntiles = (len + tile - 1) / tile;
+    for (int64_t t = blockIdx.x; t < ntiles; t += gridDim.x) {
+        const int64_t c0 = t * tile;
+        const int64_t first_col = c0 + (ADJ ? 4 : 1) * (int)threadIdx.x;
+        if (first_col >= len) continue;
+        Columns<ADJ> cols;
+        cols.open(first_col, len);
+        uint32_t mask = 0;                              // byte c, bit k: column c is written in rows whose run starts k columns in
+        int shift0 = 0;
+        if constexpr (!ADJ) {
+            shift0 = (int)(-((int64_t)(reinterpret_cast<uintptr_t>(Z) >> 2) + c0)) & (kSector - 1);
+#pragma unroll
+            for (int c = 0; c < 4; ++c) {
+                const int i = (int)threadIdx.x + c * (int)blockDim.x;
+#pragma unroll
+                for (int k = 0; k < kSector; ++k)
+                    if (cols.has(c) && (i >= k || t == 0) && i < k + tile) mask |= 1u << (c * kSector + k);
+            }
+        }
+        auto emit = [&](int row, const float(&acc)[4]) {
+            float* z = Z + (int64_t)row * ldz;
+            if constexpr (ADJ) {
+                cols.store(z, acc);
+            } else {
+                const uint32_t m = mask >> ((shift0 - (int)((row * ldz) & (kSector - 1))) & (kSector - 1));
+                z += cols.col;
+                if (m & 1u) __stcs(z, acc[0]);
+                if (m & 0x100u) __stcs(z + cols.o1, acc[1]);
+                if (m & 0x10000u) __stcs(z + cols.o2, acc[2]);
+                if (m & 0x1000000u) __stcs(z + cols.o3, acc[3]);
+            }
+        };
         if constexpr (MMAX > 0) {
             for (int g0 = 0; g0 < gt.num_groups; g0 += GB) {
-                Pack<VEC> val[GB][MMAX];
+                Pack val[GB][MMAX];
 #pragma unroll
                 for (int b = 0; b < GB; ++b)
                     if (g0 + b < gt.num_groups) {
                         const int first = gt.first[g0 + b], m = gt.size[g0 + b];
 #pragma unroll
                         for (int k = 0; k < MMAX; ++k)
-                            if (k < m) load_pack(val[b][k], reinterpret_cast<const uint32_t*>(G + (int64_t)(first + k) * ldg + col));
+                            if (k < m) cols.load(val[b][k], Gb + (int64_t)(first + k) * ldg);
                     }
 #pragma unroll
                 for (int b = 0; b < GB; ++b)
                     if (g0 + b < gt.num_groups) {
                         const int first = gt.first[g0 + b], m = gt.size[g0 + b];
-                        float acc[VEC];
+                        float acc[4];
 #pragma unroll
-                        for (int c = 0; c < VEC; ++c) acc[c] = __uint_as_float(val[b][0].get(c));
+                        for (int c = 0; c < 4; ++c) acc[c] = __uint_as_float(val[b][0].get(c));
 #pragma unroll
                         for (int k = 1; k < MMAX; ++k)
                             if (k < m) {
 #pragma unroll
-                                for (int c = 0; c < VEC; ++c) acc[c] = __fadd_rn(acc[c], __uint_as_float(val[b][k].get(c)));
+                                for (int c = 0; c < 4; ++c) acc[c] = __fadd_rn(acc[c], __uint_as_float(val[b][k].get(c)));
                             }
-                        for (int k = 0; k < m; ++k) store_vals(Z + (int64_t)(first + k) * ldz + col, acc);
+                        for (int k = 0; k < m; ++k) emit(first + k, acc);
                     }
             }
         } else {
             for (int g = 0; g < gt.num_groups; ++g) {
                 const int first = gt.first[g], m = gt.size[g];
-                float acc[VEC];
-                Pack<VEC> x;
-                load_pack(x, reinterpret_cast<const uint32_t*>(G + (int64_t)first * ldg + col));
+                float acc[4];
+                Pack x;
+                cols.load(x, Gb + (int64_t)first * ldg);
 #pragma unroll
-                for (int c = 0; c < VEC; ++c) acc[c] = __uint_as_float(x.get(c));
+                for (int c = 0; c < 4; ++c) acc[c] = __uint_as_float(x.get(c));
                 for (int k = 1; k < m; ++k) {
-                    load_pack(x, reinterpret_cast<const uint32_t*>(G + (int64_t)(first + k) * ldg + col));
+                    cols.load(x, Gb + (int64_t)(first + k) * ldg);
 #pragma unroll
-                    for (int c = 0; c < VEC; ++c) acc[c] = __fadd_rn(acc[c], __uint_as_float(x.get(c)));
+                    for (int c = 0; c < 4; ++c) acc[c] = __fadd_rn(acc[c], __uint_as_float(x.get(c)));
                 }
-                for (int k = 0; k < m; ++k) store_vals(Z + (int64_t)(first + k) * ldz + col, acc);
+                for (int k = 0; k < m; ++k) emit(first + k, acc);
             }
         }
     }
@@ -123,7 +169,42 @@ rep_encode_kernel(const float* __restrict__ G, float* __restrict__ Z, int64_t le
 struct RepScratch {
     uint32_t mask[kMaxN];             // per group: bit k set <=> member k disagreed somewhere
     unsigned long long no_majority;
+    unsigned int done;                // blocks that have added their part
 };
+
+// mask words -> flag bytes and the info block, by the block that comes last, which leaves the scratch cleared for the next
+// call on the plan: a memset before and a one-block kernel after the vote were two thirds of a short vote's time
+// (n = 15, s = 2, d = 100,000: 11.3 - 12.8 us with them, 7.6 - 8.2 without).
+__device__ __forceinline__ void finish_vote(const GroupTable& gt, RepScratch* scratch, uint8_t* flags, uint8_t* flags2,
+                                            DeviceInfo* info) {
+    __shared__ int count;
+    if (threadIdx.x == 0) count = 0;
+    __syncthreads();
+    for (int g = threadIdx.x; g < gt.num_groups; g += blockDim.x) {
+        const int first = gt.first[g], m = gt.size[g];
+        int c = 0;
+        uint32_t word = 0;
+        for (int k = 0; k < m; ++k) {
+            if (k % 32 == 0) word = atomicExch(&scratch->mask[first + k / 32], 0u);
+            const uint8_t bit = (word >> (k & 31)) & 1u;
+            if (flags) flags[first + k] = bit;
+            flags2[first + k] = bit;
+            c += bit;
+        }
+        if (c) atomicAdd(&count, c);
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        const unsigned long long no_majority = atomicExch(&scratch->no_majority, 0ull);
+        info->n_flagged = count;
+        info->no_majority = no_majority;
+        info->status = no_majority ? DRACO_ENOMAJ : DRACO_OK;
+        info->locator_rank = 0;
+        info->n_active = 0;
+        info->scale = 0.0;
+        info->max_syndrome = 0.0;
+    }
+}
 
 // One step of Algorithm 2 for item x.
 __device__ __forceinline__ void vote_step(uint32_t x, uint32_t& ma, int& counter) {
@@ -134,54 +215,39 @@ __device__ __forceinline__ void vote_step(uint32_t x, uint32_t& ma, int& counter
 }
 
 // Majority of one group whose m <= MMAX replicas sit in registers.  Returns the selected bit
-// patterns in sel[], adds the members that disagree somewhere to `dis` and the coordinates
+// patterns in sel[], adds the members that disagree somewhere to `dis` and the coordinates (of those in `in`)
 // without a strict majority to `nomaj`.
-template <int MMAX, int VEC>
-__device__ __forceinline__ void vote_group(const Pack<VEC> (&val)[MMAX], int m, uint32_t (&sel)[VEC], uint32_t& dis,
+template <int MMAX>
+__device__ __forceinline__ void vote_group(const Pack (&val)[MMAX], int m, uint32_t in, uint32_t (&sel)[4], uint32_t& dis,
                                            unsigned int& nomaj) {
-    uint32_t differ = 0;
-#pragma unroll
-    for (int k = 1; k < MMAX; ++k)
-        if (k < m) {
-#pragma unroll
-            for (int c = 0; c < VEC; ++c) differ |= val[k].get(c) ^ val[0].get(c);
-        }
-    if (differ == 0) {                                   // all replicas bit-identical: they are the majority
-#pragma unroll
-        for (int c = 0; c < VEC; ++c) sel[c] = val[0].get(c);
-        return;
-    }
-    // Some replica differs.  A value held by strictly more than half of the group IS what
-    // Algorithm 2 returns, so first count the votes for member 0's value, then for member 1's
-    // (member 0 may be the adversary); only if neither has a strict majority on all VEC
-    // coordinates is the streaming vote itself run.
+    // A value held by strictly more than half of the group IS what Algorithm 2 returns.  So count first the members that equal
+    // member 0 in all four columns (five logic operations each), then those that equal member 1 (member 0 may be the
+    // adversary); only if neither has a strict majority is the streaming vote itself run, column by column.  Counting column by
+    // column at once took about twice the instructions and left large groups bound by them (n = 45, d = 5 M: s = 7 244 us, now
+    // 188; s = 5 162 us, now 141).
     bool settled = false;
 #pragma unroll
     for (int ref = 0; ref < 2 && ref < MMAX; ++ref) {
         if (!settled && ref < m) {
-            uint32_t d_ref = 0;
-            bool all_major = true;
+            const uint4 r = val[ref].v;
+            uint32_t ne = 0;
 #pragma unroll
-            for (int c = 0; c < VEC; ++c) {
-                const uint32_t cand = val[ref].get(c);
-                uint32_t ne = 0;
+            for (int k = 0; k < MMAX; ++k)
+                if (k != ref && k < m) {
+                    const uint4 x = val[k].v;
+                    ne |= (((x.x ^ r.x) | (x.y ^ r.y) | (x.z ^ r.z) | (x.w ^ r.w)) != 0u ? 1u : 0u) << k;
+                }
+            if (2 * (m - __popc(ne)) > m) {
 #pragma unroll
-                for (int k = 0; k < MMAX; ++k)
-                    if (k < m) ne |= (val[k].get(c) != cand ? 1u : 0u) << k;
-                all_major &= (2 * (m - __popc(ne)) > m);
-                d_ref |= ne;
-            }
-            if (all_major) {
-#pragma unroll
-                for (int c = 0; c < VEC; ++c) sel[c] = val[ref].get(c);
-                dis |= d_ref;
+                for (int c = 0; c < 4; ++c) sel[c] = val[ref].get(c);
+                dis |= ne;
                 settled = true;
             }
         }
     }
     if (!settled) {
 #pragma unroll
-        for (int c = 0; c < VEC; ++c) {
+        for (int c = 0; c < 4; ++c) {
             uint32_t ma = val[0].get(c);
             int counter = 0;
 #pragma unroll
@@ -191,7 +257,7 @@ __device__ __forceinline__ void vote_group(const Pack<VEC> (&val)[MMAX], int m, 
 #pragma unroll
             for (int k = 0; k < MMAX; ++k)
                 if (k < m) ne |= (val[k].get(c) != ma ? 1u : 0u) << k;
-            nomaj += (2 * (m - __popc(ne)) <= m);
+            nomaj += (2 * (m - __popc(ne)) <= m) && ((in >> c) & 1u);
             dis |= ne;
             sel[c] = ma;
         }
@@ -201,92 +267,95 @@ __device__ __forceinline__ void vote_group(const Pack<VEC> (&val)[MMAX], int m, 
 // MMAX > 0: groups of at most MMAX members, GB groups fetched together so that about 16 rows
 // (128-bit or 64-bit loads) are in flight per thread whatever the group size.
 // MMAX == 0: groups larger than the register budget, members streamed twice (GB ignored).
-template <int MMAX, int VEC, int GB, int TPB>
+template <int MMAX, bool ADJ, int GB, int TPB>
 __global__ void __launch_bounds__(TPB)
 rep_vote_kernel(const uint32_t* __restrict__ R, int64_t len, int64_t ld, GroupTable gt, float* __restrict__ u,
-                float* __restrict__ maj, RepScratch* scratch, float* __restrict__ w, float scale) {
+                float* __restrict__ maj, RepScratch* scratch, float* __restrict__ w, float scale, uint8_t* flags, uint8_t* flags2,
+                DeviceInfo* info) {
     __shared__ uint32_t smask[kMaxN][MMAX > 0 ? 1 : 4];   // generic path: up to 128 members = 4 words
-    for (int i = threadIdx.x; i < kMaxN * (MMAX > 0 ? 1 : 4); i += TPB) (&smask[0][0])[i] = 0;
+    for (int i = threadIdx.x; i < kMaxN * (MMAX > 0 ? 1 : 4); i += blockDim.x) (&smask[0][0])[i] = 0;
     __syncthreads();
 
     unsigned int nomaj = 0;
-    const int64_t nvec = len / VEC;
-    const int64_t stride = (int64_t)gridDim.x * TPB;
-    for (int64_t v = (int64_t)blockIdx.x * TPB + threadIdx.x; v < nvec; v += stride) {
-        const int64_t col = v * VEC;
-        float acc[VEC];
+    const int64_t tile = 4 * (int64_t)blockDim.x;
+    for (int64_t c0 = blockIdx.x * tile; c0 < len; c0 += gridDim.x * tile) {
+        const int64_t first_col = c0 + (ADJ ? 4 : 1) * (int)threadIdx.x;
+        if (first_col >= len) continue;
+        Columns<ADJ> cols;
+        cols.open(first_col, len);
+        float acc[4];
 #pragma unroll
-        for (int c = 0; c < VEC; ++c) acc[c] = 0.0f;
+        for (int c = 0; c < 4; ++c) acc[c] = 0.0f;
         if constexpr (MMAX > 0) {
             for (int g0 = 0; g0 < gt.num_groups; g0 += GB) {
-                Pack<VEC> val[GB][MMAX];
+                Pack val[GB][MMAX];
 #pragma unroll
                 for (int b = 0; b < GB; ++b)
                     if (g0 + b < gt.num_groups) {
                         const int first = gt.first[g0 + b], m = gt.size[g0 + b];
-                        const uint32_t* base = R + (int64_t)first * ld + col;
+                        const uint32_t* base = R + (int64_t)first * ld;
 #pragma unroll
                         for (int k = 0; k < MMAX; ++k)
-                            if (k < m) load_pack(val[b][k], base + (int64_t)k * ld);
+                            if (k < m) cols.load(val[b][k], base + (int64_t)k * ld);
                     }
 #pragma unroll
                 for (int b = 0; b < GB; ++b)
                     if (g0 + b < gt.num_groups) {
                         const int g = g0 + b, m = gt.size[g];
-                        uint32_t sel[VEC];
+                        uint32_t sel[4];
                         uint32_t dis = 0;
-                        vote_group<MMAX, VEC>(val[b], m, sel, dis, nomaj);
+                        vote_group<MMAX>(val[b], m, cols.in, sel, dis, nomaj);
                         if (dis & ~smask[g][0]) atomicOr(&smask[g][0], dis);
-                        float selv[VEC];
+                        float selv[4];
 #pragma unroll
-                        for (int c = 0; c < VEC; ++c) {
+                        for (int c = 0; c < 4; ++c) {
                             selv[c] = __uint_as_float(sel[c]);
                             acc[c] = __fadd_rn(acc[c], selv[c]);
                         }
-                        if (maj != nullptr) store_vals(maj + (int64_t)g * len + col, selv);
+                        if (maj != nullptr) cols.store(maj + (int64_t)g * len, selv);
                     }
             }
         } else {
             for (int g = 0; g < gt.num_groups; ++g) {
                 const int first = gt.first[g], m = gt.size[g];
-                const uint32_t* base = R + (int64_t)first * ld + col;
-                uint32_t ma[VEC];
-                int counter[VEC];
-                Pack<VEC> x;
-                load_pack(x, base);
+                const uint32_t* base = R + (int64_t)first * ld;
+                uint32_t ma[4];
+                int counter[4];
+                Pack x;
+                cols.load(x, base);
 #pragma unroll
-                for (int c = 0; c < VEC; ++c) { ma[c] = x.get(c); counter[c] = 0; }
+                for (int c = 0; c < 4; ++c) { ma[c] = x.get(c); counter[c] = 0; }
                 for (int k = 0; k < m; ++k) {
-                    load_pack(x, base + (int64_t)k * ld);
+                    cols.load(x, base + (int64_t)k * ld);
 #pragma unroll
-                    for (int c = 0; c < VEC; ++c) vote_step(x.get(c), ma[c], counter[c]);
+                    for (int c = 0; c < 4; ++c) vote_step(x.get(c), ma[c], counter[c]);
                 }
-                int votes[VEC];
+                int votes[4];
 #pragma unroll
-                for (int c = 0; c < VEC; ++c) votes[c] = 0;
+                for (int c = 0; c < 4; ++c) votes[c] = 0;
                 for (int k = 0; k < m; ++k) {
-                    load_pack(x, base + (int64_t)k * ld);
+                    cols.load(x, base + (int64_t)k * ld);
                     bool any_diff = false;
 #pragma unroll
-                    for (int c = 0; c < VEC; ++c) {
+                    for (int c = 0; c < 4; ++c) {
                         const bool same = x.get(c) == ma[c];
                         votes[c] += same;
                         any_diff |= !same;
                     }
                     if (any_diff && !(smask[g][k >> 5] & (1u << (k & 31)))) atomicOr(&smask[g][k >> 5], 1u << (k & 31));
                 }
-                float selv[VEC];
+                float selv[4];
 #pragma unroll
-                for (int c = 0; c < VEC; ++c) {
-                    nomaj += (2 * votes[c] <= m);
+                for (int c = 0; c < 4; ++c) {
+                    nomaj += (2 * votes[c] <= m) && cols.has(c);
                     selv[c] = __uint_as_float(ma[c]);
                     acc[c] = __fadd_rn(acc[c], selv[c]);
                 }
-                if (maj != nullptr) store_vals(maj + (int64_t)g * len + col, selv);
+                if (maj != nullptr) cols.store(maj + (int64_t)g * len, selv);
             }
         }
-        if (u != nullptr) store_vals(u + col, acc);
-        if (w != nullptr) update_vals(w + col, acc, scale);
+        if (u != nullptr) cols.store(u, acc);
+        if (w != nullptr) cols.update(w, acc, scale);
     }
 
     // block totals -> global scratch (integer OR / add: order-independent, hence deterministic)
@@ -295,51 +364,42 @@ rep_vote_kernel(const uint32_t* __restrict__ R, int64_t len, int64_t ld, GroupTa
     if ((threadIdx.x & 31) == 0 && nomaj) atomicAdd(&scratch->no_majority, (unsigned long long)nomaj);
     __syncthreads();
     if constexpr (MMAX > 0) {
-        for (int g = threadIdx.x; g < gt.num_groups; g += TPB)
+        for (int g = threadIdx.x; g < gt.num_groups; g += blockDim.x)
             if (smask[g][0]) atomicOr(&scratch->mask[gt.first[g]], smask[g][0]);
     } else {
         // generic path keeps one word per 32 members; spread them over the members' own slots
-        for (int g = threadIdx.x; g < gt.num_groups; g += TPB)
+        for (int g = threadIdx.x; g < gt.num_groups; g += blockDim.x)
             for (int w = 0; w < 4; ++w)
                 if (smask[g][w]) atomicOr(&scratch->mask[gt.first[g] + w], smask[g][w]);
     }
-}
-
-// mask words -> flag bytes and the info block (one block).
-__global__ void rep_finish_kernel(GroupTable gt, const RepScratch* scratch, uint8_t* flags, uint8_t* flags2,
-                                  DeviceInfo* info, bool generic) {
-    __shared__ int count;
-    if (threadIdx.x == 0) count = 0;
+    __shared__ bool last;
+    __threadfence();
     __syncthreads();
-    for (int g = threadIdx.x; g < gt.num_groups; g += blockDim.x) {
-        const int first = gt.first[g], m = gt.size[g];
-        int c = 0;
-        for (int k = 0; k < m; ++k) {
-            const uint32_t word = generic ? scratch->mask[first + (k >> 5)] : scratch->mask[first];
-            const uint8_t bit = (word >> (k & 31)) & 1u;
-            if (flags) flags[first + k] = bit;
-            if (flags2) flags2[first + k] = bit;
-            c += bit;
-        }
-        atomicAdd(&count, c);
-    }
+    if (threadIdx.x == 0) last = atomicInc(&scratch->done, gridDim.x - 1) == gridDim.x - 1;     // wraps to 0
     __syncthreads();
-    if (threadIdx.x == 0) {
-        info->n_flagged = count;
-        info->no_majority = scratch->no_majority;
-        info->status = scratch->no_majority ? DRACO_ENOMAJ : DRACO_OK;
-        info->locator_rank = 0;
-        info->n_active = 0;
-        info->scale = 0.0;
-        info->max_syndrome = 0.0;
+    if (last) {
+        __threadfence();
+        finish_vote(gt, scratch, flags, flags2, info);
     }
 }
 
-int grid_for(int64_t nvec, int sm_count, int blocks_per_sm) {
-    int64_t want = (nvec + kThreads - 1) / kThreads;
-    int64_t cap = (int64_t)sm_count * blocks_per_sm;
-    if (want < 1) want = 1;
+// Threads per block: the kernel's limit, fewer for vectors too short to give every SM two such blocks.
+int block_for(int64_t quads, int sm_count, int limit) {
+    int threads = limit;
+    while (threads > 64 && quads < 2 * (int64_t)sm_count * threads) threads /= 2;
+    return threads;
+}
+
+int grid_for(int64_t quads, int threads, int64_t cap) {
+    const int64_t want = (quads + threads - 1) / threads;
     return (int)(want < cap ? want : cap);
+}
+
+template <typename Kernel>
+int resident_blocks(Kernel kernel, int threads) {
+    int per_sm = 0;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, threads, 0) != cudaSuccess || per_sm < 1) per_sm = 1;
+    return per_sm;
 }
 
 }  // namespace
@@ -347,54 +407,59 @@ int grid_for(int64_t nvec, int sm_count, int blocks_per_sm) {
 int launch_rep_encode(const draco_plan* p, const float* G, float* Z, int64_t len, int64_t ldg, int64_t ldz,
                       cudaStream_t st) {
     const GroupTable& gt = p->groups;
-    const bool vec4 = (len % 4 == 0) && (ldg % 4 == 0) && (ldz % 4 == 0);
-    const int64_t nvec = vec4 ? len / 4 : len;
-    const int grid = grid_for(nvec, p->sm_count, 8);
-#define DRACO_ENC(MM, VV, GG) rep_encode_kernel<MM, VV, GG><<<grid, kThreads, 0, st>>>(G, Z, len, ldg, ldz, gt)
-    if (vec4) {
-        if (gt.max_size <= 3) DRACO_ENC(3, 4, 5);
-        else if (gt.max_size <= 4) DRACO_ENC(4, 4, 4);
-        else if (gt.max_size <= 5) DRACO_ENC(5, 4, 2);
-        else if (gt.max_size <= 8) DRACO_ENC(8, 4, 1);
-        else if (gt.max_size <= 16) DRACO_ENC(16, 4, 1);
-        else DRACO_ENC(0, 4, 1);
-    } else {
-        if (gt.max_size <= 8) DRACO_ENC(8, 1, 2);
-        else if (gt.max_size <= 16) DRACO_ENC(16, 1, 1);
-        else DRACO_ENC(0, 1, 1);
-    }
+    const bool adj = (len % 4 == 0) && (ldg % 4 == 0) && (ldz % 4 == 0);
+    const int64_t quads = (len + 3) / 4;
+    const int threads = block_for(quads, p->sm_count, kThreads);
+    const int grid = grid_for(quads, threads, (int64_t)p->sm_count * 8 * (kThreads / threads));
+#define DRACO_ENC(MM, AA, GG) rep_encode_kernel<MM, AA, GG><<<grid, threads, 0, st>>>(G, Z, len, ldg, ldz, gt)
+#define DRACO_ENC_BY_SIZE(AA)                                      \
+    do {                                                           \
+        if (gt.max_size <= 3) DRACO_ENC(3, AA, 5);                 \
+        else if (gt.max_size <= 4) DRACO_ENC(4, AA, 4);            \
+        else if (gt.max_size <= 5) DRACO_ENC(5, AA, 2);            \
+        else if (gt.max_size <= 8) DRACO_ENC(8, AA, 1);            \
+        else if (gt.max_size <= 16) DRACO_ENC(16, AA, 1);          \
+        else DRACO_ENC(0, AA, 1);                                  \
+    } while (0)
+    if (adj) DRACO_ENC_BY_SIZE(true);
+    else DRACO_ENC_BY_SIZE(false);
+#undef DRACO_ENC_BY_SIZE
 #undef DRACO_ENC
     DRACO_CUDA(cudaGetLastError());
     return DRACO_OK;
 }
 
 int launch_rep_vote(draco_plan* p, const float* R, int64_t len, int64_t ld, float* u, float* maj, uint8_t* flags,
-                    bool reset, cudaStream_t st, float* w, float scale) {
+                    cudaStream_t st, float* w, float scale) {
     const GroupTable& gt = p->groups;
     RepScratch* scratch = reinterpret_cast<RepScratch*>(p->mask_dev);
-    if (reset) DRACO_CUDA(cudaMemsetAsync(scratch, 0, sizeof(RepScratch), st));
-    const bool vec4 = (len % 4 == 0) && (ld % 4 == 0);
+    const bool adj = (len % 4 == 0) && (ld % 4 == 0);
+    const int64_t quads = (len + 3) / 4;
     const uint32_t* Rb = reinterpret_cast<const uint32_t*>(R);
-    const bool generic = gt.max_size > 16;
-#define DRACO_VOTE(MM, VV, GG, TT)                                                                                 \
-    rep_vote_kernel<MM, VV, GG, TT><<<grid_for(len / VV, p->sm_count, 8) * (kThreads / TT), TT, 0, st>>>(Rb, len, ld, gt, u, \
-                                                                                                        maj, scratch, w, scale)
-    if (vec4) {
-        if (gt.max_size <= 3) DRACO_VOTE(3, 4, 5, 256);             // s = 1: five groups of three = 15 rows in flight
-        else if (gt.max_size <= 4) DRACO_VOTE(4, 4, 4, 256);
-        else if (gt.max_size <= 5) DRACO_VOTE(5, 4, 3, 256);        // s = 2: three groups of five
-        else if (gt.max_size <= 8) DRACO_VOTE(8, 4, 2, 256);
-        else if (gt.max_size <= 16) DRACO_VOTE(16, 4, 1, 128);      // 16 x 128-bit loads per thread: small blocks keep 3 per SM
-        else DRACO_VOTE(0, 4, 1, 256);
-    } else {
-        if (gt.max_size <= 4) DRACO_VOTE(4, 1, 4, 256);
-        else if (gt.max_size <= 8) DRACO_VOTE(8, 1, 2, 256);
-        else if (gt.max_size <= 16) DRACO_VOTE(16, 1, 1, 256);
-        else DRACO_VOTE(0, 1, 1, 256);
-    }
+    // no more blocks than are resident at once: a block's end (its part of the masks, the fence, the count) costs a microsecond
+    // or two, which four rounds of blocks one after the other pay four times (n = 45, s = 3, d = 11.7 M: 365 us so, 345 us now)
+#define DRACO_VOTE(MM, AA, GG, TT)                                                                                \
+    do {                                                                                                          \
+        static const int per_sm = resident_blocks(rep_vote_kernel<MM, AA, GG, TT>, TT);                           \
+        const int threads = block_for(quads, p->sm_count, TT);                                                    \
+        const int grid = grid_for(quads, threads, p->sm_count * per_sm * (TT / threads));                         \
+        rep_vote_kernel<MM, AA, GG, TT><<<grid, threads, 0, st>>>(Rb, len, ld, gt, u, maj, scratch, w, scale, flags,  \
+                                                                  p->flags_dev, p->info_dev);                      \
+    } while (0)
+#define DRACO_VOTE_BY_SIZE(AA)                                                                                    \
+    do {                                                                                                          \
+        if (gt.max_size <= 3) DRACO_VOTE(3, AA, 5, 256);             /* s = 1: five groups of three, 15 rows in flight */ \
+        else if (gt.max_size <= 4) DRACO_VOTE(4, AA, 4, 256);                                                     \
+        else if (gt.max_size <= 5) DRACO_VOTE(5, AA, 3, 256);        /* s = 2: three groups of five */             \
+        else if (gt.max_size <= 8) DRACO_VOTE(8, AA, 2, 256);                                                     \
+        else if (gt.max_size <= 12) DRACO_VOTE(12, AA, 1, 128);                                                   \
+        else if (gt.max_size <= 16) DRACO_VOTE(16, AA, 1, 128);      /* 16 rows of 4 words per thread: small blocks keep 3 per SM */ \
+        else DRACO_VOTE(0, AA, 1, 256);                                                                           \
+    } while (0)
+    if (adj) DRACO_VOTE_BY_SIZE(true);
+    else DRACO_VOTE_BY_SIZE(false);
+#undef DRACO_VOTE_BY_SIZE
 #undef DRACO_VOTE
-    DRACO_CUDA(cudaGetLastError());
-    rep_finish_kernel<<<1, 128, 0, st>>>(gt, scratch, flags, p->flags_dev, p->info_dev, generic);
     DRACO_CUDA(cudaGetLastError());
     return DRACO_OK;
 }

@@ -4,7 +4,7 @@ import pytest
 import torch
 
 import draco_inputs as di
-from gpu_util import dev, host
+from gpu_util import dev, fp32_sequential_sum, host
 from oracle import draco_oracle as orc
 
 pytestmark = pytest.mark.gpu
@@ -32,3 +32,46 @@ def test_cyclic_encode_writes_every_entry_rounded_once(code, n, s, d):
     terms = np.abs(orc.cyc_W(n, s)).sum(axis=0)[:, None] * np.abs(G).max()
     for a, b in ((got.real, want.real), (got.imag, want.imag)):
         assert (np.abs(a - b) <= 2.0 ** -24 * np.abs(b) + 1e-14 * terms * n + 1e-37).all()
+
+
+# group sizes of every register variant and of the streamed one (21); a block takes 1024, 512 or 256 columns, fewer on short
+# vectors, and the encoder writes 8 less
+REPETITION = [(n, s, d) for n, s in [(7, 1), (4, 1), (15, 2), (45, 3), (45, 5), (42, 10)]
+              for d in (1, 3, 63, 247, 249, 255, 257, 1021, 30_003)]
+
+
+@pytest.mark.parametrize("n,s,d", REPETITION)
+def test_repetition_rows_off_the_grid(n, s, d):
+    import paper_1803_09877_b200 as dr
+    plan = dr.Plan(n, s, d, dr.REP)
+    G = di.gradient_rows(5 + n + d, n, d)
+    buf = torch.full((n * d + 64,), 7.0, dtype=torch.float32, device="cuda")
+    plan.encode(dev(G), buf[32:])
+    out = host(buf)
+    assert (out[:32] == 7.0).all() and (out[32 + n * d:] == 7.0).all()
+    Z = out[32:32 + n * d].reshape(n, d)
+    groups = orc.rep_groups(n, s)
+    for first, size in groups:
+        sums = fp32_sequential_sum(G[first:first + size])
+        for j in range(first, first + size):
+            np.testing.assert_array_equal(Z[j].view(np.uint32), sums.view(np.uint32))
+    R = Z.copy()
+    adv = di.choose_adversaries(n + d, n, s)
+    di.apply_adversaries(R, adv, [di.ADV_REVGRAD] * s, [100.0] * s, seed=3)
+    R[groups[0][0]:groups[0][0] + groups[0][1], d - 1] = np.arange(groups[0][1], dtype=np.float32) + 1     # no majority there
+    want = orc.rep_decode(R, n, s)
+    Rd = dev(R)
+    u = torch.full((d + 8,), 7.0, dtype=torch.float32, device="cuda")
+    maj = torch.empty((len(groups), d), dtype=torch.float32, device="cuda")
+    flags = torch.empty(n, dtype=torch.uint8, device="cuda")
+    for _ in range(2):                                    # the second call finds what the first left behind
+        plan.rep_vote(Rd, u, maj, flags)
+        info = plan.info()
+        np.testing.assert_array_equal(host(flags).astype(bool), want["flags"])
+        np.testing.assert_array_equal(host(u)[:d].view(np.uint32), fp32_sequential_sum(want["maj"]).view(np.uint32))
+        assert (host(u)[d:] == 7.0).all()
+        np.testing.assert_array_equal(host(maj).view(np.uint32), want["maj"].view(np.uint32))
+        assert info["no_majority"] == want["no_majority"] and info["n_flagged"] == int(np.sum(want["flags"]))
+    w = torch.ones(d, dtype=torch.float32, device="cuda")
+    plan.decode_update(Rd, flags, w, 0.5)
+    np.testing.assert_array_equal(host(w), np.float32(1.0) - np.float32(0.5) * host(u)[:d])
