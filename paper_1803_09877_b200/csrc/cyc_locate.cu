@@ -22,6 +22,7 @@ namespace {
 
 constexpr int kThreads = kProjectWarps * 32;
 constexpr int kSolveThreads = 512;
+constexpr int kProjectChunk = 512;    // coordinates per warp and step of the few-rows projection
 
 __device__ __forceinline__ double2 cmul(double2 a, double2 b) {
     return make_double2(a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x);
@@ -65,11 +66,11 @@ __device__ __forceinline__ double* q_partials(double2* partial, int cap, int n) 
 // independent; f is read twice, 1 % more traffic): 16 rows per warp in registers halve the blocks per SM
 // (0.79 of the copy bandwidth at n = 105), and per-lane sums in shared memory left the compiler too few
 // registers to keep its loads in flight once the squared norms were added (0.98 -> 0.68).
-template <int RPW, bool VEC2>
+template <int RPW, bool VEC2, int TILE>
 __global__ void __launch_bounds__(kThreads, 4)
 cyc_project_kernel(const float2* __restrict__ R, const float* __restrict__ f, int64_t len, int64_t ld, int n,
                    int row0, int nrows, double2* __restrict__ partial, int cap, int accumulate) {
-    __shared__ __align__(16) double fs[kProjectTile];
+    __shared__ __align__(16) double fs[TILE];
     // Running sums of row warp + r * 8 over this block's tiles, kept by lane 0 of the row's warp: after every tile
     // the warp adds its lanes' sums up (fixed butterfly order) and lane 0 adds the result here.  Keeping them in
     // registers instead (2 RPW doubles per lane) left too few of the 64 registers for eight 128-bit loads in flight.
@@ -93,11 +94,11 @@ cyc_project_kernel(const float2* __restrict__ R, const float* __restrict__ f, in
         }
     }
 
-    const int64_t ntiles = (len + kProjectTile - 1) / kProjectTile;
+    const int64_t ntiles = (len + TILE - 1) / TILE;
     for (int64_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
-        const int64_t c0 = tile * kProjectTile;
-        const int cnt = (int)((len - c0) < kProjectTile ? (len - c0) : kProjectTile);
-        for (int i = threadIdx.x; i < kProjectTile; i += kThreads) fs[i] = (i < cnt) ? (double)__ldcs(f + c0 + i) : 0.0;
+        const int64_t c0 = tile * TILE;
+        const int cnt = (int)((len - c0) < TILE ? (len - c0) : TILE);
+        for (int i = threadIdx.x; i < TILE; i += kThreads) fs[i] = (i < cnt) ? (double)__ldcs(f + c0 + i) : 0.0;
         __syncthreads();
 #pragma unroll
         for (int r = 0; r < RPW; ++r) {
@@ -106,10 +107,10 @@ cyc_project_kernel(const float2* __restrict__ R, const float* __restrict__ f, in
                 const float2* row = R + (int64_t)j * ld + c0;
                 double eq = 0.0;
                 double ar = 0.0, ai = 0.0;
-                if (VEC2 && cnt == kProjectTile) {
+                if (VEC2 && cnt == TILE) {
                     const float4* row4 = reinterpret_cast<const float4*>(row);
 #pragma unroll 1
-                    for (int step0 = 0; step0 < kProjectTile / 64; step0 += 8) {
+                    for (int step0 = 0; step0 < TILE / 64; step0 += 8) {
                         float4 v[8];
 #pragma unroll
                         for (int q = 0; q < 8; ++q) v[q] = __ldcs(row4 + (step0 + q) * 32 + lane);
@@ -124,12 +125,22 @@ cyc_project_kernel(const float2* __restrict__ R, const float* __restrict__ f, in
                         }
                     }
                 } else {
-                    for (int i = lane; i < cnt; i += 32) {
-                        const float2 v = __ldcs(row + i);
-                        const double ff = fs[i], x0 = (double)v.x, y0 = (double)v.y;
-                        ar = fma(ff, x0, ar);
-                        ai = fma(ff, y0, ai);
-                        eq = fma(y0, y0, fma(x0, x0, eq));
+                    // 8-byte loads, which any row start allows; entries beyond the vector count as zero (and fs is zero there)
+#pragma unroll 1
+                    for (int step0 = 0; step0 * 32 < cnt; step0 += 16) {
+                        float2 v[16];
+#pragma unroll
+                        for (int q = 0; q < 16; ++q) {
+                            const int i = (step0 + q) * 32 + lane;
+                            v[q] = i < cnt ? __ldcs(row + i) : make_float2(0.f, 0.f);
+                        }
+#pragma unroll
+                        for (int q = 0; q < 16; ++q) {
+                            const double ff = fs[(step0 + q) * 32 + lane], x0 = (double)v[q].x, y0 = (double)v[q].y;
+                            ar = fma(ff, x0, ar);
+                            ai = fma(ff, y0, ai);
+                            eq = fma(y0, y0, fma(x0, x0, eq));
+                        }
                     }
                 }
                 ar = warp_sum(ar);
@@ -165,102 +176,103 @@ cyc_project_kernel(const float2* __restrict__ R, const float* __restrict__ f, in
 }
 
 // The same projection for few rows (n <= 16): with one or two rows per warp the block-wide tile
-// barriers of the kernel above dominate, so here every warp works alone on 256-coordinate chunks
-// of all n rows, with f for its chunk in registers (8 values per lane) and no
-// shared memory or barrier in the loop.  Per-lane running sums in fp64 registers (2 n doubles).
-template <bool VEC2>
-__global__ void __launch_bounds__(kThreads, 2)
+// barriers of the kernel above dominate, so here every warp works alone on 512-coordinate chunks of all n rows, row by row,
+// with f for its chunk in registers (16 values per lane), eight 128-bit loads per lane in flight and no barrier in the loop.
+// The three sums of a row live in registers for that row only; the lanes' sums are added by a butterfly and kept by lane 0 in
+// shared memory, so that three blocks fit on an SM.  With per-lane sums of all rows (32 doubles, and 16 more did not fit) it
+// was two blocks and ten shuffles per row and 256 coordinates for q alone (n = 15, reduction included: d = 30 M 602 us, now
+// 524 = 7.1 TB/s; d = 1 M 44 us, now 30; d = 30 M + 1, whose rows went 32 coordinates at a time, 3750 us, now 630).
+constexpr int kFewRows = 16;
+template <bool VEC2, bool SPLIT>
+__global__ void __launch_bounds__(kThreads, 3)
 cyc_project_fewrows_kernel(const float2* __restrict__ R, const float* __restrict__ f, int64_t len, int64_t ld, int n,
                            double2* __restrict__ partial, int cap, int accumulate) {
-    constexpr int NMAX = 16, CH = 256;
-    __shared__ double2 wsum[kProjectWarps][NMAX];
-    __shared__ double wq[kProjectWarps][NMAX];
+    constexpr int CH = kProjectChunk;
+    __shared__ double2 es[kProjectWarps][kFewRows];
+    __shared__ double qs[kProjectWarps][kFewRows];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    double accr[NMAX], acci[NMAX];
-#pragma unroll
-    for (int j = 0; j < NMAX; ++j) { accr[j] = 0.0; acci[j] = 0.0; }
-    if (lane < NMAX) wq[warp][lane] = 0.0;               // q_j of this warp's chunks: summed over the lanes per chunk, kept here
+    if (lane < kFewRows) {
+        es[warp][lane] = make_double2(0.0, 0.0);
+        qs[warp][lane] = 0.0;
+    }
     __syncwarp();
+    auto keep = [&](int j, double ar, double ai, double eq) {
+        ar = warp_sum(ar);
+        ai = warp_sum(ai);
+        eq = warp_sum(eq);
+        if (lane == 0) {
+            double2 acc = es[warp][j];
+            acc.x += ar;
+            acc.y += ai;
+            es[warp][j] = acc;
+            qs[warp][j] += eq;
+        }
+    };
+    int row0 = 0, nrows = n;                             // rows of this block
+    if (SPLIT) {
+        const int per = (n + (int)gridDim.y - 1) / (int)gridDim.y;
+        row0 = (int)blockIdx.y * per;
+        nrows = (n - row0) < per ? (n - row0) : per;
+    }
     const int64_t nchunks = (len + CH - 1) / CH;
     const int64_t nwarps = (int64_t)gridDim.x * kProjectWarps;
     for (int64_t chunk = (int64_t)blockIdx.x * kProjectWarps + warp; chunk < nchunks; chunk += nwarps) {
         const int64_t c0 = chunk * CH;
         const int cnt = (int)((len - c0) < CH ? (len - c0) : CH);
         if (VEC2 && cnt == CH) {
-            float2 ff[4];
+            float2 ff[CH / 64];
 #pragma unroll
-            for (int q = 0; q < 4; ++q) ff[q] = __ldcs(reinterpret_cast<const float2*>(f + c0) + q * 32 + lane);
+            for (int q = 0; q < CH / 64; ++q) ff[q] = __ldcs(reinterpret_cast<const float2*>(f + c0) + q * 32 + lane);
+#pragma unroll 1
+            for (int j = row0; j < row0 + nrows; ++j) {
+                const float4* row = reinterpret_cast<const float4*>(R + (int64_t)j * ld + c0) + lane;
+                float4 v[CH / 64];
 #pragma unroll
-            for (int jj = 0; jj < NMAX; jj += 2) {
-                if (jj < n) {
-                    float4 va[4], vb[4];
-                    const float4* ra = reinterpret_cast<const float4*>(R + (int64_t)jj * ld + c0);
-                    const bool two = jj + 1 < n;
-                    const float4* rb = reinterpret_cast<const float4*>(R + (int64_t)(two ? jj + 1 : jj) * ld + c0);
+                for (int q = 0; q < CH / 64; ++q) v[q] = __ldcs(row + q * 32);
+                double ar = 0.0, ai = 0.0, eq = 0.0;
 #pragma unroll
-                    for (int q = 0; q < 4; ++q) va[q] = __ldcs(ra + q * 32 + lane);
-                    if (two) {
-#pragma unroll
-                        for (int q = 0; q < 4; ++q) vb[q] = __ldcs(rb + q * 32 + lane);
-                    }
-                    double qa = 0.0, qb = 0.0;
-#pragma unroll
-                    for (int q = 0; q < 4; ++q) {
-                        const double fx = (double)ff[q].x, fy = (double)ff[q].y;     // shared by the two rows
-                        double x0 = (double)va[q].x, y0 = (double)va[q].y, x1 = (double)va[q].z, y1 = (double)va[q].w;
-                        accr[jj] = fma(fx, x0, accr[jj]); acci[jj] = fma(fx, y0, acci[jj]);
-                        accr[jj] = fma(fy, x1, accr[jj]); acci[jj] = fma(fy, y1, acci[jj]);
-                        qa = fma(x0, x0, qa); qa = fma(y0, y0, qa); qa = fma(x1, x1, qa); qa = fma(y1, y1, qa);
-                        if (two) {
-                            x0 = (double)vb[q].x; y0 = (double)vb[q].y; x1 = (double)vb[q].z; y1 = (double)vb[q].w;
-                            accr[jj + 1] = fma(fx, x0, accr[jj + 1]); acci[jj + 1] = fma(fx, y0, acci[jj + 1]);
-                            accr[jj + 1] = fma(fy, x1, accr[jj + 1]); acci[jj + 1] = fma(fy, y1, acci[jj + 1]);
-                            qb = fma(x0, x0, qb); qb = fma(y0, y0, qb); qb = fma(x1, x1, qb); qb = fma(y1, y1, qb);
-                        }
-                    }
-                    qa = warp_sum(qa);
-                    qb = warp_sum(qb);
-                    if (lane == 0) { wq[warp][jj] += qa; if (two) wq[warp][jj + 1] += qb; }
+                for (int q = 0; q < CH / 64; ++q) {
+                    const double fx = (double)ff[q].x, fy = (double)ff[q].y;
+                    const double x0 = (double)v[q].x, y0 = (double)v[q].y, x1 = (double)v[q].z, y1 = (double)v[q].w;
+                    ar = fma(fx, x0, ar); ai = fma(fx, y0, ai);
+                    ar = fma(fy, x1, ar); ai = fma(fy, y1, ai);
+                    eq = fma(x0, x0, eq); eq = fma(y0, y0, eq);
+                    eq = fma(x1, x1, eq); eq = fma(y1, y1, eq);
                 }
+                keep(j, ar, ai, eq);
             }
-        } else {
-            for (int i0 = 0; i0 < cnt; i0 += 32) {           // every lane takes part in the sums over the lanes below
-                const int i = i0 + lane;
-                const bool valid = i < cnt;
-                const double fi = valid ? (double)__ldcs(f + c0 + i) : 0.0;
+        } else {                                             // any row start, ragged chunk: 8-byte loads, zero beyond the vector
+            float ff[CH / 32];
 #pragma unroll
-                for (int j = 0; j < NMAX; ++j)
-                    if (j < n) {
-                        const float2 v = valid ? __ldcs(R + (int64_t)j * ld + c0 + i) : make_float2(0.f, 0.f);
-                        const double x0 = (double)v.x, y0 = (double)v.y;
-                        accr[j] = fma(fi, x0, accr[j]);
-                        acci[j] = fma(fi, y0, acci[j]);
-                        const double qv = warp_sum(fma(y0, y0, x0 * x0));
-                        if (lane == 0) wq[warp][j] += qv;
-                    }
+            for (int q = 0; q < CH / 32; ++q) ff[q] = q * 32 + lane < cnt ? __ldcs(f + c0 + q * 32 + lane) : 0.0f;
+#pragma unroll 1
+            for (int j = row0; j < row0 + nrows; ++j) {
+                const float2* row = R + (int64_t)j * ld + c0 + lane;
+                float2 v[CH / 32];
+#pragma unroll
+                for (int q = 0; q < CH / 32; ++q) v[q] = q * 32 + lane < cnt ? __ldcs(row + q * 32) : make_float2(0.f, 0.f);
+                double ar = 0.0, ai = 0.0, eq = 0.0;
+#pragma unroll
+                for (int q = 0; q < CH / 32; ++q) {
+                    const double fx = (double)ff[q], x0 = (double)v[q].x, y0 = (double)v[q].y;
+                    ar = fma(fx, x0, ar); ai = fma(fx, y0, ai);
+                    eq = fma(y0, y0, fma(x0, x0, eq));
+                }
+                keep(j, ar, ai, eq);
             }
         }
-    }
-#pragma unroll
-    for (int j = 0; j < NMAX; ++j) {
-        double a = accr[j], b = acci[j];
-#pragma unroll
-        for (int off = 16; off > 0; off >>= 1) {
-            a += __shfl_xor_sync(0xffffffffu, a, off);
-            b += __shfl_xor_sync(0xffffffffu, b, off);
-        }
-        if (lane == 0) wsum[warp][j] = make_double2(a, b);
     }
     __syncthreads();
-    if (threadIdx.x < n) {
+    if ((int)threadIdx.x < nrows) {
+        const int j = row0 + threadIdx.x;
         double a = 0.0, b = 0.0, c = 0.0;
         for (int w = 0; w < kProjectWarps; ++w) {            // fixed order: reproducible
-            a += wsum[w][threadIdx.x].x;
-            b += wsum[w][threadIdx.x].y;
-            c += wq[w][threadIdx.x];
+            a += es[w][j].x;
+            b += es[w][j].y;
+            c += qs[w][j];
         }
-        double2* dst = partial + (int64_t)blockIdx.x * n + threadIdx.x;
-        double* qdst = q_partials(partial, cap, n) + (int64_t)blockIdx.x * n + threadIdx.x;
+        double2* dst = partial + (int64_t)blockIdx.x * n + j;
+        double* qdst = q_partials(partial, cap, n) + (int64_t)blockIdx.x * n + j;
         if (accumulate) { a += dst->x; b += dst->y; c += *qdst; }
         *dst = make_double2(a, b);
         *qdst = c;
@@ -610,7 +622,8 @@ __device__ int warp_jacobi_pinv(double2* A, double2* V, const double2* rhs, int 
 }
 
 constexpr int kSmallDim = 16;         // systems up to this size are solved in shared memory by one warp
-constexpr int kFusedReduceMax = 64;   // up to this many block partials are added up by the locator kernel itself
+constexpr int kFusedReduceMax = 16 * kSolveThreads;   // up to this many block partials (3 per block and node) are added up by the
+                                                      // locator kernel itself: 16 loads per thread, about the 4 us of the reduction kernel
 
 // ------------------------------------------------------------------ decode vector
 // With B = [C_L]_{.,V} and A = [C_L]_{.,U}: A A^H = I - B B^H, so the minimum-norm solution of
@@ -752,29 +765,35 @@ cyc_solve_kernel(CycDevice* cd, const double2* __restrict__ e_in, const double2*
             qv[tid] = reinterpret_cast<const double*>(e_in + n)[tid];
         }
     } else {
-        // the projection's block partials, few enough to add up here: thread (j, part) takes one of the three sums of
-        // node j over the blocks in ascending order, four running sums in rotation (all loads of a round are in flight
-        // together), combined in a fixed order: reproducible
+        // the projection's block partials, few enough to add up here: `per` lanes (a power of two) take one of the three sums of
+        // a node, lane l the blocks l, l + per, .. in ascending order, eight loads in flight; then a butterfly: reproducible
         const double* __restrict__ qpartial = reinterpret_cast<const double*>(partial + (int64_t)cap * n);
-        for (int idx = tid; idx < 3 * n; idx += blockDim.x) {
-            const int part = idx / n, j = idx - part * n;
-            double acc[4] = {0.0, 0.0, 0.0, 0.0};
-            for (int b0 = 0; b0 < used; b0 += 4) {
-                double v[4];
+        int per = 1;
+        while (per < 32 && 2 * per * 3 * n <= kSolveThreads) per *= 2;
+        const int sub = tid & (per - 1);
+        for (int idx = tid / per; idx < (3 * n + kSolveThreads / per - 1) / (kSolveThreads / per) * (kSolveThreads / per);
+             idx += kSolveThreads / per) {
+            const bool on = idx < 3 * n;
+            const int part = on ? idx / n : 0, j = on ? idx - part * n : 0;
+            double acc = 0.0;
+            for (int b0 = sub; b0 < used; b0 += 8 * per) {
+                double v[8];
 #pragma unroll
-                for (int k = 0; k < 4; ++k) {
-                    const int b = (b0 + k < used) ? b0 + k : 0;
-                    const int64_t at = (int64_t)b * n + j;
+                for (int k = 0; k < 8; ++k) {
+                    const int b = b0 + k * per;
+                    const int64_t at = (int64_t)(b < used ? b : b0) * n + j;
                     v[k] = part == 2 ? __ldcg(qpartial + at) : (part == 0 ? __ldcg(&partial[at].x) : __ldcg(&partial[at].y));
                 }
 #pragma unroll
-                for (int k = 0; k < 4; ++k)
-                    if (b0 + k < used) acc[k] += v[k];
+                for (int k = 0; k < 8; ++k)
+                    if (b0 + k * per < used) acc += v[k];
             }
-            const double sum = (acc[0] + acc[1]) + (acc[2] + acc[3]);
-            if (part == 0) e[j].x = sum;
-            else if (part == 1) e[j].y = sum;
-            else qv[j] = sum;
+            for (int off = per >> 1; off > 0; off >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, off);
+            if (on && sub == 0) {
+                if (part == 0) e[j].x = acc;
+                else if (part == 1) e[j].y = acc;
+                else qv[j] = acc;
+            }
         }
     }
     __syncthreads();
@@ -1013,25 +1032,50 @@ cyc_solve_kernel(CycDevice* cd, const double2* __restrict__ e_in, const double2*
 
 }  // namespace
 
-// Blocks of the projection: four per SM (six measured slower at n = 15).
-int project_grid_size(int sm_count, int) { return sm_count * 4; }
+// Capacity in blocks of the projection's partials: four per SM.
 int project_grid_size(int sm_count) { return sm_count * 4; }
 
+// Blocks along x of a projection, cap at most, each leaving one partial per node: no more than have work, so that short
+// vectors leave a handful of partials.  n <= 16: a chunk per warp; as many blocks as are resident at once (three per SM) with
+// the chunks dealt out evenly.  Otherwise a tile per block; short vectors take smaller tiles, whose warps are through after one
+// round of loads (d = 4096, n = 45: four rounds one after the other with the full tile).
+struct ProjectShape {
+    int grid, gridy, tile;
+};
+static ProjectShape project_shape(int cap, int sm_count, int64_t len, int n) {
+    ProjectShape g = {1, 1, kProjectTile};
+    if (n <= kFewRows) {
+        const int64_t work = (len + (int64_t)kProjectChunk * kProjectWarps - 1) / ((int64_t)kProjectChunk * kProjectWarps);
+        int64_t room = 3 * (int64_t)sm_count;
+        if (room > cap) room = cap;
+        const int64_t rounds = (work + room - 1) / room;
+        g.grid = (int)((work + rounds - 1) / rounds);
+        g.gridy = (int)(3 * (int64_t)sm_count / g.grid);     // what is left over divides the rows
+        if (g.gridy > n) g.gridy = n;
+        if (g.gridy < 1) g.gridy = 1;
+        return g;
+    }
+    if (len <= (int64_t)kProjectTileShort * 64) g.tile = kProjectTileShort;
+    const int64_t work = (len + g.tile - 1) / g.tile;
+    g.grid = (int)(work < cap ? work : cap);
+    return g;
+}
+
 // All launches of one projection: n <= 16 the few-rows kernel, n <= 64 one launch of the tile kernel, otherwise two
-// launches of it over half the rows each.  partial: [cap][n] double2 followed by [cap][n] double.  No more blocks
-// are launched than have work (a tile each, or eight 256-coordinate chunks each in the few-rows kernel): short
-// vectors then leave a handful of partials instead of several hundred zeros.  Returns the grid used in *grid_used.
-static cudaError_t launch_project_kernels(int cap, cudaStream_t st, const float2* R, const float* f, int64_t len,
-                                          int64_t ld, int n, double2* partial, int accumulate, int* grid_used) {
+// launches of it over half the rows each.  partial: [cap][n] double2 followed by [cap][n] double.
+static cudaError_t launch_project_kernels(int cap, const ProjectShape& shape, cudaStream_t st, const float2* R, const float* f,
+                                          int64_t len, int64_t ld, int n, double2* partial, int accumulate) {
     const bool vec2 = (ld % 2 == 0);
-    const int64_t work = n <= 16 ? (len + 256 * kProjectWarps - 1) / (256 * kProjectWarps)
-                                 : (len + kProjectTile - 1) / kProjectTile;
-    int grid = cap;
-    if (work < grid) grid = (int)(work < 1 ? 1 : work);
-    *grid_used = grid;
-    if (n <= 16) {
-        if (vec2) cyc_project_fewrows_kernel<true><<<grid, kThreads, 0, st>>>(R, f, len, ld, n, partial, cap, accumulate);
-        else cyc_project_fewrows_kernel<false><<<grid, kThreads, 0, st>>>(R, f, len, ld, n, partial, cap, accumulate);
+    const int grid = shape.grid, tile = shape.tile;
+    if (n <= kFewRows) {
+        const dim3 grid2(grid, shape.gridy);
+#define DRACO_FEW(VV, SS) cyc_project_fewrows_kernel<VV, SS><<<grid2, kThreads, 0, st>>>(R, f, len, ld, n, partial, cap, accumulate)
+        if (shape.gridy > 1) {
+            if (vec2) DRACO_FEW(true, true); else DRACO_FEW(false, true);
+        } else {
+            if (vec2) DRACO_FEW(true, false); else DRACO_FEW(false, false);
+        }
+#undef DRACO_FEW
         return cudaGetLastError();
     }
     const int parts = n <= 64 ? 1 : 2;
@@ -1045,15 +1089,24 @@ static cudaError_t launch_project_kernels(int cap, cudaStream_t st, const float2
         if (ysplit < 1) ysplit = 1;
     }
     const dim3 grid2(grid, ysplit);
+#define DRACO_PROJECT(RR, VV, TT) \
+    cyc_project_kernel<RR, VV, TT><<<grid2, kThreads, 0, st>>>(R, f, len, ld, n, row0, nrows, partial, cap, accumulate)
+#define DRACO_PROJECT_TILE(RR, VV)                                           \
+    do {                                                                     \
+        if (tile == kProjectTile) DRACO_PROJECT(RR, VV, kProjectTile);       \
+        else DRACO_PROJECT(RR, VV, kProjectTileShort);                       \
+    } while (0)
     for (int row0 = 0; row0 < n; row0 += per) {
         const int nrows = (n - row0) < per ? (n - row0) : per;
         if (nrows <= 32) {
-            if (vec2) cyc_project_kernel<4, true><<<grid2, kThreads, 0, st>>>(R, f, len, ld, n, row0, nrows, partial, cap, accumulate);
-            else cyc_project_kernel<4, false><<<grid2, kThreads, 0, st>>>(R, f, len, ld, n, row0, nrows, partial, cap, accumulate);
+            if (vec2) DRACO_PROJECT_TILE(4, true);
+            else DRACO_PROJECT_TILE(4, false);
         } else {
-            if (vec2) cyc_project_kernel<8, true><<<grid2, kThreads, 0, st>>>(R, f, len, ld, n, row0, nrows, partial, cap, accumulate);
-            else cyc_project_kernel<8, false><<<grid2, kThreads, 0, st>>>(R, f, len, ld, n, row0, nrows, partial, cap, accumulate);
+            if (vec2) DRACO_PROJECT_TILE(8, true);
+            else DRACO_PROJECT_TILE(8, false);
         }
+#undef DRACO_PROJECT_TILE
+#undef DRACO_PROJECT
         const cudaError_t err = cudaGetLastError();
         if (err != cudaSuccess) return err;
     }
@@ -1065,9 +1118,8 @@ static cudaError_t launch_project_kernels(int cap, cudaStream_t st, const float2
 int launch_cyc_project(draco_plan* p, const float2* R, const float* f, int64_t len, int64_t ld, bool accumulate,
                        cudaStream_t st) {
     const int cap = p->project_grid;
-    const int64_t work = p->n <= 16 ? (len + 256 * kProjectWarps - 1) / (256 * kProjectWarps)
-                                    : (len + kProjectTile - 1) / kProjectTile;
-    const int want = (int)(work < cap ? (work < 1 ? 1 : work) : cap);
+    const ProjectShape shape = project_shape(cap, p->sm_count, len, p->n);
+    const int want = shape.grid;
     if (!accumulate) p->project_used = 0;
     if (accumulate && want > p->project_used) {
         const size_t n = (size_t)p->n;
@@ -1076,9 +1128,8 @@ int launch_cyc_project(draco_plan* p, const float2* R, const float* f, int64_t l
         double* q = reinterpret_cast<double*>(p->partial_dev + (size_t)cap * n);
         DRACO_CUDA(cudaMemsetAsync(q + (size_t)p->project_used * n, 0, sizeof(double) * n * (size_t)(want - p->project_used), st));
     }
-    int used = 0;
-    DRACO_CUDA(launch_project_kernels(cap, st, R, f, len, ld, p->n, p->partial_dev, accumulate ? 1 : 0, &used));
-    if (used > p->project_used) p->project_used = used;
+    DRACO_CUDA(launch_project_kernels(cap, shape, st, R, f, len, ld, p->n, p->partial_dev, accumulate ? 1 : 0));
+    if (want > p->project_used) p->project_used = want;
     return DRACO_OK;
 }
 
@@ -1096,7 +1147,7 @@ int launch_cyc_solve(draco_plan* p, const double2* e, uint8_t* flags, bool with_
     const double2* partial = nullptr;
     int used = 0;
     if (!e) {
-        if (p->project_used <= kFusedReduceMax) {
+        if (3 * p->n * p->project_used <= kFusedReduceMax) {
             partial = p->partial_dev;
             used = p->project_used;
         } else {
@@ -1173,9 +1224,9 @@ extern "C" int draco_cyc_project_noalloc(int n, int64_t d, const void* R, const 
     const float2* Rc = static_cast<const float2*>(R);
     // Every block that is launched writes its n partials and only those are read back, so nothing has
     // to be cleared between calls even though the array keeps the previous call's contents.
-    int used = 0;
-    DRACO_CUDA(launch_project_kernels(grid, st, Rc, f, d, d, n, partial, 0, &used));
-    cyc_reduce_partials_kernel<<<n, kReduceThreads, 0, st>>>(partial, used, grid, n, e);
+    const ProjectShape shape = project_shape(grid, sms, d, n);
+    DRACO_CUDA(launch_project_kernels(grid, shape, st, Rc, f, d, d, n, partial, 0));
+    cyc_reduce_partials_kernel<<<n, kReduceThreads, 0, st>>>(partial, shape.grid, grid, n, e);
     DRACO_CUDA(cudaGetLastError());
     return DRACO_OK;
 }

@@ -22,6 +22,9 @@ constexpr int kUnroll = 8;
 
 // PACKED: the vectors carry two gradient coordinates per complex entry (Section 3, last
 // paragraph): u[i] = Re(u-hat_i), u[len + i] = Im(u-hat_i) for len + i < d_packed.
+// VEC2: a thread owns two neighbouring coordinates, one 16-byte load per row.  Otherwise (odd row starts) two coordinates
+// kThreads apart and two 8-byte loads per row, so that a warp's loads are contiguous and as many bytes are in flight (one
+// coordinate per thread and no batch of rows: n = 45, d = 20,000,001 1589 us with the decode vector, now 1107).
 template <bool VEC2, bool PACKED>
 __global__ void __launch_bounds__(kThreads)
 cyc_recover_kernel(const float2* __restrict__ R, int64_t len, int64_t ld, const CycDevice* __restrict__ cd,
@@ -36,82 +39,89 @@ cyc_recover_kernel(const float2* __restrict__ R, int64_t len, int64_t ld, const 
     }
     __syncthreads();
     const int64_t stride = (int64_t)gridDim.x * kThreads;
-    if (VEC2) {
-        const int64_t nvec = len / 2;
-        for (int64_t v = (int64_t)blockIdx.x * kThreads + threadIdx.x; v < nvec; v += stride) {
-            const float2* col = R + v * 2;
-            const bool sampled = !PACKED && ((v >> 5) & 7) == 0;       // coordinates 2 v, 2 v + 1: floor(i / 64) mod 8 == 0
-            double a0 = 0.0, a1 = 0.0, i0 = 0.0, i1 = 0.0;
-            for (int k0 = 0; k0 < count; k0 += kUnroll) {
-                float4 x[kUnroll];
+    const int64_t units = VEC2 ? len / 2 : (len + 2 * kThreads - 1) / (2 * kThreads) * kThreads;
+    for (int64_t v = (int64_t)blockIdx.x * kThreads + threadIdx.x; v < units; v += stride) {
+        // this thread's coordinates i and i + step
+        const int64_t i = VEC2 ? 2 * v : v / kThreads * (2 * kThreads) + threadIdx.x;
+        if (!VEC2 && i >= len) continue;
+        const bool two = VEC2 || i + kThreads < len;
+        const int step = VEC2 ? 1 : two ? kThreads : 0;                // beyond the vector: the first coordinate again
+        const float2* col = R + i;
+        // adjacent: both coordinates of a thread lie in the same run of 64; apart: the second is four runs on, never sampled
+        const bool sampled = !PACKED && ((i >> 6) & 7) == 0;
+        double a0 = 0.0, a1 = 0.0, i0 = 0.0, i1 = 0.0;
+        for (int k0 = 0; k0 < count; k0 += kUnroll) {
+            float4 x[kUnroll];
 #pragma unroll
-                for (int q = 0; q < kUnroll; ++q)
-                    if (k0 + q < count) x[q] = __ldcs(reinterpret_cast<const float4*>(col + (int64_t)rows[k0 + q] * ld));
+            for (int q = 0; q < kUnroll; ++q)
+                if (k0 + q < count) {
+                    const float2* row = col + (int64_t)rows[k0 + q] * ld;
+                    if (VEC2) {
+                        x[q] = __ldcs(reinterpret_cast<const float4*>(row));
+                    } else {
+                        const float2 y0 = __ldcs(row), y1 = __ldcs(row + step);
+                        x[q] = make_float4(y0.x, y0.y, y1.x, y1.y);
+                    }
+                }
 #pragma unroll
-                for (int q = 0; q < kUnroll; ++q)
-                    if (k0 + q < count) {
-                        const double2 b = bs[k0 + q];
-                        const double xr0 = (double)x[q].x, xi0 = (double)x[q].y, xr1 = (double)x[q].z, xi1 = (double)x[q].w;
-                        a0 = fma(b.x, xr0, a0);
-                        a0 = fma(-b.y, xi0, a0);
-                        a1 = fma(b.x, xr1, a1);
-                        a1 = fma(-b.y, xi1, a1);
-                        if (PACKED || sampled) {
-                            i0 = fma(b.x, xi0, i0);
-                            i0 = fma(b.y, xr0, i0);
+            for (int q = 0; q < kUnroll; ++q)
+                if (k0 + q < count) {
+                    const double2 b = bs[k0 + q];
+                    const double xr0 = (double)x[q].x, xi0 = (double)x[q].y, xr1 = (double)x[q].z, xi1 = (double)x[q].w;
+                    a0 = fma(b.x, xr0, a0);
+                    a0 = fma(-b.y, xi0, a0);
+                    a1 = fma(b.x, xr1, a1);
+                    a1 = fma(-b.y, xi1, a1);
+                    if (PACKED || sampled) {
+                        i0 = fma(b.x, xi0, i0);
+                        i0 = fma(b.y, xr0, i0);
+                        if (PACKED || VEC2) {
                             i1 = fma(b.x, xi1, i1);
                             i1 = fma(b.y, xr1, i1);
                         }
                     }
+                }
+        }
+        if (sampled) {
+            im_max = fmax(im_max, fabs(i0));
+            re_max = fmax(re_max, fabs(a0));
+            if (VEC2) {
+                im_max = fmax(im_max, fabs(i1));
+                re_max = fmax(re_max, fabs(a1));
             }
-            if (sampled) {
-                im_max = fmax(im_max, fmax(fabs(i0), fabs(i1)));
-                re_max = fmax(re_max, fmax(fabs(a0), fabs(a1)));
-            }
+        }
+        if constexpr (VEC2) {
             if (u != nullptr) {
-                __stcs(reinterpret_cast<float2*>(u + v * 2), make_float2((float)a0, (float)a1));
-                if (PACKED) __stcs(reinterpret_cast<float2*>(u + len + v * 2), make_float2((float)i0, (float)i1));
+                __stcs(reinterpret_cast<float2*>(u + i), make_float2((float)a0, (float)a1));
+                if (PACKED) __stcs(reinterpret_cast<float2*>(u + len + i), make_float2((float)i0, (float)i1));
             }
             if (w != nullptr) {                          // w <- w - scale * u, u rounded to fp32 first as when stored
-                float2* wp = reinterpret_cast<float2*>(w + v * 2);
+                float2* wp = reinterpret_cast<float2*>(w + i);
                 float2 wv = *wp;
                 wv.x = fmaf(-scale, (float)a0, wv.x);
                 wv.y = fmaf(-scale, (float)a1, wv.y);
                 *wp = wv;
                 if (PACKED) {
-                    wp = reinterpret_cast<float2*>(w + len + v * 2);
+                    wp = reinterpret_cast<float2*>(w + len + i);
                     wv = *wp;
                     wv.x = fmaf(-scale, (float)i0, wv.x);
                     wv.y = fmaf(-scale, (float)i1, wv.y);
                     *wp = wv;
                 }
             }
-        }
-    } else {
-        for (int64_t i = (int64_t)blockIdx.x * kThreads + threadIdx.x; i < len; i += stride) {
-            const bool sampled = !PACKED && ((i >> 6) & 7) == 0;
-            double a0 = 0.0, i0 = 0.0;
-            for (int k = 0; k < count; ++k) {
-                const float2 x = __ldcs(R + (int64_t)rows[k] * ld + i);
-                const double2 b = bs[k];
-                a0 = fma(b.x, (double)x.x, a0);
-                a0 = fma(-b.y, (double)x.y, a0);
-                if (PACKED || sampled) {
-                    i0 = fma(b.x, (double)x.y, i0);
-                    i0 = fma(b.y, (double)x.x, i0);
-                }
-            }
-            if (sampled) {
-                im_max = fmax(im_max, fabs(i0));
-                re_max = fmax(re_max, fabs(a0));
-            }
+        } else {
+            const bool im0 = PACKED && len + i < d_packed, im1 = PACKED && two && len + i + step < d_packed;
             if (u != nullptr) {
                 u[i] = (float)a0;
-                if (PACKED && len + i < d_packed) u[len + i] = (float)i0;
+                if (two) u[i + step] = (float)a1;
+                if (im0) u[len + i] = (float)i0;
+                if (im1) u[len + i + step] = (float)i1;
             }
             if (w != nullptr) {
                 w[i] = fmaf(-scale, (float)a0, w[i]);
-                if (PACKED && len + i < d_packed) w[len + i] = fmaf(-scale, (float)i0, w[len + i]);
+                if (two) w[i + step] = fmaf(-scale, (float)a1, w[i + step]);
+                if (im0) w[len + i] = fmaf(-scale, (float)i0, w[len + i]);
+                if (im1) w[len + i + step] = fmaf(-scale, (float)i1, w[len + i + step]);
             }
         }
     }
@@ -138,7 +148,7 @@ int launch_cyc_recover(draco_plan* p, const float2* R, int64_t len, int64_t ld, 
     const bool packed = d_packed > 0;
     // 64-bit stores of u need len even; in packed mode the second half starts at u + len and must cover it fully
     const bool vec2 = (len % 2 == 0) && (ld % 2 == 0) && (!packed || d_packed == 2 * len);
-    const int64_t nvec = vec2 ? len / 2 : len;
+    const int64_t nvec = (len + 1) / 2;
     int64_t want = (nvec + kThreads - 1) / kThreads;
     const int64_t cap = (int64_t)p->sm_count * 16;
     if (want > cap) want = cap;

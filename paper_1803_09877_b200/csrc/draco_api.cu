@@ -175,7 +175,7 @@ int draco_plan_create(int n, int s, int64_t d, int code, draco_plan** out) {
         DRACO_TRY(cudaMalloc(&p->taps_full_dev, sizeof(double2) * taps_full.size()));
         DRACO_TRY(cudaMemcpy(p->taps_full_dev, taps_full.data(), sizeof(double2) * taps_full.size(),
                              cudaMemcpyHostToDevice));
-        p->project_grid = project_grid_size(p->sm_count, n);
+        p->project_grid = project_grid_size(p->sm_count);
         // per block and node: a double2 partial of e_j, then (after all of those) a double partial of q_j
         const size_t partial_bytes = (sizeof(double2) + sizeof(double)) * (size_t)p->project_grid * n;
         DRACO_TRY(cudaMalloc(&p->partial_dev, partial_bytes));

@@ -11,6 +11,7 @@ namespace draco {
 constexpr int kMaxN = DRACO_MAX_N;
 constexpr int kMaxTaps = 15;          // 2 s + 1 for the register-window encoder (s <= 7)
 constexpr int kProjectTile = 2048;    // coordinates per tile of the projection kernel
+constexpr int kProjectTileShort = 512;   // the same for short vectors
 constexpr int kProjectWarps = 8;
 constexpr double kMarginBar = 10.0;        // locator_margin below this, or ..
 constexpr double kImResidualBar = 1e-2;    // .. im_residual above this fraction of re_max: status DRACO_EUNSURE
@@ -133,6 +134,5 @@ int launch_generate(float* out, int rows, int64_t len, int64_t ld, int64_t i0, i
 int launch_corrupt(float* R, int64_t row_pitch, int64_t nvals, int64_t v0, const int* node, const int* model,
                    const float* param, int n_adv, uint64_t seed, bool is_complex, int sm_count, cudaStream_t st);
 int project_grid_size(int sm_count);
-int project_grid_size(int sm_count, int n);
 
 }  // namespace draco

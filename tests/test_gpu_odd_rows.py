@@ -75,3 +75,44 @@ def test_repetition_rows_off_the_grid(n, s, d):
     w = torch.ones(d, dtype=torch.float32, device="cuda")
     plan.decode_update(Rd, flags, w, 0.5)
     np.testing.assert_array_equal(host(w), np.float32(1.0) - np.float32(0.5) * host(u)[:d])
+
+
+# the few-rows projection takes 512 coordinates per warp and splits the rows of short vectors over blocks, the tile kernel 512 or
+# (from 32,769 coordinates on) 2048 per block; the recovery takes 512 per block
+DECODE = [(code, n, s, d) for code in ("CYC", "CYC_PACKED")
+          for n, s, d in [(5, 1, 1), (15, 2, 511), (15, 2, 513), (16, 3, 4097), (15, 2, 8200), (17, 2, 513), (45, 5, 2047),
+                          (45, 5, 4100), (45, 5, 32_767), (45, 5, 32_770), (45, 5, 65_539), (70, 2, 1025), (105, 2, 33_001)]]
+
+
+@pytest.mark.parametrize("code,n,s,d", DECODE)
+def test_projection_and_recovery_at_the_edges_of_their_tiles(code, n, s, d):
+    """Projection: exact products, so only the order of fp64 additions differs from the oracle (bars as in test_gpu_cyc.py);
+    recovery: fp64 sums of the given vectors, rounded once to fp32 (2^-24 of the largest entry, 1e-7)."""
+    import paper_1803_09877_b200 as dr
+    packed = code == "CYC_PACKED"
+    plan = dr.Plan(n, s, d, getattr(dr, code))
+    v = (d + 1) // 2 if packed else d
+    G = di.gradient_rows(11 + n + d, n, d)
+    R = (orc.cyc_encode_packed if packed else orc.cyc_encode)(G, n, s)
+    adv = di.choose_adversaries(n + d, n, s) if v > 64 else []
+    di.apply_adversaries(R, adv, [di.ADV_REVGRAD] * len(adv), [100.0] * len(adv), seed=3)
+    f = di.projection_vector(7 + d, v)
+    Rd, fd = dev(R), dev(f)
+    e = torch.empty(3 * n, dtype=torch.float64, device="cuda")
+    plan.cyc_project(Rd, fd, e)
+    got = host(e)
+    eo, qo = orc.cyc_project(R, f), orc.cyc_project_energy(R)
+    assert np.abs(got[:2 * n].view(np.complex128) - eo).max() <= 1e-11 * np.sqrt(2 * v * qo.max())
+    assert (np.abs(got[2 * n:] - qo) <= 1e-12 * qo).all()
+    flags = torch.empty(n, dtype=torch.uint8, device="cuda")
+    u = torch.full((d + 8,), 7.0, dtype=torch.float32, device="cuda")
+    plan.locate_decode(Rd, fd, flags, u)
+    fl = host(flags).astype(bool)
+    assert set(adv) <= set(np.flatnonzero(fl))
+    want = orc.cyc_decode_packed(R, n, s, fl, d) if packed else orc.cyc_decode(R, n, s, fl)
+    assert (host(u)[d:] == 7.0).all()
+    assert np.abs(host(u)[:d] - want).max() <= 1e-7 * np.abs(want).max() + 1e-9
+    w = torch.ones(d + 8, dtype=torch.float32, device="cuda")
+    plan.decode_update(Rd, flags, w, 0.5)
+    np.testing.assert_array_equal(host(w)[:d], np.float32(1.0) - np.float32(0.5) * host(u)[:d])
+    assert (host(w)[d:] == 1.0).all()
