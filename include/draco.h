@@ -84,7 +84,8 @@ typedef struct draco_info {
     int32_t internal_error; /* non-zero: a kernel gave up a bounded wait (sticky); draco_get_info then returns DRACO_EINTERNAL.
                                Always 0 with the current kernels, none of which spins on a flag */
     int32_t svd_sweeps;    /* cyclic locate: Jacobi sweeps the singular-value iteration of the s x s syndrome system took
-                              (0 when it was skipped: s = 0, or all syndromes within the cutoff); negative (minus the
+                              (0 when it was skipped: s = 0, all syndromes within the cutoff, or a system of
+                              at most 8 unknowns that certainly has full rank, which is solved directly); negative (minus the
                               limit of 60) when it was still rotating at the limit: rank and V are then not to be trusted */
     double locator_margin; /* cyclic locate: |t| of the weakest flagged node / |t| of the strongest unflagged one (exactly
                               `rank` entries of t are non-zero in exact arithmetic, so this is large when the flags can be

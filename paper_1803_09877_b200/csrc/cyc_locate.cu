@@ -12,6 +12,8 @@
 //
 // The small solves run in fp64 in a single thread block; only the projection touches HBM:
 // 8 n len + 4 len bytes read.
+#include <math.h>
+
 #include <mutex>
 
 #include "draco_internal.cuh"
@@ -625,33 +627,196 @@ constexpr int kSmallDim = 16;         // systems up to this size are solved in s
 constexpr int kFusedReduceMax = 16 * kSolveThreads;   // up to this many block partials (3 per block and node) are added up by the
                                                       // locator kernel itself: 16 loads per thread, about the 4 us of the reduction kernel
 
+// ------------------------------------------------------------------ small systems, one warp
+// What follows runs once per call, in one warp or one block, so its time is the chain of dependent operations and the
+// instructions fetched for it (with the compiler's own unrolling 774 requests went past the instruction cache in 37,000
+// cycles, n = 45, s = 5, five adversaries): loops are kept rolled, the elements of a system are spread over the lanes, and nothing divides by
+// a run-time number (x mod n and the lanes of a sum are shifts and one multiplication).
+constexpr int kRegSystem = 8;                              // unknowns of the systems below
+struct ModN {                                              // x mod n for x < 2^16; magic = ceil(2^32 / n)
+    uint32_t n, magic;
+    __device__ __forceinline__ int operator()(int x) const { return x - (int)(__umulhi((uint32_t)x, magic) * n); }
+};
+
+// Gauss-Jordan elimination of the S x W matrix M (row-major, W <= 2 S + 1; its first S columns the system, the others right-hand
+// sides), S <= 8.  PIVOT: rows are searched (never moved); otherwise the system is Hermitian positive definite.  Lane k gets the
+// row and the reciprocal of pivot k: unknown k of right-hand side c is M[row][c] * inv.  False on a zero or non-finite pivot.
+// QN: elements per lane, 32 QN >= S W.
+template <bool PIVOT, int QN>
+__device__ __forceinline__ bool warp_eliminate(double2* M, int S, int W, int& row, double2& inv) {
+    const unsigned full = 0xffffffffu;
+    const int lane = threadIdx.x & 31;
+    int ei[QN], ci[QN];                                    // row and column of this lane's elements; others: element 0, not stored
+    bool live[QN];
+#pragma unroll
+    for (int q = 0; q < QN; ++q) {
+        const int e = lane + 32 * q;
+        live[q] = e < S * W;
+        ei[q] = live[q] ? (int)((float)e * __frcp_rn((float)W) + 1e-3f) : 0;        // e / W, e < 136
+        ci[q] = live[q] ? e - ei[q] * W : 0;
+    }
+    unsigned used = 0;
+    row = 0;
+    inv = make_double2(0.0, 0.0);
+#pragma unroll 1
+    for (int k = 0; k < S; ++k) {
+        int pr = k;
+        if (PIVOT) {                                       // largest |.|^2 to 20 bits
+            const bool open = lane < S && !((used >> lane) & 1u);
+            const double size = cabs2(M[(open ? lane : 0) * W + k]);
+            const unsigned key = open ? (unsigned)__double2hiint(size) + 1u : 0u;
+            const unsigned best = __reduce_max_sync(full, key);
+            pr = __ffs(__ballot_sync(full, open && key == best)) - 1;
+            used |= 1u << pr;
+        }
+        const double2 p = M[pr * W + k];
+        double2 f[QN], m[QN], v[QN];
+#pragma unroll
+        for (int q = 0; q < QN; ++q) {
+            f[q] = M[ei[q] * W + k];
+            m[q] = M[pr * W + ci[q]];
+            v[q] = M[ei[q] * W + ci[q]];
+        }
+        const double den = cabs2(p);
+        if (!(den > 0.0 && den < 1e300)) return false;     // the same in every lane
+        const double r = 1.0 / den;
+        const double2 ip = make_double2(p.x * r, -p.y * r);
+        if (lane == k) { row = pr; inv = ip; }
+#pragma unroll
+        for (int q = 0; q < QN; ++q) {
+            const double2 g = cmul(m[q], ip), t = cmul(f[q], g);
+            v[q].x -= t.x;
+            v[q].y -= t.y;
+        }
+        __syncwarp();
+#pragma unroll
+        for (int q = 0; q < QN; ++q)
+            if (live[q] && ei[q] != pr) M[ei[q] * W + ci[q]] = v[q];
+        __syncwarp();
+    }
+    return true;
+}
+
+// beta = A^{-1} rhs for the S x S syndrome system (row i: [h_{n-S-1-i} .. h_{n-2-i}] beta = h_{n-1-i}) when it certainly has
+// full rank: sigma_min >= 1 / |A^{-1}|_F, so |A^{-1}|_F cut < 0.9 leaves every singular value above the cutoff and the
+// pseudo-inverse solution is the solution.  The usual case, s adversaries at work, then needs no singular-value iteration
+// (n = 45, s = 5: 24 us, the elimination about 2 us).  The bound on |A|_F |A^{-1}|_F keeps the computed inverse good to
+// three digits.  Returns false, with beta untouched, when there is any doubt.  M: S (2 S + 1) elements of work space.
+__device__ __forceinline__ bool warp_full_rank_solve(double2* M, const double2* h, int n, int S, double cut, double fro2,
+                                                     double2* beta) {
+    const int lane = threadIdx.x & 31, W = 2 * S + 1;
+#pragma unroll 4
+    for (int i = 0; i < S; ++i)
+        if (lane < W) M[i * W + lane] = lane <= S ? h[n - S - 1 - i + lane] : make_double2(lane == S + 1 + i ? 1.0 : 0.0, 0.0);
+    __syncwarp();
+    int row;
+    double2 inv;
+    if (!(S * W <= 64 ? warp_eliminate<true, 2>(M, S, W, row, inv) : warp_eliminate<true, 5>(M, S, W, row, inv))) return false;
+    double inv2 = 0.0;
+    if (lane < S) {
+#pragma unroll 1
+        for (int c = S + 1; c < W; ++c) inv2 += cabs2(M[row * W + c]);
+        inv2 *= cabs2(inv);
+    }
+    inv2 = warp_sum(inv2);
+    if (!(inv2 * cut * cut < 0.81 && inv2 * fro2 < 1e24)) return false;
+    if (lane < S) beta[lane] = cmul(M[row * W + S], inv);
+    __syncwarp();
+    return true;
+}
+
+// h_l = sum_u beta_u h_{l+u-S}, l = 0 .. count - 1, from h_{n-S} .. h_{n-1}: one thread, the last S values in registers.  The
+// terms of the older values are summed in two chains while the newest value is still on its way, so that a step waits for
+// two multiply-adds.
+template <int S>
+__device__ __noinline__ void run_recurrence(double2* h, int n, int count, const double2* beta) {
+    double2 b[S], w[S];
+#pragma unroll
+    for (int u = 0; u < S; ++u) {
+        b[u] = beta[u];
+        w[u] = h[n - S + u];
+    }
+#pragma unroll 1
+    for (int l0 = 0; l0 < count; l0 += S) {
+#pragma unroll
+        for (int k = 0; k < S; ++k) {                              // w[(k + u) mod S] = h_{l+u-S}
+            double2 a = make_double2(0.0, 0.0), c = make_double2(0.0, 0.0);
+#pragma unroll
+            for (int u = 0; u < S - 1; ++u) {
+                const double2 v = w[(k + u) % S];
+                a.x = fma(b[u].x, v.x, a.x);
+                c.x = fma(-b[u].y, v.y, c.x);
+                a.y = fma(b[u].x, v.y, a.y);
+                c.y = fma(b[u].y, v.x, c.y);
+            }
+            const double2 v = w[(k + S - 1) % S];
+            const double2 o = make_double2(a.x + c.x, a.y + c.y);
+            w[k] = make_double2(fma(-b[S - 1].y, v.y, fma(b[S - 1].x, v.x, o.x)), fma(b[S - 1].y, v.x, fma(b[S - 1].x, v.y, o.y)));
+            h[l0 + k < count ? l0 + k : kMaxN] = w[k];             // beyond the end: the spare entry
+        }
+    }
+}
+
+#define DRACO_BY_SIZE(size, CALL)                                                                            \
+    switch (size) {                                                                                          \
+        case 1: CALL(1); break;                                                                              \
+        case 2: CALL(2); break;                                                                              \
+        case 3: CALL(3); break;                                                                              \
+        case 4: CALL(4); break;                                                                              \
+        case 5: CALL(5); break;                                                                              \
+        case 6: CALL(6); break;                                                                              \
+        case 7: CALL(7); break;                                                                              \
+        case 8: CALL(8); break;                                                                              \
+        default: break;                                                                                      \
+    }
+static_assert(kRegSystem == 8, "the sizes of DRACO_BY_SIZE");
+
+// Lanes that share one of `items` sums, as a shift: the largest power of two that the block has threads for, 32 at most.  The
+// groups do not straddle warps, and every thread of the block takes part in the butterfly.
+__device__ __forceinline__ int lanes_shift(int items) {
+    const int shift = 9 - (32 - __clz(items - 1));
+    return shift > 5 ? 5 : shift < 0 ? 0 : shift;
+}
+static_assert(kSolveThreads == 512, "2^9 in lanes_shift");
+__device__ __forceinline__ double lane_sum(double a, int shift) {
+#pragma unroll 1
+    for (int off = (1 << shift) >> 1; off > 0; off >>= 1) a += __shfl_xor_sync(0xffffffffu, a, off);
+    return a;
+}
+
+// The nodes with fl != 0 in ascending order; returns how many.  bits: kMaxN / 32 words.  Called by the whole block.
+__device__ __forceinline__ int list_flagged(const uint8_t* fl, int n, int* list, uint32_t* bits) {
+    const int tid = threadIdx.x;
+    const bool set = tid < n && fl[tid] != 0;
+    const uint32_t w = __ballot_sync(0xffffffffu, set);
+    if (tid < kMaxN && (tid & 31) == 0) bits[tid >> 5] = w;
+    __syncthreads();
+    int total = 0, before = 0;
+#pragma unroll
+    for (int k = 0; k < kMaxN / 32; ++k) {
+        if (k == (tid >> 5)) before = total + __popc(bits[k] & ((1u << (tid & 31)) - 1u));
+        total += __popc(bits[k]);
+    }
+    if (set) list[before] = tid;
+    __syncthreads();
+    return total;
+}
+
 // ------------------------------------------------------------------ decode vector
 // With B = [C_L]_{.,V} and A = [C_L]_{.,U}: A A^H = I - B B^H, so the minimum-norm solution of
 // A b_U = e_last is b_U = A^H y, y = e_last + B (I - B^H B)^{-1} B^H e_last, and
 // I - B^H B = [C_R]_{.,V}^H [C_R]_{.,V} is only |V| x |V| (|V| <= 2 s).
-// Called by every thread of a block of kSolveThreads threads; flags may point to global or to shared memory.
-__device__ void decode_vector_body(CycDevice* cd, const uint8_t* flags, int n, int s, DeviceInfo* info) {
-    __shared__ int vlist[kMaxN], rowbestc[kMaxN], perm_s[kMaxN], sh[4], a_s;
-    __shared__ uint8_t fl[kMaxN];
+// Called by every thread of a block of kSolveThreads threads; fl (the flags) and tw (w^k) in shared memory.
+__device__ void decode_vector_body(CycDevice* cd, const uint8_t* fl, const double2* tw, int n, int s, ModN mod, double rsn,
+                                   DeviceInfo* info) {
+    __shared__ int vlist[kMaxN], rowbestc[kMaxN], perm_s[kMaxN], sh[4];
+    __shared__ uint32_t bits[kMaxN / 32];
     __shared__ double rowbest[kMaxN];
-    __shared__ double2 y[kMaxN], tw[kMaxN], x_s[kMaxN], b_s[kMaxN];
+    __shared__ double2 y[kMaxN], x_s[kMaxN];
     __shared__ double2 As[kSmallDim * (kSmallDim + 1)];
     const int tid = threadIdx.x;
     const int rows = n - 2 * s, L = rows - 1;
-    const double rsn = 1.0 / sqrt((double)n);
-    if (tid < n) {
-        tw[tid] = cd->twiddle[tid];
-        fl[tid] = flags[tid];
-    }
-    __syncthreads();
-    if (tid == 0) {
-        int a = 0;
-        for (int j = 0; j < n; ++j)
-            if (fl[j]) vlist[a++] = j;
-        a_s = a;
-    }
-    __syncthreads();
-    const int a = a_s;
+    const int a = list_flagged(fl, n, vlist, bits);
     if (a > 2 * s) {                                       // fewer than n - 2 s rows left: no b exists
         if (tid < n) cd->b[tid] = make_double2(0.0, 0.0);
         if (tid == 0) {
@@ -664,31 +829,43 @@ __device__ void decode_vector_body(CycDevice* cd, const uint8_t* flags, int n, i
     if (a > 0) {
         const bool small = a <= kSmallDim;
         double2* A = small ? As : cd->work;
-        for (int idx = tid; idx < a * (a + 1); idx += blockDim.x) {
-            const int p = idx / (a + 1), q = idx % (a + 1);
-            double2 val;
-            if (q < a) {                                   // (1/n) sum_{m >= n-2s} w^(m (v_q - v_p))
-                int dv = vlist[q] - vlist[p];
-                if (dv < 0) dv += n;
-                double re = 0.0, im = 0.0;
-                int k = ((n - 2 * s) * dv) % n;
-                for (int m = n - 2 * s; m < n; ++m) {
-                    const double2 w = tw[k];
-                    re += w.x;
-                    im += w.y;
-                    k += dv;
-                    if (k >= n) k -= n;
+#pragma unroll 1
+        for (int p = tid >> 5; p < a; p += kSolveThreads / 32)                  // a row per warp
+#pragma unroll 1
+            for (int q = tid & 31; q <= a; q += 32) {
+                double2 val;
+                if (q < a) {                               // (1/n) sum_{m >= n-2s} w^(m (v_q - v_p))
+                    int dv = vlist[q] - vlist[p];
+                    if (dv < 0) dv += n;
+                    double re = 0.0, im = 0.0;
+                    int k = mod((n - 2 * s) * dv);
+#pragma unroll 1
+                    for (int m = n - 2 * s; m < n; ++m) {
+                        const double2 w = tw[k];
+                        re += w.x;
+                        im += w.y;
+                        k += dv;
+                        if (k >= n) k -= n;
+                    }
+                    val = make_double2(re * (rsn * rsn), im * (rsn * rsn));
+                } else {                                   // conj(C[L][v_p])
+                    const double2 w = tw[mod(L * vlist[p])];
+                    val = make_double2(w.x * rsn, -w.y * rsn);
                 }
-                val = make_double2(re / n, im / n);
-            } else {                                       // conj(C[L][v_p])
-                const double2 w = tw[(L * vlist[p]) % n];
-                val = make_double2(w.x * rsn, -w.y * rsn);
+                A[p * (a + 1) + q] = val;
             }
-            A[idx] = val;
-        }
         __syncthreads();
         if (small) {
-            if (tid < 32) block_gauss_jordan<true>(A, a, 0.0, x, perm_s, rowbest, rowbestc, sh);
+            if (tid < 32) {
+                if (a <= kRegSystem) {                     // [C_R]_{.,V} has full column rank: positive definite
+                    int row;
+                    double2 inv;
+                    warp_eliminate<false, 3>(As, a, a + 1, row, inv);
+                    if (tid < a) x_s[tid] = cmul(As[row * (a + 1) + a], inv);
+                } else {
+                    block_gauss_jordan<true>(As, a, 0.0, x, perm_s, rowbest, rowbestc, sh);
+                }
+            }
             __syncthreads();
         } else {
             block_gauss_jordan<false>(A, a, 0.0, x, perm_s, rowbest, rowbestc, sh);
@@ -696,8 +873,9 @@ __device__ void decode_vector_body(CycDevice* cd, const uint8_t* flags, int n, i
     }
     if (tid < rows) {
         double re = (tid == L) ? 1.0 : 0.0, im = 0.0;
+#pragma unroll 1
         for (int p = 0; p < a; ++p) {
-            const double2 w = tw[(tid * vlist[p]) % n];
+            const double2 w = tw[mod(tid * vlist[p])];
             const double2 q = cmul(w, x[p]);
             re += q.x * rsn;
             im += q.y * rsn;
@@ -705,32 +883,35 @@ __device__ void decode_vector_body(CycDevice* cd, const uint8_t* flags, int n, i
         y[tid] = make_double2(re, im);
     }
     __syncthreads();
-    if (tid < n) {
-        double2 b = make_double2(0.0, 0.0);
-        if (!fl[tid]) {
-            double re = 0.0, im = 0.0;
-            int k = 0;                                     // (m tid) mod n
-            for (int m = 0; m < rows; ++m) {
-                const double2 q = cmulc(y[m], tw[k]);
-                re += q.x;
-                im += q.y;
-                k += tid;
-                if (k >= n) k -= n;
-            }
-            b = make_double2(re * rsn, im * rsn);
+    const int shift = lanes_shift(n), per = 1 << shift, node = tid >> shift, sub = tid & (per - 1);
+    double re = 0.0, im = 0.0;
+    if (node < n) {
+        int k = mod(sub * node);                           // (m node) mod n
+        const int step = mod(per * node);
+#pragma unroll 1
+        for (int m = sub; m < rows; m += per) {
+            const double2 q = cmulc(y[m], tw[k]);
+            re += q.x;
+            im += q.y;
+            k += step;
+            if (k >= n) k -= n;
         }
-        cd->b[tid] = b;
-        b_s[tid] = b;
     }
-    __syncthreads();
-    // the active rows in ascending order: position = number of unflagged nodes before this one
-    if (tid < n && !fl[tid]) {
-        int k = 0;
-        for (int j = 0; j < tid; ++j) k += fl[j] ? 0 : 1;
-        cd->active[k] = tid;
-        cd->b_active[k] = b_s[tid];
+    re = lane_sum(re, shift);
+    im = lane_sum(im, shift);
+    if (node < n && sub == 0) {
+        const bool flagged = fl[node] != 0;
+        const double2 b = flagged ? make_double2(0.0, 0.0) : make_double2(re * rsn, im * rsn);
+        cd->b[node] = b;
+        if (!flagged) {                                    // the active rows in ascending order
+            int before = 0;
+            for (int k = 0; k <= node >> 5; ++k)
+                before += __popc(k < node >> 5 ? bits[k] : bits[k] & ((1u << (node & 31)) - 1u));
+            cd->active[node - before] = node;
+            cd->b_active[node - before] = b;
+        }
     }
-    if (tid == 0) {
+    if (tid == kSolveThreads - 1) {
         info->n_active = n - a;
         info->n_flagged = a;
         info->im_residual_bits = 0ull;                     // the recovery kernel's blocks merge their maxima into these
@@ -741,22 +922,36 @@ __device__ void decode_vector_body(CycDevice* cd, const uint8_t* flags, int n, i
 
 
 __global__ void __launch_bounds__(kSolveThreads)
-cyc_decode_vector_kernel(CycDevice* cd, const uint8_t* __restrict__ flags, int n, int s, DeviceInfo* info) {
-    decode_vector_body(cd, flags, n, s, info);
+cyc_decode_vector_kernel(CycDevice* cd, const uint8_t* __restrict__ flags, int n, int s, ModN mod, double rsn,
+                         DeviceInfo* info) {
+    __shared__ double2 tw[kMaxN];
+    __shared__ uint8_t fl[kMaxN];
+    const int tid = threadIdx.x;
+    if (tid < n) {
+        tw[tid] = cd->twiddle[tid];
+        fl[tid] = flags[tid];
+    }
+    __syncthreads();
+    decode_vector_body(cd, fl, tw, n, s, mod, rsn, info);
 }
 
 // ------------------------------------------------------------------ locator after the projection
+// One block; what bounds it is the length of the chain of dependent fp64 operations (9 cycles each), shuffles (46 a double)
+// and barriers (59), not their number.  Sums over the nodes are therefore spread over as many lanes as the block has, lists
+// come from ballots, and the systems of up to 8 unknowns are solved in one warp's registers.  n = 45, s = 5, five adversaries,
+// decode vector included: 47 us with a thread per sum, one-thread list building and the singular-value iteration.
 __global__ void __launch_bounds__(kSolveThreads)
 cyc_solve_kernel(CycDevice* cd, const double2* __restrict__ e_in, const double2* __restrict__ partial, int used, int cap,
-                 int n, int s, double theta, uint8_t* flags, uint8_t* flags2, DeviceInfo* info, int with_b) {
-    __shared__ double2 e[kMaxN], h[kMaxN], tw[kMaxN];
+                 int n, int s, double theta, ModN mod, double rsn, uint8_t* flags, uint8_t* flags2, DeviceInfo* info, int with_b) {
+    __shared__ double2 e[kMaxN], h[kMaxN + 1], tw[kMaxN];
     __shared__ double2 As[kSmallDim * kSmallDim], Vs[kSmallDim * kSmallDim];
     __shared__ double2 rhs_s[kMaxN / 2], beta_s[kMaxN / 2], coef_s[kMaxN / 2];
     __shared__ double mag[kMaxN], sorted[kMaxN], qv[kMaxN];
-    __shared__ int sh[4], count;
-    __shared__ double scale_s, maxsyn_s;
+    __shared__ int sh[4], rank_s;
+    __shared__ double maxsyn_s;
     const int tid = threadIdx.x;
-    const double rsn = 1.0 / sqrt((double)n);
+    // lanes of one node, for the sums over the nodes
+    const int shift = lanes_shift(n), per = 1 << shift, node = tid >> shift, sub = tid & (per - 1);
 
     if (tid < n) tw[tid] = cd->twiddle[tid];
     if (e_in != nullptr) {                                 // the projection record: n (re, im) pairs, then n values q_j
@@ -765,31 +960,31 @@ cyc_solve_kernel(CycDevice* cd, const double2* __restrict__ e_in, const double2*
             qv[tid] = reinterpret_cast<const double*>(e_in + n)[tid];
         }
     } else {
-        // the projection's block partials, few enough to add up here: `per` lanes (a power of two) take one of the three sums of
-        // a node, lane l the blocks l, l + per, .. in ascending order, eight loads in flight; then a butterfly: reproducible
+        // the projection's block partials, few enough to add up here: `lanes` lanes take one of the three sums of a node,
+        // lane l the blocks l, l + lanes, .. in ascending order, eight loads in flight; then a butterfly: reproducible
         const double* __restrict__ qpartial = reinterpret_cast<const double*>(partial + (int64_t)cap * n);
-        int per = 1;
-        while (per < 32 && 2 * per * 3 * n <= kSolveThreads) per *= 2;
-        const int sub = tid & (per - 1);
-        for (int idx = tid / per; idx < (3 * n + kSolveThreads / per - 1) / (kSolveThreads / per) * (kSolveThreads / per);
-             idx += kSolveThreads / per) {
+        const int lshift = lanes_shift(3 * n), lanes = 1 << lshift, first = tid & (lanes - 1), groups = kSolveThreads >> lshift;
+#pragma unroll 1
+        for (int base = 0; base < 3 * n; base += groups) {
+            const int idx = base + (tid >> lshift);
             const bool on = idx < 3 * n;
-            const int part = on ? idx / n : 0, j = on ? idx - part * n : 0;
+            const int part = idx < n || !on ? 0 : idx < 2 * n ? 1 : 2, j = on ? idx - part * n : 0;
             double acc = 0.0;
-            for (int b0 = sub; b0 < used; b0 += 8 * per) {
+#pragma unroll 1
+            for (int b0 = first; b0 < used; b0 += 8 * lanes) {
                 double v[8];
 #pragma unroll
                 for (int k = 0; k < 8; ++k) {
-                    const int b = b0 + k * per;
+                    const int b = b0 + k * lanes;
                     const int64_t at = (int64_t)(b < used ? b : b0) * n + j;
                     v[k] = part == 2 ? __ldcg(qpartial + at) : (part == 0 ? __ldcg(&partial[at].x) : __ldcg(&partial[at].y));
                 }
 #pragma unroll
                 for (int k = 0; k < 8; ++k)
-                    if (b0 + k * per < used) acc += v[k];
+                    if (b0 + k * lanes < used) acc += v[k];
             }
-            for (int off = per >> 1; off > 0; off >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, off);
-            if (on && sub == 0) {
+            acc = lane_sum(acc, lshift);
+            if (on && first == 0) {
                 if (part == 0) e[j].x = acc;
                 else if (part == 1) e[j].y = acc;
                 else qv[j] = acc;
@@ -800,50 +995,61 @@ cyc_solve_kernel(CycDevice* cd, const double2* __restrict__ e_in, const double2*
     // A node whose record is not finite sent NaN or infinities: no honest vector does.  It is flagged outright and
     // its record taken as zero, which keeps the arithmetic below finite (the node then looks to the locator as if it
     // had sent a vector with f R_j = 0: one of the at most s errors it locates anyway).
-    __shared__ uint8_t nonfinite[kMaxN];
+    __shared__ uint8_t fl_s[kMaxN];                        // V so far
     if (tid < n) {
         const bool bad = !(isfinite(e[tid].x) && isfinite(e[tid].y) && isfinite(qv[tid]));
-        nonfinite[tid] = bad ? 1 : 0;
+        fl_s[tid] = bad ? 1 : 0;
         if (bad) {
             e[tid] = make_double2(0.0, 0.0);
             qv[tid] = 0.0;
         }
-        cd->e[tid] = e[tid];
         mag[tid] = sqrt(qv[tid]);
         h[tid] = make_double2(0.0, 0.0);
     }
-    if (tid == 0) { count = 0; sh[3] = 0; }
+    if (tid == 0) sh[3] = 0;
     __syncthreads();
-    // scale = median of q_j^(1/2) by rank counting
-    if (tid < n) {
+    __shared__ double2 syn[kMaxN];                         // h_{n-2s+i}: every pass rewrites h
+    {
+        // scale = median of q_j^(1/2) by rank counting
         int rank = 0;
-        for (int k = 0; k < n; ++k) rank += (mag[k] < mag[tid]) || (mag[k] == mag[tid] && k < tid);
-        sorted[rank] = mag[tid];
-    }
-    __syncthreads();
-    if (tid == 0) scale_s = (n & 1) ? sorted[n / 2] : 0.5 * (sorted[n / 2 - 1] + sorted[n / 2]);
-    // syndromes h_m = n^(-1/2) sum_j e_j w^(-m j), m = n-2s .. n-1
-    if (tid < 2 * s) {
-        const int m = n - 2 * s + tid;
+        if (node < n)
+#pragma unroll 1
+            for (int k = sub; k < n; k += per) rank += (mag[k] < mag[node]) || (mag[k] == mag[node] && k < node);
+#pragma unroll 1
+        for (int off = per >> 1; off > 0; off >>= 1) rank += __shfl_xor_sync(0xffffffffu, rank, off);
+        if (node < n && sub == 0) sorted[rank] = mag[node];
+        // syndromes h_m = n^(-1/2) sum_j e_j w^(-m j), m = n-2s .. n-1
+        const int lshift = lanes_shift(2 * s), lanes = 1 << lshift, i = tid >> lshift, first = tid & (lanes - 1);
         double a = 0.0, b = 0.0;
-        int idx = 0;                                       // (m j) mod n
-        for (int j = 0; j < n; ++j) {
-            const double2 q = cmulc(e[j], tw[idx]);
-            a += q.x;
-            b += q.y;
-            idx += m;
-            if (idx >= n) idx -= n;
+        if (i < 2 * s) {
+            const int m = n - 2 * s + i;
+            int idx = mod(first * m);                      // (m j) mod n
+            const int step = mod(lanes * m);
+#pragma unroll 1
+            for (int j = first; j < n; j += lanes) {
+                const double2 q = cmulc(e[j], tw[idx]);
+                a += q.x;
+                b += q.y;
+                idx += step;
+                if (idx >= n) idx -= n;
+            }
         }
-        h[m] = make_double2(a * rsn, b * rsn);
+        a = lane_sum(a, lshift);
+        b = lane_sum(b, lshift);
+        if (i < 2 * s && first == 0) syn[i] = make_double2(a * rsn, b * rsn);
     }
     __syncthreads();
-    if (tid == 0) {
+    const double scale = (n & 1) ? sorted[n / 2] : 0.5 * (sorted[n / 2 - 1] + sorted[n / 2]);
+    if (tid >= kSolveThreads - 32) {                       // the last warp, which the passes below leave idle
+        const int lane = tid & 31;
         double mx = 0.0;
-        for (int m = n - 2 * s; m < n; ++m) mx = fmax(mx, sqrt(cabs2(h[m])));
-        maxsyn_s = mx;
+#pragma unroll 1
+        for (int i = lane; i < 2 * s; i += 32) mx = fmax(mx, cabs2(syn[i]));
+#pragma unroll
+        for (int off = 16; off > 0; off >>= 1) mx = fmax(mx, __shfl_xor_sync(0xffffffffu, mx, off));
+        if (lane == 0) maxsyn_s = sqrt(mx);
     }
-    __syncthreads();
-    const double tol = theta * scale_s;
+    const double tol = theta * scale;
     // The locator runs in passes.  The first is the paper's phi.  Each further pass treats the set E of nodes flagged
     // so far (nodes with a non-finite record from the start) as erasures: with lambda(x) = prod_{v in E} (x - w^v) =
     // sum_k lambda_k x^k the sequence T_m = sum_k lambda_k h_{m-k} no longer contains the nodes of E and is again a sum
@@ -851,182 +1057,218 @@ cyc_solve_kernel(CycDevice* cd, const double2* __restrict__ e_in, const double2*
     // through the same Toeplitz system, recurrence and IDFT with s2 in place of s.  A pass that finds nothing (the
     // usual second pass: rounding noise) ends the search.  Adversaries that sit side by side make one pass miss some of
     // them with complex64 vectors; the passes then still end with a set that contains them all.
-    __shared__ double2 syn[kMaxN];                         // h_{n-2s+i}: every pass rewrites h
     __shared__ double2 lam[kMaxN + 2];
-    __shared__ uint8_t fl_s[kMaxN];                        // V so far
     __shared__ int elist[kMaxN];
-    __shared__ int eps_s, rank_total_s, sweeps_s;
-    __shared__ double lam1_s, margin_s;
-    if (tid < 2 * s) syn[tid] = h[n - 2 * s + tid];
-    if (tid < n) {
-        fl_s[tid] = nonfinite[tid];
-        cd->t[tid] = make_double2(0.0, 0.0);
-        cd->h[tid] = h[tid];
-    }
-    if (tid == 0) { rank_total_s = 0; sweeps_s = 0; margin_s = 1e300; }
-    __syncthreads();
-    double2* beta = beta_s;
-    bool first = true;
+    __shared__ uint32_t bits[kMaxN / 32];
+    __shared__ double lam1_s, weakest_s, strongest_s;
+    int rank_total = 0, sweeps = 0;                        // the same in every thread
+    bool first = true, has_margin = false;
+#pragma unroll 1
     for (int pass = 0; pass <= 2 * s && s > 0; ++pass) {
-        if (tid == 0) {
-            int a = 0;
-            for (int j = 0; j < n; ++j)
-                if (fl_s[j]) elist[a++] = j;
-            eps_s = a;
-        }
-        __syncthreads();
-        const int eps = eps_s;
+        const int eps = __syncthreads_count(tid < n && fl_s[tid] != 0);
         const int s2 = (2 * s - eps) / 2;
         if (s2 < 1) break;
-        // lambda: one factor (x - w^v) at a time, new_k = old_{k-1} - w^v old_k
-        if (tid <= eps) lam[tid] = make_double2(tid == 0 ? 1.0 : 0.0, 0.0);
-        __syncthreads();
-        for (int a = 0; a < eps; ++a) {
-            double2 nv = make_double2(0.0, 0.0);
-            if (tid <= a + 1) {
-                const double2 wv = tw[elist[a]];
-                const double2 prev = tid > 0 ? lam[tid - 1] : make_double2(0.0, 0.0);
-                const double2 cur = tid <= a ? lam[tid] : make_double2(0.0, 0.0);
-                const double2 q = cmul(wv, cur);
-                nv = make_double2(prev.x - q.x, prev.y - q.y);
+        if (eps == 0) {                                    // T = h
+            if (tid < 2 * s) h[n - 2 * s + tid] = syn[tid];
+            if (tid == 0) lam1_s = 1.0;
+        } else {
+            // lambda: one factor (x - w^v) at a time, new_k = old_{k-1} - w^v old_k
+            list_flagged(fl_s, n, elist, bits);
+            if (eps < 32) {                                // lambda_k in lane k of the first warp
+                if (tid < 32) {
+                    double2 l = make_double2(tid == 0 ? 1.0 : 0.0, 0.0);
+#pragma unroll 1
+                    for (int a = 0; a < eps; ++a) {
+                        const double2 q = cmul(tw[elist[a]], l);
+                        const double px = __shfl_up_sync(0xffffffffu, l.x, 1), py = __shfl_up_sync(0xffffffffu, l.y, 1);
+                        l = make_double2((tid > 0 ? px : 0.0) - q.x, (tid > 0 ? py : 0.0) - q.y);
+                    }
+                    lam[tid] = l;
+                }
+            } else {
+                if (tid <= eps) lam[tid] = make_double2(tid == 0 ? 1.0 : 0.0, 0.0);
+                __syncthreads();
+#pragma unroll 1
+                for (int a = 0; a < eps; ++a) {
+                    double2 nv = make_double2(0.0, 0.0);
+                    if (tid <= a + 1) {
+                        const double2 wv = tw[elist[a]];
+                        const double2 prev = tid > 0 ? lam[tid - 1] : make_double2(0.0, 0.0);
+                        const double2 cur = tid <= a ? lam[tid] : make_double2(0.0, 0.0);
+                        const double2 q = cmul(wv, cur);
+                        nv = make_double2(prev.x - q.x, prev.y - q.y);
+                    }
+                    __syncthreads();
+                    if (tid <= a + 1) lam[tid] = nv;
+                    __syncthreads();
+                }
             }
             __syncthreads();
-            if (tid <= a + 1) lam[tid] = nv;
-            __syncthreads();
-        }
-        if (tid < 32) {
-            double acc = 0.0;
-            for (int k = tid; k <= eps; k += 32) acc += sqrt(cabs2(lam[k]));
-            acc = warp_sum(acc);
-            if (tid == 0) lam1_s = acc;
-        }
-        if (tid < n) {                                     // T_m on its window m = n - 2 s2 .. n - 1, zero before it
-            double a = 0.0, b = 0.0;
-            if (tid >= n - 2 * s2)
-                for (int k = 0; k <= eps; ++k) {
-                    const double2 q = cmul(lam[k], syn[tid - k - (n - 2 * s)]);
-                    a += q.x;
-                    b += q.y;
-                }
-            h[tid] = make_double2(a, b);
+            if (tid < n) {                                 // T_m on its window m = n - 2 s2 .. n - 1, zero before it
+                double a = 0.0, b = 0.0;
+                if (tid >= n - 2 * s2)
+#pragma unroll 1
+                    for (int k = 0; k <= eps; ++k) {
+                        const double2 q = cmul(lam[k], syn[tid - k - (n - 2 * s)]);
+                        a += q.x;
+                        b += q.y;
+                    }
+                h[tid] = make_double2(a, b);
+            } else if (tid >= kSolveThreads - 32) {
+                double acc = 0.0;
+#pragma unroll 1
+                for (int k = tid & 31; k <= eps; k += 32) acc += sqrt(cabs2(lam[k]));
+                acc = warp_sum(acc);
+                if ((tid & 31) == 0) lam1_s = acc;
+            }
         }
         __syncthreads();
         const double cut = tol * lam1_s;                   // the rounding noise of h enters T through |lambda_k|
-        int rank = 0;
-        {
-            // row i: [h_{n-s2-1-i} .. h_{n-2-i}] beta = h_{n-1-i}; stored by columns
-            const int sp = s2 + (s2 & 1);
-            const bool small = sp <= kSmallDim;
-            double2* A = small ? As : cd->work;
-            double2* V = small ? Vs : cd->work + sp * sp;
+        // row i of the system: [h_{n-s2-1-i} .. h_{n-2-i}] beta = h_{n-1-i}.  No singular value exceeds the Frobenius norm:
+        // when that is within the cutoff (the usual step without any adversary, and the usual last pass: rounding noise) the
+        // rank is 0 and nothing is solved.
+        const int sp = s2 + (s2 & 1);
+        if (sp <= kSmallDim) {
+            if (tid < 32) {
+                double fro2 = 0.0;
+                if (tid < 2 * s2 - 1) {                    // h_{n-2 s2+i} stands in the matrix once per anti-diagonal entry
+                    const int times = tid < s2 ? tid + 1 : 2 * s2 - 1 - tid;
+                    fro2 = times * cabs2(h[n - 2 * s2 + tid]);
+                }
+                fro2 = warp_sum(fro2);
+                int rank = 0, swept = 0;
+                if (fro2 > cut * cut) {
+                    const bool done = s2 <= kRegSystem && warp_full_rank_solve(As, h, n, s2, cut, fro2, beta_s);
+                    if (done) {
+                        rank = s2;
+                    } else {                               // stored by columns
+#pragma unroll 1
+                        for (int idx = tid; idx < sp * sp; idx += 32) {
+                            const int c = idx / sp, i = idx % sp;
+                            As[idx] = (c < s2 && i < s2) ? h[n - s2 - 1 - i + c] : make_double2(0.0, 0.0);
+                        }
+                        if (tid < s2) rhs_s[tid] = h[n - 1 - tid];
+                        __syncwarp();
+                        rank = warp_jacobi_pinv(As, Vs, rhs_s, s2, cut, beta_s, coef_s, sh);
+                        swept = sh[3];
+                    }
+                }
+                if (tid == 0) { rank_s = rank; sh[3] = swept; }
+            }
+            __syncthreads();
+        } else {
+            double2* A = cd->work;
+#pragma unroll 1
             for (int idx = tid; idx < sp * sp; idx += blockDim.x) {
                 const int c = idx / sp, i = idx % sp;
                 A[idx] = (c < s2 && i < s2) ? h[n - s2 - 1 - i + c] : make_double2(0.0, 0.0);
             }
             if (tid < s2) rhs_s[tid] = h[n - 1 - tid];
+            if (tid == 0) sh[3] = 0;
             __syncthreads();
-            // No singular value exceeds the Frobenius norm: when that is within the cutoff (the usual step without any
-            // adversary, and the usual last pass: rounding noise) the rank is 0 and the SVD is skipped.
             if (tid < 32) {
                 double fro2 = 0.0;
+#pragma unroll 1
                 for (int idx = tid; idx < sp * sp; idx += 32) fro2 += cabs2(A[idx]);
                 fro2 = warp_sum(fro2);
                 if (tid == 0) sh[2] = (fro2 > cut * cut) ? 1 : 0;
             }
             __syncthreads();
-            if (sh[2]) {
-                if (small) {
-                    if (tid < 32) warp_jacobi_pinv(A, V, rhs_s, s2, cut, beta_s, coef_s, sh);
-                    __syncthreads();
-                    rank = sh[1];
-                } else {
-                    rank = block_jacobi_pinv(A, V, rhs_s, s2, cut, beta_s, coef_s, sh);
-                }
-                if (tid == 0) {                            // sweeps of the longest iteration; negative once one hit the limit
-                    if (sh[3] < 0) sweeps_s = sh[3];
-                    else if (sweeps_s >= 0 && sh[3] > sweeps_s) sweeps_s = sh[3];
-                }
-            }
+            int rank = 0;
+            if (sh[2]) rank = block_jacobi_pinv(A, cd->work + sp * sp, rhs_s, s2, cut, beta_s, coef_s, sh);
+            if (tid == 0) rank_s = rank;
+            __syncthreads();
         }
+        const int rank = rank_s;
+        // sweeps of the longest iteration; negative once one hit the limit
+        if (sh[3] < 0) sweeps = sh[3];
+        else if (sweeps >= 0 && sh[3] > sweeps) sweeps = sh[3];
         if (rank == 0) break;
         if (tid == 0) {
-            for (int l = 0; l < n - 2 * s2; ++l) {
-                double a = 0.0, b = 0.0;
-                for (int u = 0; u < s2; ++u) {
-                    int idx = l + u - s2;
-                    if (idx < 0) idx += n;
-                    const double2 q = cmul(beta[u], h[idx]);
-                    a += q.x;
-                    b += q.y;
+            const int count = n - 2 * s2;
+            if (s2 <= kRegSystem) {
+#define DRACO_RECUR(S) run_recurrence<S>(h, n, count, beta_s)
+                DRACO_BY_SIZE(s2, DRACO_RECUR)
+#undef DRACO_RECUR
+            } else {
+#pragma unroll 1
+                for (int l = 0; l < count; ++l) {
+                    double a = 0.0, b = 0.0;
+#pragma unroll 1
+                    for (int u = 0; u < s2; ++u) {
+                        int idx = l + u - s2;
+                        if (idx < 0) idx += n;
+                        const double2 q = cmul(beta_s[u], h[idx]);
+                        a += q.x;
+                        b += q.y;
+                    }
+                    h[l] = make_double2(a, b);
                 }
-                h[l] = make_double2(a, b);
             }
         }
         __syncthreads();
-        if (tid < n) {
+        {
             double a = 0.0, b = 0.0;
-            int idx = 0;                                   // (tid m) mod n
-            for (int m = 0; m < n; ++m) {
-                const double2 q = cmul(h[m], tw[idx]);
-                a += q.x;
-                b += q.y;
-                idx += tid;
-                if (idx >= n) idx -= n;
+            if (node < n) {
+                int idx = mod(sub * node);                 // (node m) mod n
+                const int step = mod(per * node);
+#pragma unroll 1
+                for (int m = sub; m < n; m += per) {
+                    const double2 q = cmul(h[m], tw[idx]);
+                    a += q.x;
+                    b += q.y;
+                    idx += step;
+                    if (idx >= n) idx -= n;
+                }
             }
-            const double2 t = make_double2(a * rsn, b * rsn);
-            if (first) {
-                cd->t[tid] = t;
-                cd->h[tid] = h[tid];
-            }
-            mag[tid] = fl_s[tid] ? -1.0 : cabs2(t);        // nodes already in V are not candidates
+            a = lane_sum(a, shift);
+            b = lane_sum(b, shift);
+            // |t_j|^2; nodes already in V are not candidates
+            if (node < n && sub == 0) mag[node] = fl_s[node] ? -1.0 : cabs2(make_double2(a * rsn, b * rsn));
         }
         __syncthreads();
         // exactly `rank` entries of t are non-zero in exact arithmetic: the rank largest |t_j| join V
-        bool found = false;
-        if (tid < n) {
-            int pos = 0;
-            for (int k = 0; k < n; ++k) pos += (mag[k] > mag[tid]) || (mag[k] == mag[tid] && k < tid);
-            found = pos < rank;
-            if (first && pos == rank - 1) sorted[0] = mag[tid];     // |t|^2 of the weakest flagged node ..
-            if (first && pos == rank) sorted[1] = mag[tid];         // .. and of the strongest unflagged one
+        int pos = 0;
+        if (node < n)
+#pragma unroll 1
+            for (int k = sub; k < n; k += per) pos += (mag[k] > mag[node]) || (mag[k] == mag[node] && k < node);
+#pragma unroll 1
+        for (int off = per >> 1; off > 0; off >>= 1) pos += __shfl_xor_sync(0xffffffffu, pos, off);
+        if (node < n && sub == 0) {
+            if (first && pos == rank - 1) weakest_s = mag[node];    // |t|^2 of the weakest flagged node ..
+            if (first && pos == rank) strongest_s = mag[node];      // .. and of the strongest unflagged one
+            if (pos < rank) fl_s[node] = 1;
         }
-        __syncthreads();
-        if (found) fl_s[tid] = 1;
-        if (tid == 0) {
-            rank_total_s += rank;
-            if (first && rank < n - eps) margin_s = sqrt(sorted[0] / fmax(sorted[1], 1e-300));
-        }
+        rank_total += rank;
+        if (first) has_margin = rank < n - eps;
         first = false;
         __syncthreads();
     }
     __syncthreads();
-    bool flagged = false;
     if (tid < n) {
-        flagged = fl_s[tid] != 0;
-        if (flags) flags[tid] = flagged ? 1 : 0;
-        if (flags2) flags2[tid] = flagged ? 1 : 0;
-        if (flagged) atomicAdd(&count, 1);
+        if (flags) flags[tid] = fl_s[tid];
+        if (flags2) flags2[tid] = fl_s[tid];
     }
-    __syncthreads();
-    if (tid == 0) {
+    const int count = __syncthreads_count(tid < n && fl_s[tid] != 0);
+    if (tid == kSolveThreads - 1) {
         info->n_flagged = count;
-        info->locator_rank = rank_total_s;
-        info->scale = scale_s;
+        info->locator_rank = rank_total;
+        info->scale = scale;
         info->max_syndrome = maxsyn_s;
-        const double margin = margin_s;
+        const double margin = has_margin ? sqrt(weakest_s / fmax(strongest_s, 1e-300)) : 1e300;
         // exactly `rank` entries of t are non-zero in exact arithmetic: where the weakest flagged and the strongest
         // unflagged |t_j| of the first pass are less than a decade apart the choice of V is not to be trusted, nor is a
         // rank that comes from an iteration that was stopped at its sweep limit
-        info->status = (margin >= kMarginBar && sweeps_s >= 0) ? DRACO_OK : DRACO_EUNSURE;
+        info->status = (margin >= kMarginBar && sweeps >= 0) ? DRACO_OK : DRACO_EUNSURE;
         info->no_majority = 0;
         info->locator_margin = margin;
-        info->svd_sweeps = sweeps_s;
+        info->svd_sweeps = sweeps;
         info->im_residual_bits = 0ull;                     // a decode's self-check belongs to the locate before it
         info->re_max_bits = 0ull;
     }
     if (with_b) {                                          // the decode vector for the V just found, same launch
         __syncthreads();
-        decode_vector_body(cd, fl_s, n, s, info);
+        decode_vector_body(cd, fl_s, tw, n, s, mod, rsn, info);
     }
 }
 
@@ -1140,6 +1382,8 @@ int launch_cyc_project_finish(draco_plan* p, double2* e_out, cudaStream_t st) {
     return DRACO_OK;
 }
 
+static ModN mod_n(int n) { return ModN{(uint32_t)n, (uint32_t)(((1ull << 32) + (uint64_t)n - 1) / (uint64_t)n)}; }
+
 // e == nullptr: the record of the plan's own projection (launch_cyc_project) is formed first: by the locator kernel
 // itself when the projection left few block partials (short vectors, where every launch counts), by the reduction
 // kernel otherwise.  with_b: the decode vector for the set V just found is formed in the same launch.
@@ -1157,14 +1401,15 @@ int launch_cyc_solve(draco_plan* p, const double2* e, uint8_t* flags, bool with_
             e = own;
         }
     }
-    cyc_solve_kernel<<<1, kSolveThreads, 0, st>>>(p->cyc_dev, e, partial, used, p->project_grid, p->n, p->s, p->theta, flags,
-                                                  p->flags_dev, p->info_dev, with_b ? 1 : 0);
+    cyc_solve_kernel<<<1, kSolveThreads, 0, st>>>(p->cyc_dev, e, partial, used, p->project_grid, p->n, p->s, p->theta, mod_n(p->n),
+                                                  1.0 / sqrt((double)p->n), flags, p->flags_dev, p->info_dev, with_b ? 1 : 0);
     DRACO_CUDA(cudaGetLastError());
     return DRACO_OK;
 }
 
 int launch_cyc_decode_vector(draco_plan* p, const uint8_t* flags, cudaStream_t st) {
-    cyc_decode_vector_kernel<<<1, kSolveThreads, 0, st>>>(p->cyc_dev, flags, p->n, p->s, p->info_dev);
+    cyc_decode_vector_kernel<<<1, kSolveThreads, 0, st>>>(p->cyc_dev, flags, p->n, p->s, mod_n(p->n), 1.0 / sqrt((double)p->n),
+                                                          p->info_dev);
     DRACO_CUDA(cudaGetLastError());
     return DRACO_OK;
 }

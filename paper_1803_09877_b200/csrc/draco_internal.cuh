@@ -43,15 +43,10 @@ struct EncodePhase64 {
 // Device-resident state of the cyclic decoder (lives in the plan's scratch).
 struct CycDevice {
     double2 twiddle[kMaxN];           // w^k, w = exp(2 pi i / n)
-    double2 e[kMaxN];                 // projection f R
-    double2 h[kMaxN];                 // syndromes, then the full DFT of gamma
-    double2 t[kMaxN];                 // IDFT(h)
     double2 b[kMaxN];                 // decode vector (zero on flagged nodes)
     double2 b_active[kMaxN];          // b_j of the active rows, packed
     int32_t active[kMaxN];            // their node indices
     double2 work[kMaxN * (kMaxN + 1)];  // elimination work space
-    double2 vec[4 * kMaxN];
-    int32_t perm[kMaxN];
     double record[3 * kMaxN];         // the plan's own projection record: n (re, im) pairs, then n values q_j
 };
 
