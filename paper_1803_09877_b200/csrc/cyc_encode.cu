@@ -5,8 +5,9 @@
 // row 0 up to a unit phase: W[j][k] = w^(j M) W[0][(k - j) mod n], M = n - 2 s - 1.  Hence
 //
 //     z_j = phase[j] * sum_{t=0..2s} tap[t] * g_{(j - t) mod n},
-//     tap[t] = w^(-t M) W[0][t],   phase[j] = w^(j M):
+//     tap[t] = w^(-t M) W[0][t],   phase[j] = w^(j M)
 //
+// (with a unit factor moved from the taps to the phases that makes the centre tap real):
 // one fixed (2 s + 1)-tap complex filter run around the circle of gradients, then one unit
 // rotation per output.  The taps do not depend on j, so they sit in the kernel's constant
 // parameter bank and every multiply-add takes its coefficient from there.
@@ -26,7 +27,14 @@
 // outer taps are accumulated in fp32, smallest first; the three centre taps, the rotation
 // and the final sum run in fp64, and each output is rounded to fp32 once.  That keeps the
 // encoder at the accuracy floor of complex64 transport (2 n (2 s + 1) FMA per coordinate,
-// of which 6 n + 4 n in fp64).
+// of which 5 n + 4 n in fp64).
+//
+// Packed mode filters complex inputs: the two halves' sums are combined before the rotation, which halves its cost and the
+// conversions of the results, and up to s = 4 everything runs in fp64 (each fp32 partial sum costs a conversion of 8 cycles, a
+// fp64 multiply-add 2).  n = 45, d = 60.2 M: s = 5 5.64 -> 5.31 ms, s = 3 5.06 -> 4.34 ms, s = 4 5.44 -> 5.2 ms; n = 15, s = 2
+// 1.35 -> 1.21 ms; s = 7, d = 30 M 3.24 -> 2.98 ms; error against fp64 at s <= 4 2.7e-8 -> 2.53e-8, elsewhere unchanged.  All of
+// s = 5 in fp64 measured 5.79 ms, five fp64 taps 6.02 ms.  The real centre tap (one fp64 operation per coordinate less) took
+// the unpacked encoder from 6.29 to 6.24 ms at s = 5 and from 3.64 to 3.45 ms at s = 7, d = 30 M.
 #include "draco_internal.cuh"
 
 namespace draco {
@@ -40,10 +48,10 @@ constexpr int kGenericThreads = 256;
 // Shapes per s.  The window of the s >= 3 kernels needs 140-168 registers, which a scheduler's 16 K
 // registers allow for 3 warps: 12 warps per block, one block per SM.  The s <= 2 kernels fit in 128
 // registers and run 16 warps.
-template <int S>
+template <int S, bool PACKED>
 struct StreamCfg {
     static constexpr int R = 2 * S + 1;                            // taps
-    static constexpr int NBIG = R < 3 ? R : 3;                     // centre taps in fp64
+    static constexpr int NBIG = R < 3 || (PACKED && S <= 4) ? R : 3;   // centre taps in fp64
     static constexpr int H = (NBIG - 1) / 2;
     static constexpr int SL = ((R + NBIG - 1) / NBIG) * NBIG;      // register slots: a multiple of NBIG
     static constexpr int kThreads = S <= 2 ? 512 : 384;
@@ -74,10 +82,10 @@ __device__ __forceinline__ void sts128(uint32_t a, float4 v) {
 }
 
 // ---------------------------------------------------------------- per-thread state
-template <int S>
+template <int S, bool PACKED>
 struct Window {
-    float4 win[StreamCfg<S>::SL];                  // rows (vv - t), slot = vv mod SL
-    double cw[StreamCfg<S>::NBIG][4];              // fp64 copies of the rows under the centre taps
+    float4 win[StreamCfg<S, PACKED>::SL];                 // rows (vv - t), slot = vv mod SL
+    double cw[StreamCfg<S, PACKED>::NBIG][4];              // fp64 copies of the rows under the centre taps
 };
 
 // The fetch side: the rows of this warp's strips, one after the other, kRing rows ahead of the row being
@@ -127,11 +135,11 @@ struct Cursor {
 // MODE 0: first SL steps of a strip (all rows from the ring; outputs from step 2 S on);
 // MODE 1: steady state (ring row + output);  MODE 2: anything (run-time guards).
 template <int S, int P, int MODE, bool PACKED>
-__device__ __forceinline__ void encode_step(Window<S>& w, Cursor& cur, Fetcher<PACKED>& f, int vv, int n, int64_t ldz,
+__device__ __forceinline__ void encode_step(Window<S, PACKED>& w, Cursor& cur, Fetcher<PACKED>& f, int vv, int n, int64_t ldz,
                                             uint32_t stash0, float2* zcol, bool act0, bool act1,
                                             const EncodeTaps& taps, const EncodeTaps64& taps64,
                                             const EncodePhase64& ph64) {
-    using Cfg = StreamCfg<S>;
+    using Cfg = StreamCfg<S, PACKED>;
     constexpr int R = Cfg::R, NBIG = Cfg::NBIG, H = Cfg::H, SL = Cfg::SL;
     constexpr uint32_t kRowBytes = Cfg::kRowBytes;
     const int total = n + 2 * S;
@@ -171,20 +179,48 @@ __device__ __forceinline__ void encode_step(Window<S>& w, Cursor& cur, Fetcher<P
             ar[2] = fmaf(cr, g.z, ar[2]); ai[2] = fmaf(ci, g.z, ai[2]);
             ar[3] = fmaf(cr, g.w, ar[3]); ai[3] = fmaf(ci, g.w, ai[3]);
         }
-        double dr[4], di[4];
+        constexpr int NOUT = PACKED ? 2 : 4;             // complex outputs of this thread
+        double dr[NOUT], di[NOUT];
+        if constexpr (PACKED) {
+            // components 0, 1 of a row are the real parts of two complex coordinates, 2, 3 their imaginary parts
 #pragma unroll
-        for (int c = 0; c < 4; ++c) { dr[c] = (double)ar[c]; di[c] = (double)ai[c]; }
+            for (int c = 0; c < 2; ++c) {
+                dr[c] = S > H ? (double)ar[c] - (double)ai[c + 2] : 0.0;
+                di[c] = S > H ? (double)ai[c] + (double)ar[c + 2] : 0.0;
+            }
 #pragma unroll
-        for (int t = S - H; t <= S + H; ++t) {
-            const int q = ((P - t + 2 * SL) % SL) % NBIG;
-            const double cr = taps64.tap[t].x, ci = taps64.tap[t].y;
+            for (int k = 0; k < NBIG; ++k) {
+                const int t = (k & 1) ? S + H - (k >> 1) : S - H + (k >> 1);
+                const double cr = taps64.tap[t].x, ci = taps64.tap[t].y;
+                const double(&g)[4] = w.cw[((P - t + 2 * SL) % SL) % NBIG];
 #pragma unroll
-            for (int c = 0; c < 4; ++c) { dr[c] = fma(cr, w.cw[q][c], dr[c]); di[c] = fma(ci, w.cw[q][c], di[c]); }
+                for (int c = 0; c < 2; ++c) {
+                    dr[c] = fma(cr, g[c], dr[c]);
+                    di[c] = fma(cr, g[c + 2], di[c]);
+                    if (t != S) {                        // the centre tap is real
+                        dr[c] = fma(-ci, g[c + 2], dr[c]);
+                        di[c] = fma(ci, g[c], di[c]);
+                    }
+                }
+            }
+        } else {
+#pragma unroll
+            for (int c = 0; c < 4; ++c) { dr[c] = (double)ar[c]; di[c] = (double)ai[c]; }
+#pragma unroll
+            for (int t = S - H; t <= S + H; ++t) {
+                const int q = ((P - t + 2 * SL) % SL) % NBIG;
+                const double cr = taps64.tap[t].x, ci = taps64.tap[t].y;
+#pragma unroll
+                for (int c = 0; c < 4; ++c) {
+                    dr[c] = fma(cr, w.cw[q][c], dr[c]);
+                    if (t != S) di[c] = fma(ci, w.cw[q][c], di[c]);
+                }
+            }
         }
         const double2 rot = ph64.phase[j];
-        double xr[4], xi[4];
+        double xr[NOUT], xi[NOUT];
 #pragma unroll
-        for (int c = 0; c < 4; ++c) {
+        for (int c = 0; c < NOUT; ++c) {
             xr[c] = fma(dr[c], rot.x, -di[c] * rot.y);
             xi[c] = fma(dr[c], rot.y, di[c] * rot.x);
         }
@@ -195,11 +231,8 @@ __device__ __forceinline__ void encode_step(Window<S>& w, Cursor& cur, Fetcher<P
             dst = cur.zout;
             cur.zout += ldz;
         }
-        if (PACKED) {
-            // components 0,1 filtered the real parts (X), 2,3 the imaginary parts (Y): z = X + i Y
-            if (act0)
-                __stcs(reinterpret_cast<float4*>(dst), make_float4((float)(xr[0] - xi[2]), (float)(xi[0] + xr[2]),
-                                                                   (float)(xr[1] - xi[3]), (float)(xi[1] + xr[3])));
+        if constexpr (PACKED) {
+            if (act0) __stcs(reinterpret_cast<float4*>(dst), make_float4((float)xr[0], (float)xi[0], (float)xr[1], (float)xi[1]));
         } else {
             // A lane's two 16-byte stores are 512 bytes apart, so that each store instruction of the warp
             // covers 512 contiguous bytes (whole 32-byte sectors).  With the 4 coordinates of a lane adjacent,
@@ -219,11 +252,11 @@ __device__ __forceinline__ void encode_step(Window<S>& w, Cursor& cur, Fetcher<P
 }
 
 template <int S, int MODE, bool PACKED, int P = 0>
-__device__ __forceinline__ void encode_chunk(Window<S>& w, Cursor& cur, Fetcher<PACKED>& f, int v0, int n, int64_t ldz,
+__device__ __forceinline__ void encode_chunk(Window<S, PACKED>& w, Cursor& cur, Fetcher<PACKED>& f, int v0, int n, int64_t ldz,
                                              uint32_t stash0, float2* zcol, bool act0, bool act1,
                                              const EncodeTaps& taps, const EncodeTaps64& taps64,
                                              const EncodePhase64& ph64) {
-    if constexpr (P < StreamCfg<S>::SL) {
+    if constexpr (P < StreamCfg<S, PACKED>::SL) {
         encode_step<S, P, MODE, PACKED>(w, cur, f, v0 + P, n, ldz, stash0, zcol, act0, act1, taps, taps64, ph64);
         encode_chunk<S, MODE, PACKED, P + 1>(w, cur, f, v0, n, ldz, stash0, zcol, act0, act1, taps, taps64, ph64);
     }
@@ -233,12 +266,12 @@ __device__ __forceinline__ void encode_chunk(Window<S>& w, Cursor& cur, Fetcher<
 // coordinates, a strip holds 64 of them, and a lane receives two pairs of each row:
 // G[r][c], G[r][c + 1] (real parts) and G[r][half + c], G[r][half + c + 1] (imaginary parts).
 template <int S, bool PACKED>
-__global__ void __launch_bounds__(StreamCfg<S>::kThreads, 1)
+__global__ void __launch_bounds__(StreamCfg<S, PACKED>::kThreads, 1)
 cyc_encode_stream_kernel(const float* __restrict__ G, float2* __restrict__ Z, int64_t len, int64_t ldg, int64_t ldz,
                          int64_t half, int n,
                          const __grid_constant__ EncodeTaps taps, const __grid_constant__ EncodeTaps64 taps64,
                          const __grid_constant__ EncodePhase64 ph64) {
-    using Cfg = StreamCfg<S>;
+    using Cfg = StreamCfg<S, PACKED>;
     constexpr int SL = Cfg::SL, kWarps = Cfg::kThreads / 32;
     constexpr int kStrip = PACKED ? 64 : 128;
     extern __shared__ __align__(16) unsigned char smem_raw[];        // ring[kRing][kThreads], stash[2 S][kThreads], 16 bytes each
@@ -255,7 +288,7 @@ cyc_encode_stream_kernel(const float* __restrict__ G, float2* __restrict__ Z, in
     f.open_strip();
 #pragma unroll 1
     for (int q = 0; q < kRing; ++q) f.fetch(cur.ring0 + q * Cfg::kRowBytes);
-    Window<S> w;
+    Window<S, PACKED> w;
 #pragma unroll
     for (int q = 0; q < SL; ++q) w.win[q] = make_float4(0.f, 0.f, 0.f, 0.f);
     const int total = n + 2 * S;
@@ -349,10 +382,10 @@ __device__ __forceinline__ void fir_step(FirState<S, PACKED>& w, int vv, int n, 
 #pragma unroll
         for (int c = 0; c < C; ++c) {
             ar[c] = fma(cr, x[c], ar[c]);
-            ai[c] = fma(ci, x[c], ai[c]);
+            if (t != S) ai[c] = fma(ci, x[c], ai[c]);              // the centre tap is real
         }
         if constexpr (PACKED) {
-            ar[0] = fma(-ci, x[1], ar[0]);
+            if (t != S) ar[0] = fma(-ci, x[1], ar[0]);
             ai[0] = fma(cr, x[1], ai[0]);
         }
     }
@@ -462,7 +495,7 @@ cyc_encode_generic_kernel(const float* __restrict__ G, float2* __restrict__ Z, i
 template <int S, bool PACKED>
 int launch_stream(const draco_plan* p, const float* G, float2* Z, int64_t len, int64_t ldg, int64_t ldz, int64_t half,
                   cudaStream_t st) {
-    using Cfg = StreamCfg<S>;
+    using Cfg = StreamCfg<S, PACKED>;
     constexpr int kThreads = Cfg::kThreads;
     auto kern = cyc_encode_stream_kernel<S, PACKED>;
     static bool configured[64] = {};
@@ -538,8 +571,9 @@ int launch_cyc_encode(const draco_plan* p, const float* G, float2* Z, int64_t le
     // are multiples of 4 floats
     const bool packed = half > 0;
     bool fast = (ldg % 4 == 0) && (ldz % 2 == 0) && p->s <= 7;
-    if (packed) fast = fast && (len % 4 == 0) && (half % 4 == 0) && (half + len <= d_real);
-    else fast = fast && (len % 4 == 0);
+    // (and, for a column chunk of a longer vector, what the whole vector's call would need: all of it goes the same way)
+    if (packed) fast = fast && (len % 4 == 0) && (half % 4 == 0) && (half + len <= d_real) && (ldz % 4 == 0) && (p->d % 2 == 0);
+    else fast = fast && (len % 4 == 0) && (ldz % 4 == 0);
     if (fast) return packed ? launch_stream_any<true>(p, G, Z, len, ldg, ldz, half, st)
                             : launch_stream_any<false>(p, G, Z, len, ldg, ldz, 0, st);
     if (p->s >= 1 && p->s <= 7)                            // the register window's sizes

@@ -82,11 +82,14 @@ int build_cyclic_tables(draco_plan* p, std::vector<double2>* taps_full, std::vec
         }
     }
     taps_full->resize(2 * s + 1);
+    // a unit factor common to all taps is moved to the phases so that the centre tap, the largest, is real
+    const cld centre = root_of_unity(n, -(long long)s * M) * w0[s];
+    const cld unit = centre / std::abs(centre);
     memset(&p->taps, 0, sizeof(p->taps));
     memset(&p->taps64, 0, sizeof(p->taps64));
     memset(&p->phase64, 0, sizeof(p->phase64));
     for (int t = 0; t <= 2 * s; ++t) {
-        const cld v = root_of_unity(n, -(long long)t * M) * w0[t];
+        const cld v = t == s ? cld(std::abs(centre), 0.0L) : root_of_unity(n, -(long long)t * M) * w0[t] / unit;
         (*taps_full)[t] = make_double2((double)v.real(), (double)v.imag());
         if (t < kMaxTaps) {
             p->taps.tap[t] = make_float2((float)v.real(), (float)v.imag());
@@ -97,7 +100,7 @@ int build_cyclic_tables(draco_plan* p, std::vector<double2>* taps_full, std::vec
     twiddle->resize(kMaxN);
     for (int j = 0; j < kMaxN; ++j) (*twiddle)[j] = make_double2(0.0, 0.0);
     for (int j = 0; j < n; ++j) {
-        const cld ph = root_of_unity(n, (long long)j * M);
+        const cld ph = root_of_unity(n, (long long)j * M) * unit;
         p->phase.phase[j] = make_float2((float)ph.real(), (float)ph.imag());
         p->phase64.phase[j] = make_double2((double)ph.real(), (double)ph.imag());
         const cld tw = root_of_unity(n, j);
