@@ -236,10 +236,10 @@ class ClockSampler:
 def stage_launches(code, n, n_adv):
     """Kernels launched per step: encode 1; corrupt 1 (all adversaries in one launch); cyclic locate = projection
     (two launches over half the rows each when n > 64) + reduction of the block partials fused with the solve;
-    decode = decode vector + recovery (repetition: vote + finish, no separate locate)."""
+    decode = decode vector + recovery (repetition: the vote alone, no separate locate)."""
     cyc = code in ("cyc", "cycp")
     return {"encode": 1, "corrupt": 1 if n_adv else 0, "locate": ((2 if n > 64 else 1) + LOCATE_TAIL_LAUNCHES) if cyc else 0,
-            "decode": 2}
+            "decode": 2 if cyc else 1}
 
 
 LOCATE_TAIL_LAUNCHES = 2     # cyc_reduce_partials_kernel, cyc_solve_kernel
