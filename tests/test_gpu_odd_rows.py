@@ -78,10 +78,10 @@ def test_repetition_rows_off_the_grid(n, s, d):
 
 
 # the few-rows projection takes 512 coordinates per warp and splits the rows of short vectors over blocks, the tile kernel 512 or
-# (from 32,769 coordinates on) 2048 per block; the recovery takes 512 per block
+# (from 32,769 coordinates on) 2048 per block; the recovery takes 64 per block up to 640 per SM, then 512
 DECODE = [(code, n, s, d) for code in ("CYC", "CYC_PACKED")
           for n, s, d in [(5, 1, 1), (15, 2, 511), (15, 2, 513), (16, 3, 4097), (15, 2, 8200), (17, 2, 513), (45, 5, 2047),
-                          (45, 5, 4100), (45, 5, 32_767), (45, 5, 32_770), (45, 5, 65_539), (70, 2, 1025), (105, 2, 33_001)]]
+                          (45, 5, 4100), (45, 5, 32_767), (45, 5, 32_770), (45, 5, 65_539), (70, 2, 1025), (105, 2, 33_001), (15, 2, 94_720), (15, 2, 94_722), (15, 2, 95_003), (15, 2, 189_447)]]
 
 
 @pytest.mark.parametrize("code,n,s,d", DECODE)
@@ -116,3 +116,49 @@ def test_projection_and_recovery_at_the_edges_of_their_tiles(code, n, s, d):
     plan.decode_update(Rd, flags, w, 0.5)
     np.testing.assert_array_equal(host(w)[:d], np.float32(1.0) - np.float32(0.5) * host(u)[:d])
     assert (host(w)[d:] == 1.0).all()
+
+
+@pytest.mark.parametrize("code", ["REP", "CYC"])
+@pytest.mark.parametrize("d", [1, 2, 3, 4, 5, 7, 1021, 4099])
+def test_adversary_rows_of_any_alignment(code, d):
+    """The values before a row's first 16-byte boundary and after its last whole 16 bytes: same bits as the generator's."""
+    import paper_1803_09877_b200 as dr
+    n = 9
+    plan = dr.Plan(n, 1, d, getattr(dr, code))
+    R = di.gradient_rows(31 + d, n, d if code == "REP" else 2 * d)
+    if code == "CYC":
+        R = np.ascontiguousarray(R).view(np.complex64)
+    models, params = [di.ADV_REVGRAD, di.ADV_CONST, di.ADV_GAUSS] * 3, [100.0, 1e4, 1e3] * 3
+    Rd = dev(R)
+    plan.corrupt(Rd, list(range(n)), models, params, seed=17)
+    want = di.apply_adversaries(R.copy(), list(range(n)), models, params, seed=17)
+    got = host(Rd, complex64=code == "CYC")
+    np.testing.assert_array_equal(np.ascontiguousarray(got).view(np.uint32), np.ascontiguousarray(want).view(np.uint32))
+
+
+@pytest.mark.parametrize("code", ["REP", "CYC", "CYC_PACKED"])
+@pytest.mark.parametrize("d", [39_999, 40_000, 40_002, 65_536])
+def test_host_pipeline_with_a_split_last_chunk(code, d):
+    """More than 2 MB of G: the call copies it in two pieces, and gives the bits of the device-resident path."""
+    import paper_1803_09877_b200 as dr
+    n, s = 15, 2
+    cyc, v = code != "REP", (d + 1) // 2 if code == "CYC_PACKED" else d
+    plan = dr.Plan(n, s, d, getattr(dr, code))
+    G = di.gradient_rows(63 + d, n, d)
+    f = di.projection_vector(64 + d, v)
+    adv = di.choose_adversaries(65 + d, n, s)
+    model, param = [di.ADV_REVGRAD] * s, [100.0] * s
+    Z = torch.empty((n, 2 * v if cyc else v), dtype=torch.float32, device="cuda")
+    Zh = torch.empty_like(Z)
+    plan.encode(dev(G), Z)
+    plan.corrupt(Z, adv, model, param, seed=5)
+    flags = torch.empty(n, dtype=torch.uint8, device="cuda")
+    u = torch.empty(d, dtype=torch.float32, device="cuda")
+    plan.locate_decode(Z, dev(f) if cyc else None, flags, u)
+    torch.cuda.synchronize()
+    Gh, fh = torch.from_numpy(G).pin_memory(), torch.from_numpy(f).pin_memory()
+    uh, flh = torch.empty(d).pin_memory(), torch.empty(n, dtype=torch.uint8).pin_memory()
+    info = plan.pipeline_host(Gh, fh if cyc else None, adv, model, param, 5, Zh, uh, flh)
+    assert torch.equal(Zh, Z) and torch.equal(flh, flags.cpu())
+    assert sorted(np.flatnonzero(flh.numpy())) == adv.tolist() and info["n_flagged"] == s
+    assert np.abs(uh.numpy() - host(u)).max() <= 2.0 ** -22 * np.abs(host(u)).max()      # e sums in another order: b to 1e-12
