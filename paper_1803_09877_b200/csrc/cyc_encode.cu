@@ -271,6 +271,7 @@ cyc_encode_stream_kernel(const float* __restrict__ G, float2* __restrict__ Z, in
                          int64_t half, int n,
                          const __grid_constant__ EncodeTaps taps, const __grid_constant__ EncodeTaps64 taps64,
                          const __grid_constant__ EncodePhase64 ph64) {
+    pdl_begin();
     using Cfg = StreamCfg<S, PACKED>;
     constexpr int SL = Cfg::SL, kWarps = Cfg::kThreads / 32;
     constexpr int kStrip = PACKED ? 64 : 128;
@@ -416,6 +417,7 @@ __global__ void __launch_bounds__(FirCfg<S, PACKED>::kThreads, FirCfg<S, PACKED>
 cyc_encode_fir_kernel(const float* __restrict__ G, float2* __restrict__ Z, int64_t len, int64_t ldg, int64_t ldz,
                       int64_t half, int64_t d_real, int n, const __grid_constant__ EncodeTaps64 taps,
                       const __grid_constant__ EncodePhase64 ph) {
+    pdl_begin();
     using Cfg = FirCfg<S, PACKED>;
     constexpr int R = Cfg::R, C = Cfg::C, kT = Cfg::kThreads, kTile = Cfg::kTile, kAlign = Cfg::kAlign;
     __shared__ float stash_all[2 * S * Cfg::NI * kT];
@@ -466,6 +468,7 @@ __global__ void __launch_bounds__(kGenericThreads)
 cyc_encode_generic_kernel(const float* __restrict__ G, float2* __restrict__ Z, int64_t len, int64_t ldg, int64_t ldz,
                           int64_t half, int64_t d_real, int n, int s, const double2* __restrict__ taps,
                           const __grid_constant__ EncodePhase64 ph) {
+    pdl_begin();
     const int64_t stride = (int64_t)gridDim.x * kGenericThreads;
     for (int64_t i = (int64_t)blockIdx.x * kGenericThreads + threadIdx.x; i < len; i += stride) {
         const bool has_b = half > 0 && half + i < d_real;
@@ -514,7 +517,7 @@ int launch_stream(const draco_plan* p, const float* G, float2* Z, int64_t len, i
     int64_t grid = (int64_t)p->sm_count * per_sm;
     if (grid > nblocks) grid = nblocks;
     if (grid < 1) grid = 1;
-    kern<<<(int)grid, kThreads, Cfg::kSmem, st>>>(G, Z, len, ldg, ldz, half, p->n, p->taps, p->taps64, p->phase64);
+    launch_dependent(kern, (int)grid, kThreads, Cfg::kSmem, st, G, Z, len, ldg, ldz, half, p->n, p->taps, p->taps64, p->phase64);
     DRACO_CUDA(cudaGetLastError());
     return DRACO_OK;
 }
@@ -541,8 +544,8 @@ int launch_fir(const draco_plan* p, const float* G, float2* Z, int64_t len, int6
     const int64_t nstrips = (len + Cfg::kTile - 1) / Cfg::kTile;
     int64_t grid = (int64_t)p->sm_count * Cfg::kBlocks;
     if (grid > nstrips) grid = nstrips;
-    cyc_encode_fir_kernel<S, PACKED><<<(int)grid, Cfg::kThreads, 0, st>>>(G, Z, len, ldg, ldz, half, d_real, p->n, p->taps64,
-                                                                          p->phase64);
+    launch_dependent(cyc_encode_fir_kernel<S, PACKED>, (int)grid, Cfg::kThreads, 0, st, G, Z, len, ldg, ldz, half, d_real,
+                     p->n, p->taps64, p->phase64);
     DRACO_CUDA(cudaGetLastError());
     return DRACO_OK;
 }
@@ -583,8 +586,8 @@ int launch_cyc_encode(const draco_plan* p, const float* G, float2* Z, int64_t le
     const int64_t cap = (int64_t)p->sm_count * 16;
     if (want > cap) want = cap;
     if (want < 1) want = 1;
-    cyc_encode_generic_kernel<<<(int)want, kGenericThreads, 0, st>>>(G, Z, len, ldg, ldz, half, d_real, p->n, p->s,
-                                                                     p->taps_full_dev, p->phase64);
+    launch_dependent(cyc_encode_generic_kernel, (int)want, kGenericThreads, 0, st, G, Z, len, ldg, ldz, half, d_real, p->n,
+                     p->s, p->taps_full_dev, p->phase64);
     DRACO_CUDA(cudaGetLastError());
     return DRACO_OK;
 }

@@ -72,6 +72,7 @@ template <int RPW, bool VEC2, int TILE>
 __global__ void __launch_bounds__(kThreads, 4)
 cyc_project_kernel(const float2* __restrict__ R, const float* __restrict__ f, int64_t len, int64_t ld, int n,
                    int row0, int nrows, double2* __restrict__ partial, int cap, int accumulate) {
+    pdl_begin();
     __shared__ __align__(16) double fs[TILE];
     // Running sums of row warp + r * 8 over this block's tiles, kept by lane 0 of the row's warp: after every tile
     // the warp adds its lanes' sums up (fixed butterfly order) and lane 0 adds the result here.  Keeping them in
@@ -189,6 +190,7 @@ template <bool VEC2, bool SPLIT>
 __global__ void __launch_bounds__(kThreads, 3)
 cyc_project_fewrows_kernel(const float2* __restrict__ R, const float* __restrict__ f, int64_t len, int64_t ld, int n,
                            double2* __restrict__ partial, int cap, int accumulate) {
+    pdl_begin();
     constexpr int CH = kProjectChunk;
     __shared__ double2 es[kProjectWarps][kFewRows];
     __shared__ double qs[kProjectWarps][kFewRows];
@@ -289,6 +291,7 @@ cyc_project_fewrows_kernel(const float2* __restrict__ R, const float* __restrict
 constexpr int kReduceThreads = 128;
 __global__ void __launch_bounds__(kReduceThreads)
 cyc_reduce_partials_kernel(const double2* __restrict__ partial, int grid, int cap, int n, double* __restrict__ record) {
+    pdl_begin();
     constexpr int kBatch = 8;
     __shared__ double wsum[3][kReduceThreads / 32];
     const int j = blockIdx.x, tid = threadIdx.x;
@@ -924,6 +927,7 @@ __device__ void decode_vector_body(CycDevice* cd, const uint8_t* fl, const doubl
 __global__ void __launch_bounds__(kSolveThreads)
 cyc_decode_vector_kernel(CycDevice* cd, const uint8_t* __restrict__ flags, int n, int s, ModN mod, double rsn,
                          DeviceInfo* info) {
+    pdl_begin();
     __shared__ double2 tw[kMaxN];
     __shared__ uint8_t fl[kMaxN];
     const int tid = threadIdx.x;
@@ -953,7 +957,8 @@ cyc_solve_kernel(CycDevice* cd, const double2* __restrict__ e_in, const double2*
     // lanes of one node, for the sums over the nodes
     const int shift = lanes_shift(n), per = 1 << shift, node = tid >> shift, sub = tid & (per - 1);
 
-    if (tid < n) tw[tid] = cd->twiddle[tid];
+    if (tid < n) tw[tid] = cd->twiddle[tid];              // written when the plan was made: no need to wait
+    pdl_begin();
     if (e_in != nullptr) {                                 // the projection record: n (re, im) pairs, then n values q_j
         if (tid < n) {
             e[tid] = e_in[tid];
@@ -1311,7 +1316,7 @@ static cudaError_t launch_project_kernels(int cap, const ProjectShape& shape, cu
     const int grid = shape.grid, tile = shape.tile;
     if (n <= kFewRows) {
         const dim3 grid2(grid, shape.gridy);
-#define DRACO_FEW(VV, SS) cyc_project_fewrows_kernel<VV, SS><<<grid2, kThreads, 0, st>>>(R, f, len, ld, n, partial, cap, accumulate)
+#define DRACO_FEW(VV, SS) launch_dependent(cyc_project_fewrows_kernel<VV, SS>, grid2, kThreads, 0, st, R, f, len, ld, n, partial, cap, accumulate)
         if (shape.gridy > 1) {
             if (vec2) DRACO_FEW(true, true); else DRACO_FEW(false, true);
         } else {
@@ -1332,7 +1337,7 @@ static cudaError_t launch_project_kernels(int cap, const ProjectShape& shape, cu
     }
     const dim3 grid2(grid, ysplit);
 #define DRACO_PROJECT(RR, VV, TT) \
-    cyc_project_kernel<RR, VV, TT><<<grid2, kThreads, 0, st>>>(R, f, len, ld, n, row0, nrows, partial, cap, accumulate)
+    launch_dependent(cyc_project_kernel<RR, VV, TT>, grid2, kThreads, 0, st, R, f, len, ld, n, row0, nrows, partial, cap, accumulate)
 #define DRACO_PROJECT_TILE(RR, VV)                                           \
     do {                                                                     \
         if (tile == kProjectTile) DRACO_PROJECT(RR, VV, kProjectTile);       \
@@ -1376,8 +1381,8 @@ int launch_cyc_project(draco_plan* p, const float2* R, const float* f, int64_t l
 }
 
 int launch_cyc_project_finish(draco_plan* p, double2* e_out, cudaStream_t st) {
-    cyc_reduce_partials_kernel<<<p->n, kReduceThreads, 0, st>>>(p->partial_dev, p->project_used, p->project_grid, p->n,
-                                                                reinterpret_cast<double*>(e_out));
+    launch_dependent(cyc_reduce_partials_kernel, p->n, kReduceThreads, 0, st, p->partial_dev, p->project_used,
+                     p->project_grid, p->n, reinterpret_cast<double*>(e_out));
     DRACO_CUDA(cudaGetLastError());
     return DRACO_OK;
 }
@@ -1401,15 +1406,15 @@ int launch_cyc_solve(draco_plan* p, const double2* e, uint8_t* flags, bool with_
             e = own;
         }
     }
-    cyc_solve_kernel<<<1, kSolveThreads, 0, st>>>(p->cyc_dev, e, partial, used, p->project_grid, p->n, p->s, p->theta, mod_n(p->n),
-                                                  1.0 / sqrt((double)p->n), flags, p->flags_dev, p->info_dev, with_b ? 1 : 0);
+    launch_dependent(cyc_solve_kernel, 1, kSolveThreads, 0, st, p->cyc_dev, e, partial, used, p->project_grid, p->n, p->s,
+                     p->theta, mod_n(p->n), 1.0 / sqrt((double)p->n), flags, p->flags_dev, p->info_dev, with_b ? 1 : 0);
     DRACO_CUDA(cudaGetLastError());
     return DRACO_OK;
 }
 
 int launch_cyc_decode_vector(draco_plan* p, const uint8_t* flags, cudaStream_t st) {
-    cyc_decode_vector_kernel<<<1, kSolveThreads, 0, st>>>(p->cyc_dev, flags, p->n, p->s, mod_n(p->n), 1.0 / sqrt((double)p->n),
-                                                          p->info_dev);
+    launch_dependent(cyc_decode_vector_kernel, 1, kSolveThreads, 0, st, p->cyc_dev, flags, p->n, p->s, mod_n(p->n),
+                     1.0 / sqrt((double)p->n), p->info_dev);
     DRACO_CUDA(cudaGetLastError());
     return DRACO_OK;
 }
@@ -1471,7 +1476,7 @@ extern "C" int draco_cyc_project_noalloc(int n, int64_t d, const void* R, const 
     // to be cleared between calls even though the array keeps the previous call's contents.
     const ProjectShape shape = project_shape(grid, sms, d, n);
     DRACO_CUDA(launch_project_kernels(grid, shape, st, Rc, f, d, d, n, partial, 0));
-    cyc_reduce_partials_kernel<<<n, kReduceThreads, 0, st>>>(partial, shape.grid, grid, n, e);
+    launch_dependent(cyc_reduce_partials_kernel, n, kReduceThreads, 0, st, partial, shape.grid, grid, n, e);
     DRACO_CUDA(cudaGetLastError());
     return DRACO_OK;
 }

@@ -30,6 +30,7 @@ template <bool VEC2, bool PACKED>
 __global__ void __launch_bounds__(kThreads)
 cyc_recover_kernel(const float2* __restrict__ R, int64_t len, int64_t ld, const CycDevice* __restrict__ cd,
                    DeviceInfo* info, float* __restrict__ u, int64_t d_packed, float* __restrict__ w, float scale) {
+    pdl_begin();
     __shared__ double2 bs[kMaxN];
     __shared__ int rows[kMaxN];
     const int count = info->n_active;
@@ -150,6 +151,7 @@ template <bool VEC2, bool PACKED>
 __global__ void __launch_bounds__(kThreads)
 cyc_recover_short_kernel(const float2* __restrict__ R, int64_t len, int64_t ld, const CycDevice* __restrict__ cd,
                          DeviceInfo* info, float* __restrict__ u, int64_t d_packed, float* __restrict__ w, float scale) {
+    pdl_begin();
     constexpr int kWarps = kThreads / 32;
     __shared__ double sums[kWarps][4][32];                // a0, a1, i0, i1 of every lane
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -229,9 +231,9 @@ int launch_cyc_recover(draco_plan* p, const float2* R, int64_t len, int64_t ld, 
     if (want > cap) want = cap;
     if (want < 1) want = 1;
 #define DRACO_REC(V2, PK) \
-    cyc_recover_kernel<V2, PK><<<(int)want, kThreads, 0, st>>>(R, len, ld, p->cyc_dev, p->info_dev, u, d_packed, w, scale)
+    launch_dependent(cyc_recover_kernel<V2, PK>, (int)want, kThreads, 0, st, R, len, ld, p->cyc_dev, p->info_dev, u, d_packed, w, scale)
 #define DRACO_REC_SHORT(V2, PK)                                                                                                    \
-    cyc_recover_short_kernel<V2, PK><<<(int)((len + 63) / 64), kThreads, 0, st>>>(R, len, ld, p->cyc_dev, p->info_dev, u, d_packed, w, \
+    launch_dependent(cyc_recover_short_kernel<V2, PK>, (int)((len + 63) / 64), kThreads, 0, st, R, len, ld, p->cyc_dev, p->info_dev, u, d_packed, w, \
                                                                                   scale)
     if (len <= (int64_t)p->sm_count * kShortCoordinates) {
         if (vec2) {

@@ -47,6 +47,7 @@ __device__ __forceinline__ uint64_t normal_state(uint64_t key, uint64_t i) { ret
 __global__ void __launch_bounds__(kThreads)
 generate_kernel(float* __restrict__ out, int rows, int64_t len, int64_t ld, int64_t i0, int row0, float mean, float sd,
                 uint64_t seed, float inv_sigma) {
+    pdl_begin();
     const int64_t stride = (int64_t)gridDim.x * kThreads;
     for (int r = 0; r < rows; ++r) {
         const uint64_t key = splitmix64_at(seed, (uint64_t)(row0 + r));
@@ -79,6 +80,7 @@ struct CorruptTable {
 __global__ void __launch_bounds__(kThreads)
 corrupt_kernel(float* __restrict__ R, int64_t row_pitch, int64_t nvals, int64_t v0, int is_complex, float inv_sigma,
                const __grid_constant__ CorruptTable tab) {
+    pdl_begin();
     const int a = blockIdx.y;
     const int model = tab.model[a];
     const float param = tab.param[a];
@@ -137,8 +139,8 @@ int device_sm_count() {                     // of the current device; looked up 
 
 int launch_generate(float* out, int rows, int64_t len, int64_t ld, int64_t i0, int row0, float mean, float sd,
                     uint64_t seed, cudaStream_t st) {
-    generate_kernel<<<grid_for(len, device_sm_count(), 16), kThreads, 0, st>>>(out, rows, len, ld, i0, row0, mean, sd, seed,
-                                                                              inv_sigma_f32());
+    launch_dependent(generate_kernel, grid_for(len, device_sm_count(), 16), kThreads, 0, st, out, rows, len, ld, i0, row0,
+                     mean, sd, seed, inv_sigma_f32());
     DRACO_CUDA(cudaGetLastError());
     return DRACO_OK;
 }
@@ -158,7 +160,7 @@ int launch_corrupt(float* R, int64_t row_pitch, int64_t nvals, int64_t v0, const
     int per_sm = 16 / n_adv;
     if (per_sm < 2) per_sm = 2;
     const dim3 grid(grid_for((nvals + 3) / 4, sm_count, per_sm), n_adv);
-    corrupt_kernel<<<grid, kThreads, 0, st>>>(R, row_pitch, nvals, v0, is_complex ? 1 : 0, inv_sigma_f32(), tab);
+    launch_dependent(corrupt_kernel, grid, kThreads, 0, st, R, row_pitch, nvals, v0, is_complex ? 1 : 0, inv_sigma_f32(), tab);
     DRACO_CUDA(cudaGetLastError());
     return DRACO_OK;
 }

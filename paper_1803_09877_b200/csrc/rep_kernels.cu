@@ -85,6 +85,7 @@ template <int MMAX, bool ADJ, int GB>
 __global__ void __launch_bounds__(kThreads)
 rep_encode_kernel(const float* __restrict__ G, float* __restrict__ Z, int64_t len, int64_t ldg, int64_t ldz,
                   GroupTable gt) {
+    pdl_begin();
     const uint32_t* Gb = reinterpret_cast<const uint32_t*>(G);
     const int span = 4 * (int)blockDim.x, tile = ADJ ? span : span - kSector;
     const int64_t ntiles = (len + tile - 1) / tile;
@@ -272,6 +273,7 @@ __global__ void __launch_bounds__(TPB)
 rep_vote_kernel(const uint32_t* __restrict__ R, int64_t len, int64_t ld, GroupTable gt, float* __restrict__ u,
                 float* __restrict__ maj, RepScratch* scratch, float* __restrict__ w, float scale, uint8_t* flags, uint8_t* flags2,
                 DeviceInfo* info) {
+    pdl_begin();
     __shared__ uint32_t smask[kMaxN][MMAX > 0 ? 1 : 4];   // generic path: up to 128 members = 4 words
     for (int i = threadIdx.x; i < kMaxN * (MMAX > 0 ? 1 : 4); i += blockDim.x) (&smask[0][0])[i] = 0;
     __syncthreads();
@@ -411,7 +413,7 @@ int launch_rep_encode(const draco_plan* p, const float* G, float* Z, int64_t len
     const int64_t quads = (len + 3) / 4;
     const int threads = block_for(quads, p->sm_count, kThreads);
     const int grid = grid_for(quads, threads, (int64_t)p->sm_count * 8 * (kThreads / threads));
-#define DRACO_ENC(MM, AA, GG) rep_encode_kernel<MM, AA, GG><<<grid, threads, 0, st>>>(G, Z, len, ldg, ldz, gt)
+#define DRACO_ENC(MM, AA, GG) launch_dependent(rep_encode_kernel<MM, AA, GG>, grid, threads, 0, st, G, Z, len, ldg, ldz, gt)
 #define DRACO_ENC_BY_SIZE(AA)                                      \
     do {                                                           \
         if (gt.max_size <= 3) DRACO_ENC(3, AA, 5);                 \
@@ -443,7 +445,7 @@ int launch_rep_vote(draco_plan* p, const float* R, int64_t len, int64_t ld, floa
         static const int per_sm = resident_blocks(rep_vote_kernel<MM, AA, GG, TT>, TT);                           \
         const int threads = block_for(quads, p->sm_count, TT);                                                    \
         const int grid = grid_for(quads, threads, p->sm_count * per_sm * (TT / threads));                         \
-        rep_vote_kernel<MM, AA, GG, TT><<<grid, threads, 0, st>>>(Rb, len, ld, gt, u, maj, scratch, w, scale, flags,  \
+        launch_dependent(rep_vote_kernel<MM, AA, GG, TT>, grid, threads, 0, st, Rb, len, ld, gt, u, maj, scratch, w, scale, flags,  \
                                                                   p->flags_dev, p->info_dev);                      \
     } while (0)
 #define DRACO_VOTE_BY_SIZE(AA)                                                                                    \
