@@ -97,10 +97,26 @@ def _ptr(x):
     return x.data_ptr()
 
 
+def _find_current_stream():
+    """torch.cuda.current_stream().cuda_stream, without the Stream object that it builds on every call where torch offers the
+    handle itself: 0.2 us instead of 3.3 us of the 8.1 us that a call of this module took (a launch is 3.9 us of it)."""
+    global _current_stream
+    import torch
+    first = torch.cuda.current_stream().cuda_stream        # also sets CUDA up
+    raw, device = getattr(torch._C, "_cuda_getCurrentRawStream", None), getattr(torch._C, "_cuda_getDevice", None)
+    if raw and device:
+        _current_stream = lambda: raw(device())
+    else:
+        _current_stream = lambda: torch.cuda.current_stream().cuda_stream
+    return first
+
+
+_current_stream = _find_current_stream
+
+
 def _stream(stream):
     if stream is None:
-        import torch
-        return torch.cuda.current_stream().cuda_stream
+        return _current_stream()
     if isinstance(stream, int):
         return stream
     return stream.cuda_stream
