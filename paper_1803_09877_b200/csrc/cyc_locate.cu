@@ -430,13 +430,14 @@ __device__ __forceinline__ void jacobi_rotation(double alpha, double bet, double
     st = make_double2(gr * k, gi * k);
 }
 
-// one column pair, rows i0, i0 + step, ..: (x, y) <- (c x - conj(st) y, st x + c y)
+// (xo, yo) = (c x - conj(st) y, st x + c y)
+__device__ __forceinline__ void rotate(double2 x, double2 y, double c, double2 st, double2& xo, double2& yo) {
+    xo = make_double2(c * x.x - (st.x * y.x + st.y * y.y), c * x.y - (st.x * y.y - st.y * y.x));
+    yo = make_double2(st.x * x.x - st.y * x.y + c * y.x, st.x * x.y + st.y * x.x + c * y.y);
+}
+// one column pair, rows i0, i0 + step, ..
 __device__ __forceinline__ void rotate_pair(double2* xp, double2* yp, int i0, int step, int rows, double c, double2 st) {
-    for (int i = i0; i < rows; i += step) {
-        const double2 x = xp[i], y = yp[i];
-        xp[i] = make_double2(c * x.x - (st.x * y.x + st.y * y.y), c * x.y - (st.x * y.y - st.y * y.x));
-        yp[i] = make_double2(st.x * x.x - st.y * x.y + c * y.x, st.x * x.y + st.y * x.x + c * y.y);
-    }
+    for (int i = i0; i < rows; i += step) rotate(xp[i], yp[i], c, st, xp[i], yp[i]);
 }
 
 // ------------------------------------------------------------------ small SVD solve
@@ -539,10 +540,6 @@ __device__ int warp_jacobi_pinv(double2* A, double2* V, const double2* rhs, int 
     const unsigned full = 0xffffffffu;
     const int lane = threadIdx.x & 31;
     const int sp = s + (s & 1), npairs = sp / 2;
-    int lp = 1;
-    while (lp * 2 * npairs <= 32) lp *= 2;
-    const int pair = lane / lp, sub = lane % lp;
-    const bool act = pair < npairs;
     for (int idx = lane; idx < sp * sp; idx += 32) {
         const int c = idx / sp, i = idx % sp;
         V[idx] = make_double2(c == i ? 1.0 : 0.0, 0.0);
@@ -550,52 +547,99 @@ __device__ int warp_jacobi_pinv(double2* A, double2* V, const double2* rhs, int 
     __syncwarp();
     int sweeps = 0;
     bool converged = false;
-    for (int sweep = 0; sweep < kJacobiSweepLimit; ++sweep) {
-        bool rotated = false;
-        for (int step = 0; step < sp - 1; ++step) {
-            int p = 0, q = 1;
-            if (act) {
-                int a, b;
-                if (pair == 0) { a = sp - 1; b = step; }
-                else {                                    // (step +- pair) mod (sp - 1); both are below sp - 1
-                    a = step + pair;
-                    if (a >= sp - 1) a -= sp - 1;
-                    b = step - pair;
-                    if (b < 0) b += sp - 1;
-                }
-                p = a < b ? a : b;
-                q = a < b ? b : a;
-            }
-            double2* ap = A + p * sp;
-            double2* aq = A + q * sp;
-            double alpha = 0.0, bet = 0.0, gr = 0.0, gi = 0.0;
-            if (act)
-                for (int i = sub; i < s; i += lp) {
-                    const double2 x = ap[i], y = aq[i];
-                    alpha += x.x * x.x + x.y * x.y;
-                    bet += y.x * y.x + y.y * y.y;
-                    gr += x.x * y.x + x.y * y.y;          // conj(x) * y
-                    gi += x.x * y.y - x.y * y.x;
-                }
-            for (int off = lp >> 1; off > 0; off >>= 1) {
-                alpha += __shfl_xor_sync(full, alpha, off);
-                bet += __shfl_xor_sync(full, bet, off);
-                gr += __shfl_xor_sync(full, gr, off);
-                gi += __shfl_xor_sync(full, gi, off);
-            }
-            const double g2 = gr * gr + gi * gi;
-            if (act && g2 > 1e-30 * alpha * bet && g2 > 0.0) {
-                double c;
-                double2 st;
-                jacobi_rotation(alpha, bet, gr, gi, g2, c, st);
-                rotate_pair(ap, aq, sub, lp, s, c, st);
-                rotate_pair(V + p * sp, V + q * sp, sub, lp, sp, c, st);
-                rotated = true;
-            }
-            __syncwarp();
+    // the columns of a pair at a step
+    auto columns = [&](int pair, int step, int& p, int& q) {
+        int a, b;
+        if (pair == 0) { a = sp - 1; b = step; }
+        else {                                            // (step +- pair) mod (sp - 1); both are below sp - 1
+            a = step + pair;
+            if (a >= sp - 1) a -= sp - 1;
+            b = step - pair;
+            if (b < 0) b += sp - 1;
         }
-        ++sweeps;
-        if (!__any_sync(full, rotated)) { converged = true; break; }
+        p = a < b ? a : b;
+        q = a < b ? b : a;
+    };
+    if (sp <= 8) {
+        // Eight lanes per pair, a row of A and of V per lane: everything of a step sits in registers between one round of loads
+        // and one of stores.  s = 5: an iteration of about 35 steps takes 12 us instead of 18 with loops over the rows.
+        const int pair = lane >> 3, sub = lane & 7;
+        const bool act = pair < npairs, ra = act && sub < s, rv = act && sub < sp;
+#pragma unroll 1
+        for (int sweep = 0; sweep < kJacobiSweepLimit; ++sweep) {
+            bool rotated = false;
+#pragma unroll 1
+            for (int step = 0; step < sp - 1; ++step) {
+                int p = 0, q = 1;
+                if (act) columns(pair, step, p, q);
+                double2* const at[4] = {A + p * sp + sub, A + q * sp + sub, V + p * sp + sub, V + q * sp + sub};
+                const double2 zero = make_double2(0.0, 0.0);
+                const double2 x = ra ? *at[0] : zero, y = ra ? *at[1] : zero;
+                const double2 vx = rv ? *at[2] : zero, vy = rv ? *at[3] : zero;
+                double alpha = x.x * x.x + x.y * x.y, bet = y.x * y.x + y.y * y.y;
+                double gr = x.x * y.x + x.y * y.y, gi = x.x * y.y - x.y * y.x;      // conj(x) * y
+#pragma unroll
+                for (int off = 4; off > 0; off >>= 1) {
+                    alpha += __shfl_xor_sync(full, alpha, off);
+                    bet += __shfl_xor_sync(full, bet, off);
+                    gr += __shfl_xor_sync(full, gr, off);
+                    gi += __shfl_xor_sync(full, gi, off);
+                }
+                const double g2 = gr * gr + gi * gi;
+                if (act && g2 > 1e-30 * alpha * bet && g2 > 0.0) {
+                    double c;
+                    double2 st;
+                    jacobi_rotation(alpha, bet, gr, gi, g2, c, st);
+                    if (ra) rotate(x, y, c, st, *at[0], *at[1]);
+                    if (rv) rotate(vx, vy, c, st, *at[2], *at[3]);
+                    rotated = true;
+                }
+                __syncwarp();
+            }
+            ++sweeps;
+            if (!__any_sync(full, rotated)) { converged = true; break; }
+        }
+    } else {
+        int lp = 1;
+        while (lp * 2 * npairs <= 32) lp *= 2;
+        const int pair = lane / lp, sub = lane % lp;
+        const bool act = pair < npairs;
+        for (int sweep = 0; sweep < kJacobiSweepLimit; ++sweep) {
+            bool rotated = false;
+            for (int step = 0; step < sp - 1; ++step) {
+                int p = 0, q = 1;
+                if (act) columns(pair, step, p, q);
+                double2* ap = A + p * sp;
+                double2* aq = A + q * sp;
+                double alpha = 0.0, bet = 0.0, gr = 0.0, gi = 0.0;
+                if (act)
+                    for (int i = sub; i < s; i += lp) {
+                        const double2 x = ap[i], y = aq[i];
+                        alpha += x.x * x.x + x.y * x.y;
+                        bet += y.x * y.x + y.y * y.y;
+                        gr += x.x * y.x + x.y * y.y;          // conj(x) * y
+                        gi += x.x * y.y - x.y * y.x;
+                    }
+                for (int off = lp >> 1; off > 0; off >>= 1) {
+                    alpha += __shfl_xor_sync(full, alpha, off);
+                    bet += __shfl_xor_sync(full, bet, off);
+                    gr += __shfl_xor_sync(full, gr, off);
+                    gi += __shfl_xor_sync(full, gi, off);
+                }
+                const double g2 = gr * gr + gi * gi;
+                if (act && g2 > 1e-30 * alpha * bet && g2 > 0.0) {
+                    double c;
+                    double2 st;
+                    jacobi_rotation(alpha, bet, gr, gi, g2, c, st);
+                    rotate_pair(ap, aq, sub, lp, s, c, st);
+                    rotate_pair(V + p * sp, V + q * sp, sub, lp, sp, c, st);
+                    rotated = true;
+                }
+                __syncwarp();
+            }
+            ++sweeps;
+            if (!__any_sync(full, rotated)) { converged = true; break; }
+        }
     }
     bool keep = false;
     if (lane < sp) {
