@@ -1328,8 +1328,11 @@ int project_grid_size(int sm_count) { return sm_count * 4; }
 
 // Blocks along x of a projection, cap at most, each leaving one partial per node: no more than have work, so that short
 // vectors leave a handful of partials.  n <= 16: a chunk per warp; as many blocks as are resident at once (three per SM) with
-// the chunks dealt out evenly.  Otherwise a tile per block; short vectors take smaller tiles, whose warps are through after one
-// round of loads (d = 4096, n = 45: four rounds one after the other with the full tile).
+// the chunks dealt out evenly.  Otherwise a tile per block.  Short vectors take smaller tiles, whose warps are through after one
+// round of loads (d = 4096, n = 45: four rounds one after the other with the full tile), and so do those whose full tiles
+// would not occupy the device twice over, once the locator kernel would not add their few partials up itself (n = 45,
+// reduction included: d = 200 k 42 -> 26 us, 600 k 65 -> 50 us; n = 105, d = 100 k 42 -> 34 us; but 1 M, where small tiles are
+// four rounds of blocks, 62 -> 69 us, and n = 45, d = 60 k, where they cost the reduction a kernel, 32 -> 37 us with the decode).
 struct ProjectShape {
     int grid, gridy, tile;
 };
@@ -1346,8 +1349,12 @@ static ProjectShape project_shape(int cap, int sm_count, int64_t len, int n) {
         if (g.gridy < 1) g.gridy = 1;
         return g;
     }
-    if (len <= (int64_t)kProjectTileShort * 64) g.tile = kProjectTileShort;
-    const int64_t work = (len + g.tile - 1) / g.tile;
+    int64_t work = (len + kProjectTile - 1) / kProjectTile;
+    const int64_t work_short = (len + kProjectTileShort - 1) / kProjectTileShort;
+    if (work_short <= 64 || (3 * n * work > kFusedReduceMax && work_short <= 2 * (int64_t)cap)) {
+        g.tile = kProjectTileShort;
+        work = work_short;
+    }
     g.grid = (int)(work < cap ? work : cap);
     return g;
 }
