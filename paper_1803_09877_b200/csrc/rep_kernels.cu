@@ -175,11 +175,16 @@ struct RepScratch {
 
 // mask words -> flag bytes and the info block, by the block that comes last, which leaves the scratch cleared for the next
 // call on the plan: a memset before and a one-block kernel after the vote were two thirds of a short vote's time
-// (n = 15, s = 2, d = 100,000: 11.3 - 12.8 us with them, 7.6 - 8.2 without).
+// (n = 15, s = 2, d = 100,000: 11.3 - 12.8 us with them, 7.6 - 8.2 without;
+// 7.15 against 7.43 us a call with one thread's fence instead of every thread's and the two exchanges under way together).
 __device__ __forceinline__ void finish_vote(const GroupTable& gt, RepScratch* scratch, uint8_t* flags, uint8_t* flags2,
                                             DeviceInfo* info) {
     __shared__ int count;
-    if (threadIdx.x == 0) count = 0;
+    unsigned long long no_majority = 0;
+    if (threadIdx.x == 0) {
+        count = 0;
+        no_majority = atomicExch(&scratch->no_majority, 0ull);     // under way while the masks are fetched
+    }
     __syncthreads();
     for (int g = threadIdx.x; g < gt.num_groups; g += blockDim.x) {
         const int first = gt.first[g], m = gt.size[g];
@@ -196,7 +201,6 @@ __device__ __forceinline__ void finish_vote(const GroupTable& gt, RepScratch* sc
     }
     __syncthreads();
     if (threadIdx.x == 0) {
-        const unsigned long long no_majority = atomicExch(&scratch->no_majority, 0ull);
         info->n_flagged = count;
         info->no_majority = no_majority;
         info->status = no_majority ? DRACO_ENOMAJ : DRACO_OK;
@@ -375,9 +379,11 @@ rep_vote_kernel(const uint32_t* __restrict__ R, int64_t len, int64_t ld, GroupTa
                 if (smask[g][w]) atomicOr(&scratch->mask[gt.first[g] + w], smask[g][w]);
     }
     __shared__ bool last;
-    __threadfence();
     __syncthreads();
-    if (threadIdx.x == 0) last = atomicInc(&scratch->done, gridDim.x - 1) == gridDim.x - 1;     // wraps to 0
+    if (threadIdx.x == 0) {
+        __threadfence();                       // the block's parts come before its count: the barrier, then one thread's fence
+        last = atomicInc(&scratch->done, gridDim.x - 1) == gridDim.x - 1;     // wraps to 0
+    }
     __syncthreads();
     if (last) {
         __threadfence();
