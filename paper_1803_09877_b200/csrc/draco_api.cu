@@ -175,6 +175,8 @@ int draco_plan_create(int n, int s, int64_t d, int code, draco_plan** out) {
     if (code == DRACO_REP) {
         DRACO_TRY(cudaMalloc(&p->mask_dev, rep_scratch_bytes()));
         DRACO_TRY(cudaMemset(p->mask_dev, 0, rep_scratch_bytes()));
+        // every vote relies on the cleared scratch, also on streams that do not wait for the default one
+        DRACO_TRY(cudaStreamSynchronize(nullptr));
     } else {
         DRACO_TRY(cudaMalloc(&p->cyc_dev, sizeof(CycDevice)));
         DRACO_TRY(cudaMemset(p->cyc_dev, 0, sizeof(CycDevice)));
@@ -188,8 +190,6 @@ int draco_plan_create(int n, int s, int64_t d, int code, draco_plan** out) {
         DRACO_TRY(cudaMalloc(&p->partial_dev, partial_bytes));
         DRACO_TRY(cudaMemset(p->partial_dev, 0, partial_bytes));
     }
-    // the calls that use the plan may come on streams that do not wait for the default one
-    DRACO_TRY(cudaStreamSynchronize(nullptr));
 #undef DRACO_TRY
     *out = p;
     return DRACO_OK;
