@@ -175,8 +175,6 @@ int draco_plan_create(int n, int s, int64_t d, int code, draco_plan** out) {
     if (code == DRACO_REP) {
         DRACO_TRY(cudaMalloc(&p->mask_dev, rep_scratch_bytes()));
         DRACO_TRY(cudaMemset(p->mask_dev, 0, rep_scratch_bytes()));
-        // every vote relies on the cleared scratch, also on streams that do not wait for the default one
-        DRACO_TRY(cudaStreamSynchronize(nullptr));
     } else {
         DRACO_TRY(cudaMalloc(&p->cyc_dev, sizeof(CycDevice)));
         DRACO_TRY(cudaMemset(p->cyc_dev, 0, sizeof(CycDevice)));
@@ -186,10 +184,12 @@ int draco_plan_create(int n, int s, int64_t d, int code, draco_plan** out) {
                              cudaMemcpyHostToDevice));
         p->project_grid = project_grid_size(p->sm_count);
         // per block and node: a double2 partial of e_j, then (after all of those) a double partial of q_j
+        // (not cleared: a projection writes every partial that is read after it)
         const size_t partial_bytes = (sizeof(double2) + sizeof(double)) * (size_t)p->project_grid * n;
         DRACO_TRY(cudaMalloc(&p->partial_dev, partial_bytes));
-        DRACO_TRY(cudaMemset(p->partial_dev, 0, partial_bytes));
     }
+    // The clears and the last uploads may still be under way on the default stream, which the caller's streams need not wait for.
+    DRACO_TRY(cudaStreamSynchronize(nullptr));
 #undef DRACO_TRY
     *out = p;
     return DRACO_OK;
