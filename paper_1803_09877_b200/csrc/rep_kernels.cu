@@ -77,51 +77,29 @@ struct Columns {
 
 // ---------------------------------------------------------------- encode
 // MMAX > 0: groups of at most MMAX members, GB groups fetched together so that about 16 rows are in flight per
-// thread whatever the group size (as in the vote kernel); MMAX == 0: larger groups, members streamed.
+// thread whatever the group size (as in the vote kernel); MMAX == 0: larger groups, members streamed, eight at a time.
+// Groups do not depend on one another: where the columns alone give few blocks, gridDim.y blocks share the groups of a column
+// range.  A thread that walks all of them is a chain of latencies (n = 45, s = 3, d = 100,000: 15.6 us so, 4.7 us shared; with
+// rows off the grid, d = 100,003, 19.1 and 8.9; streamed groups, n = 42, s = 10, d = 100,003, 41 and 10.7).
 // Rows off the 16-byte grid (ADJ false): a block reads kSector columns more than it writes and writes of each row the run that
-// starts on a 32-byte sector, so that no sector is shared between blocks (a shared one may go to memory half filled).
+// starts on a 32-byte sector, so that no sector is shared between blocks (a shared one may go to memory half filled).  Aligned
+// rows keep a loop of their own: in the other's the loads of a batch are issued a few at a time (n = 15, s = 2, d = 30 M 617 us,
+// 586 so; n = 45, s = 5 1789 and 1763).
 constexpr int kSector = 8;                              // fp32 values
+constexpr int kStreamBatch = 8;
 template <int MMAX, bool ADJ, int GB>
 __global__ void __launch_bounds__(kThreads)
 rep_encode_kernel(const float* __restrict__ G, float* __restrict__ Z, int64_t len, int64_t ldg, int64_t ldz,
                   GroupTable gt) {
-    pdl_begin();
+    // Streamed groups let the kernel after them be set up only at their end (n = 42, s = 10, d = 30,000,001: 3107 us with the
+    // others' early start, 2823 so; d = 100,000: 9.1 and 7.2).
+    if constexpr (MMAX > 0) pdl_begin();
+    else cudaGridDependencySynchronize();
     const uint32_t* Gb = reinterpret_cast<const uint32_t*>(G);
-    const int span = 4 * (int)blockDim.x, tile = ADJ ? span : span - kSector;
-    const int64_t ntiles = (len + tile - 1) / tile;
-    for (int64_t t = blockIdx.x; t < ntiles; t += gridDim.x) {
-        const int64_t c0 = t * tile;
-        const int64_t first_col = c0 + (ADJ ? 4 : 1) * (int)threadIdx.x;
-        if (first_col >= len) continue;
-        Columns<ADJ> cols;
-        cols.open(first_col, len);
-        uint32_t mask = 0;                              // byte c, bit k: column c is written in rows whose run starts k columns in
-        int shift0 = 0;
-        if constexpr (!ADJ) {
-            shift0 = (int)(-((int64_t)(reinterpret_cast<uintptr_t>(Z) >> 2) + c0)) & (kSector - 1);
-#pragma unroll
-            for (int c = 0; c < 4; ++c) {
-                const int i = (int)threadIdx.x + c * (int)blockDim.x;
-#pragma unroll
-                for (int k = 0; k < kSector; ++k)
-                    if (cols.has(c) && (i >= k || t == 0) && i < k + tile) mask |= 1u << (c * kSector + k);
-            }
-        }
-        auto emit = [&](int row, const float(&acc)[4]) {
-            float* z = Z + (int64_t)row * ldz;
-            if constexpr (ADJ) {
-                cols.store(z, acc);
-            } else {
-                const uint32_t m = mask >> ((shift0 - (int)((row * ldz) & (kSector - 1))) & (kSector - 1));
-                z += cols.col;
-                if (m & 1u) __stcs(z, acc[0]);
-                if (m & 0x100u) __stcs(z + cols.o1, acc[1]);
-                if (m & 0x10000u) __stcs(z + cols.o2, acc[2]);
-                if (m & 0x1000000u) __stcs(z + cols.o3, acc[3]);
-            }
-        };
+    // this block's groups, for the columns of one thread; emit(row, sums) writes them to one row
+    auto encode_columns = [&](const Columns<ADJ>& cols, auto emit) {
         if constexpr (MMAX > 0) {
-            for (int g0 = 0; g0 < gt.num_groups; g0 += GB) {
+            for (int g0 = (int)blockIdx.y * GB; g0 < gt.num_groups; g0 += GB * (int)gridDim.y) {
                 Pack val[GB][MMAX];
 #pragma unroll
                 for (int b = 0; b < GB; ++b)
@@ -148,22 +126,64 @@ rep_encode_kernel(const float* __restrict__ G, float* __restrict__ Z, int64_t le
                     }
             }
         } else {
-            for (int g = 0; g < gt.num_groups; ++g) {
+            for (int g = (int)blockIdx.y; g < gt.num_groups; g += (int)gridDim.y) {
                 const int first = gt.first[g], m = gt.size[g];
                 float acc[4];
-                Pack x;
-                cols.load(x, Gb + (int64_t)first * ldg);
+                for (int k0 = 0; k0 < m; k0 += kStreamBatch) {
+                    Pack x[kStreamBatch];
 #pragma unroll
-                for (int c = 0; c < 4; ++c) acc[c] = __uint_as_float(x.get(c));
-                for (int k = 1; k < m; ++k) {
-                    cols.load(x, Gb + (int64_t)(first + k) * ldg);
+                    for (int q = 0; q < kStreamBatch; ++q)
+                        if (k0 + q < m) cols.load(x[q], Gb + (int64_t)(first + k0 + q) * ldg);
 #pragma unroll
-                    for (int c = 0; c < 4; ++c) acc[c] = __fadd_rn(acc[c], __uint_as_float(x.get(c)));
+                    for (int q = 0; q < kStreamBatch; ++q)
+                        if (k0 + q < m) {
+#pragma unroll
+                            for (int c = 0; c < 4; ++c) {
+                                const float v = __uint_as_float(x[q].get(c));
+                                acc[c] = k0 + q == 0 ? v : __fadd_rn(acc[c], v);
+                            }
+                        }
                 }
                 for (int k = 0; k < m; ++k) emit(first + k, acc);
             }
         }
+    };
+    if constexpr (ADJ) {
+        const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+        for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < len / 4; v += stride) {
+            Columns<ADJ> cols;
+            cols.open(4 * v, len);
+            encode_columns(cols, [&](int row, const float(&acc)[4]) { cols.store(Z + (int64_t)row * ldz, acc); });
+        }
+    } else {
+        const int tile = 4 * (int)blockDim.x - kSector;
+        const int64_t ntiles = (len + tile - 1) / tile;
+        for (int64_t t = blockIdx.x; t < ntiles; t += gridDim.x) {
+            const int64_t c0 = t * tile;
+            const int64_t first_col = c0 + threadIdx.x;
+            if (first_col >= len) continue;
+            Columns<ADJ> cols;
+            cols.open(first_col, len);
+            uint32_t mask = 0;                          // byte c, bit k: column c is written in rows whose run starts k columns in
+            const int shift0 = (int)(-((int64_t)(reinterpret_cast<uintptr_t>(Z) >> 2) + c0)) & (kSector - 1);
+#pragma unroll
+            for (int c = 0; c < 4; ++c) {
+                const int i = (int)threadIdx.x + c * (int)blockDim.x;
+#pragma unroll
+                for (int k = 0; k < kSector; ++k)
+                    if (cols.has(c) && (i >= k || t == 0) && i < k + tile) mask |= 1u << (c * kSector + k);
+            }
+            encode_columns(cols, [&](int row, const float(&acc)[4]) {
+                const uint32_t m = mask >> ((shift0 - (int)((row * ldz) & (kSector - 1))) & (kSector - 1));
+                float* z = Z + (int64_t)row * ldz + cols.col;
+                if (m & 1u) __stcs(z, acc[0]);
+                if (m & 0x100u) __stcs(z + cols.o1, acc[1]);
+                if (m & 0x10000u) __stcs(z + cols.o2, acc[2]);
+                if (m & 0x1000000u) __stcs(z + cols.o3, acc[3]);
+            });
+        }
     }
+    if constexpr (MMAX == 0) cudaTriggerProgrammaticLaunchCompletion();
 }
 
 // ---------------------------------------------------------------- vote
@@ -417,9 +437,15 @@ int launch_rep_encode(const draco_plan* p, const float* G, float* Z, int64_t len
     const GroupTable& gt = p->groups;
     const bool adj = (len % 4 == 0) && (ldg % 4 == 0) && (ldz % 4 == 0);
     const int64_t quads = (len + 3) / 4;
-    const int threads = block_for(quads, p->sm_count, kThreads);
-    const int grid = grid_for(quads, threads, (int64_t)p->sm_count * 8 * (kThreads / threads));
-#define DRACO_ENC(MM, AA, GG) launch_dependent(rep_encode_kernel<MM, AA, GG>, grid, threads, 0, st, G, Z, len, ldg, ldz, gt)
+    const int grid = grid_for(quads, kThreads, (int64_t)p->sm_count * 8);
+    // blocks that share the groups of a column range: as many as make sixteen blocks per SM (aligned rows) or eight.  More for
+    // the others costs where the shares are unequal: n = 15, s = 2, d = 1,000,003, two shares of three groups, 21.9 -> 24.4 us.
+    const int64_t room = (int64_t)p->sm_count * (adj ? 16 : 8) / grid;
+    auto blocks = [&](int gb) {
+        const int64_t steps = (gt.num_groups + gb - 1) / gb, share = room < steps ? room : steps;
+        return dim3(grid, share < 1 ? 1 : (unsigned)share);
+    };
+#define DRACO_ENC(MM, AA, GG) launch_dependent(rep_encode_kernel<MM, AA, GG>, blocks(GG), kThreads, 0, st, G, Z, len, ldg, ldz, gt)
 #define DRACO_ENC_BY_SIZE(AA)                                      \
     do {                                                           \
         if (gt.max_size <= 3) DRACO_ENC(3, AA, 5);                 \

@@ -46,6 +46,24 @@ def test_encode_parity(n, s, d):
             np.testing.assert_array_equal(Zg[j].view(np.uint32), Zg[first].view(np.uint32))
 
 
+# blocks that share a column range's groups: one group each, several (uneven shares, last ones short), none to share; groups of
+# more than 16 members are streamed eight at a time (17 = 8 + 8 + 1, 21, 64 = 8 * 8)
+@pytest.mark.parametrize("n,s", [(7, 1), (45, 1), (128, 1), (15, 2), (45, 3), (45, 5), (17, 8), (42, 10), (128, 31)])
+@pytest.mark.parametrize("d", [4, 1021, 1024, 30_004, 30_007])
+def test_encode_bits_with_groups_shared_between_blocks(n, s, d):
+    dr, plan = _plan(n, s, d)
+    G = di.gradient_rows(0xE0 + n + d, n, d)
+    buf = torch.full((n * d + 64,), 7.0, dtype=torch.float32, device="cuda")
+    plan.encode(dev(G), buf[32:])
+    out = host(buf)
+    assert (out[:32] == 7.0).all() and (out[32 + n * d:] == 7.0).all()
+    Z = out[32:32 + n * d].reshape(n, d)
+    for first, size in orc.rep_groups(n, s):
+        want = fp32_sequential_sum(G[first:first + size])
+        for j in range(first, first + size):
+            np.testing.assert_array_equal(Z[j].view(np.uint32), want.view(np.uint32))
+
+
 def _received(n, s, d, seed, n_adv, models=None):
     G = di.gradient_rows(seed, n, d)
     R = orc.rep_encode(G, n, s)
