@@ -245,6 +245,23 @@ __device__ __forceinline__ void vote_step(uint32_t x, uint32_t& ma, int& counter
 template <int MMAX>
 __device__ __forceinline__ void vote_group(const Pack (&val)[MMAX], int m, uint32_t in, uint32_t (&sel)[4], uint32_t& dis,
                                            unsigned int& nomaj) {
+    // Small groups: nearly all of them agree bit for bit, which is cheaper to see than to count (n = 45, s = 1, d = 60.2 M 1843
+    // -> 1675 us, rows off the 16-byte grid, 11.7 M + 1, 383 -> 348; from six members on the count below is as cheap, n = 45,
+    // s = 5, 60.2 M 1691 us without and 1912 with this).
+    if constexpr (MMAX <= 5) {
+        uint32_t differ = 0;
+#pragma unroll
+        for (int k = 1; k < MMAX; ++k)
+            if (k < m) {
+#pragma unroll
+                for (int c = 0; c < 4; ++c) differ |= val[k].get(c) ^ val[0].get(c);
+            }
+        if (differ == 0) {
+#pragma unroll
+            for (int c = 0; c < 4; ++c) sel[c] = val[0].get(c);
+            return;
+        }
+    }
     // A value held by strictly more than half of the group IS what Algorithm 2 returns.  So count first the members that equal
     // member 0 in all four columns (five logic operations each), then those that equal member 1 (member 0 may be the
     // adversary); only if neither has a strict majority is the streaming vote itself run, column by column.  Counting column by
@@ -303,12 +320,7 @@ rep_vote_kernel(const uint32_t* __restrict__ R, int64_t len, int64_t ld, GroupTa
     __syncthreads();
 
     unsigned int nomaj = 0;
-    const int64_t tile = 4 * (int64_t)blockDim.x;
-    for (int64_t c0 = blockIdx.x * tile; c0 < len; c0 += gridDim.x * tile) {
-        const int64_t first_col = c0 + (ADJ ? 4 : 1) * (int)threadIdx.x;
-        if (first_col >= len) continue;
-        Columns<ADJ> cols;
-        cols.open(first_col, len);
+    auto vote_columns = [&](const Columns<ADJ>& cols) {
         float acc[4];
 #pragma unroll
         for (int c = 0; c < 4; ++c) acc[c] = 0.0f;
@@ -342,33 +354,49 @@ rep_vote_kernel(const uint32_t* __restrict__ R, int64_t len, int64_t ld, GroupTa
                     }
             }
         } else {
+            // Off the 16-byte grid eight members' loads at a time (n = 42, s = 10, d = 100,003: 29.5 us one by one, 21.0 so; n = 128,
+            // s = 31, 1 M + 3: 320 and 242); aligned rows four, left to the compiler: with eight the second pass finds fewer of them
+            // cached (n = 42, s = 10, 11.7 M: 561 us, 682 with batches of eight).
+            constexpr int kBatch = ADJ ? 1 : kStreamBatch;
             for (int g = 0; g < gt.num_groups; ++g) {
                 const int first = gt.first[g], m = gt.size[g];
                 const uint32_t* base = R + (int64_t)first * ld;
                 uint32_t ma[4];
-                int counter[4];
-                Pack x;
-                cols.load(x, base);
+                int counter[4], votes[4];
 #pragma unroll
-                for (int c = 0; c < 4; ++c) { ma[c] = x.get(c); counter[c] = 0; }
-                for (int k = 0; k < m; ++k) {
-                    cols.load(x, base + (int64_t)k * ld);
+                for (int c = 0; c < 4; ++c) { ma[c] = 0u; counter[c] = 0; votes[c] = 0; }
+#pragma unroll (ADJ ? 4 : 1)
+                for (int k0 = 0; k0 < m; k0 += kBatch) {
+                    Pack x[kBatch];
 #pragma unroll
-                    for (int c = 0; c < 4; ++c) vote_step(x.get(c), ma[c], counter[c]);
+                    for (int q = 0; q < kBatch; ++q)
+                        if (k0 + q < m) cols.load(x[q], base + (int64_t)(k0 + q) * ld);
+#pragma unroll
+                    for (int q = 0; q < kBatch; ++q)
+                        if (k0 + q < m) {
+#pragma unroll
+                            for (int c = 0; c < 4; ++c) vote_step(x[q].get(c), ma[c], counter[c]);
+                        }
                 }
-                int votes[4];
+#pragma unroll (ADJ ? 4 : 1)
+                for (int k0 = 0; k0 < m; k0 += kBatch) {
+                    Pack x[kBatch];
 #pragma unroll
-                for (int c = 0; c < 4; ++c) votes[c] = 0;
-                for (int k = 0; k < m; ++k) {
-                    cols.load(x, base + (int64_t)k * ld);
-                    bool any_diff = false;
+                    for (int q = 0; q < kBatch; ++q)
+                        if (k0 + q < m) cols.load(x[q], base + (int64_t)(k0 + q) * ld);
 #pragma unroll
-                    for (int c = 0; c < 4; ++c) {
-                        const bool same = x.get(c) == ma[c];
-                        votes[c] += same;
-                        any_diff |= !same;
-                    }
-                    if (any_diff && !(smask[g][k >> 5] & (1u << (k & 31)))) atomicOr(&smask[g][k >> 5], 1u << (k & 31));
+                    for (int q = 0; q < kBatch; ++q)
+                        if (k0 + q < m) {
+                            const int k = k0 + q;
+                            bool any_diff = false;
+#pragma unroll
+                            for (int c = 0; c < 4; ++c) {
+                                const bool same = x[q].get(c) == ma[c];
+                                votes[c] += same;
+                                any_diff |= !same;
+                            }
+                            if (any_diff && !(smask[g][k >> 5] & (1u << (k & 31)))) atomicOr(&smask[g][k >> 5], 1u << (k & 31));
+                        }
                 }
                 float selv[4];
 #pragma unroll
@@ -382,6 +410,25 @@ rep_vote_kernel(const uint32_t* __restrict__ R, int64_t len, int64_t ld, GroupTa
         }
         if (u != nullptr) cols.store(u, acc);
         if (w != nullptr) cols.update(w, acc, scale);
+    };
+    // Aligned rows, groups of up to eight: a loop without the block's tiles, whose loads the compiler issues together (n = 15,
+    // s = 1, d = 4 M 52.8 -> 45.5 us); from nine on the loop over tiles is as good or better (n = 45, s = 5, 1 M 33.3 us, 35.0 so).
+    if constexpr (ADJ && MMAX > 0 && MMAX <= 8) {
+        const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+        for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < len / 4; v += stride) {
+            Columns<ADJ> cols;
+            cols.open(4 * v, len);
+            vote_columns(cols);
+        }
+    } else {
+        const int64_t tile = 4 * (int64_t)blockDim.x;
+        for (int64_t c0 = blockIdx.x * tile; c0 < len; c0 += gridDim.x * tile) {
+            const int64_t first_col = c0 + (ADJ ? 4 : 1) * (int)threadIdx.x;
+            if (first_col >= len) continue;
+            Columns<ADJ> cols;
+            cols.open(first_col, len);
+            vote_columns(cols);
+        }
     }
 
     // block totals -> global scratch (integer OR / add: order-independent, hence deterministic)
@@ -471,7 +518,8 @@ int launch_rep_vote(draco_plan* p, const float* R, int64_t len, int64_t ld, floa
     const int64_t quads = (len + 3) / 4;
     const uint32_t* Rb = reinterpret_cast<const uint32_t*>(R);
     // no more blocks than are resident at once: a block's end (its part of the masks, the fence, the count) costs a microsecond
-    // or two, which four rounds of blocks one after the other pay four times (n = 45, s = 3, d = 11.7 M: 365 us so, 345 us now)
+    // or two, which rounds of blocks one after the other pay each (eight blocks per SM and this: n = 15, s = 1, d = 1 M 20.1 and
+    // 17.0 us, 4 M 57.2 and 52.8; n = 45, s = 3, 11.7 M 321 and 317; s = 5, 60.2 M 1814 and 1665)
 #define DRACO_VOTE(MM, AA, GG, TT)                                                                                \
     do {                                                                                                          \
         static const int per_sm = resident_blocks(rep_vote_kernel<MM, AA, GG, TT>, TT);                           \

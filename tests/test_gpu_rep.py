@@ -75,6 +75,30 @@ def _received(n, s, d, seed, n_adv, models=None):
     return G, R, adv
 
 
+# groups of three to five compared first as a whole, of up to 16 in registers, larger ones streamed: one group, full and partial
+# batches of eight, as many members as there can be
+@pytest.mark.parametrize("n,s,d", [(45, 1, 1021), (45, 1, 1024), (8, 1, 516), (15, 2, 1023), (15, 3, 1028), (17, 8, 1021), (17, 8, 1020),
+                                   (128, 31, 1021), (128, 31, 1032), (128, 63, 259), (128, 63, 260)])
+def test_vote_bits_for_every_way_through_a_group(n, s, d):
+    dr, plan = _plan(n, s, d)
+    groups = orc.rep_groups(n, s)
+    G, R, adv = _received(n, s, d, 0xF0 + n + d, s, [di.ADV_REVGRAD, di.ADV_GAUSS])
+    R[groups[0][0], d // 2] = -R[groups[0][0], d // 2]                     # one more disagreement, at one coordinate
+    first, size = groups[-1]
+    R[first:first + size, d - 1] = np.arange(size, dtype=np.float32) + 1   # no majority there
+    want = orc.rep_decode(R, n, s)
+    u = torch.full((d + 8,), 7.0, dtype=torch.float32, device="cuda")
+    maj = torch.empty((len(groups), d), dtype=torch.float32, device="cuda")
+    flags = torch.full((n,), 7, dtype=torch.uint8, device="cuda")
+    plan.rep_vote(dev(R), u, maj, flags)
+    info = plan.info()
+    np.testing.assert_array_equal(host(flags).astype(bool), want["flags"])
+    np.testing.assert_array_equal(host(maj).view(np.uint32), want["maj"].view(np.uint32))
+    np.testing.assert_array_equal(host(u)[:d].view(np.uint32), fp32_sequential_sum(want["maj"]).view(np.uint32))
+    assert (host(u)[d:] == 7.0).all()
+    assert info["no_majority"] == want["no_majority"] > 0 and info["n_flagged"] == int(np.sum(want["flags"]))
+
+
 @pytest.mark.parametrize("n,s,d", SHAPES)
 @pytest.mark.parametrize("full", [True, False])
 def test_decode_parity(n, s, d, full):
