@@ -93,7 +93,8 @@ typedef struct draco_info {
     double im_residual;    /* cyclic decode, unpacked plans: max |Im(u-hat_i)| over the coordinates i with floor(i / 64) mod 8 = 0.
                               u-hat = R_{.,U} b is real when every node of U is honest, so against re_max this tells a decode
                               whose U still holds an adversary (wrong or missing flags, more than s adversaries) from a good
-                              one, whose residual is the rounding floor of complex64 vectors; 0 for packed plans */
+                              one, whose residual is the rounding floor of complex64 vectors; infinite where U holds a vector
+                              with NaN or infinities (seen at the sampled coordinates); 0 for packed plans */
     double re_max;         /* the same maximum of |Re(u-hat_i)|, the scale for im_residual */
 } draco_info;
 

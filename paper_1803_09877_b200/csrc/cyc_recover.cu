@@ -21,6 +21,9 @@ constexpr int kThreads = 256;
 constexpr int kUnroll = 8;
 constexpr int kShortCoordinates = 640;   // per SM: up to this length the short kernel is the faster one
 
+// |a| for the self-check's maxima; NaN, which a node may send and fmax would drop, counts as infinity
+__device__ __forceinline__ double magnitude(double a) { return a == a ? fabs(a) : __longlong_as_double(0x7ff0000000000000ll); }
+
 // PACKED: the vectors carry two gradient coordinates per complex entry (Section 3, last
 // paragraph): u[i] = Re(u-hat_i), u[len + i] = Im(u-hat_i) for len + i < d_packed.
 // VEC2: a thread owns two neighbouring coordinates, one 16-byte load per row.  Otherwise (odd row starts) two coordinates
@@ -72,8 +75,8 @@ cyc_recover_kernel(const float2* __restrict__ R, int64_t len, int64_t ld, const 
                     }
             }
             if (sampled) {
-                im_max = fmax(im_max, fmax(fabs(i0), fabs(i1)));
-                re_max = fmax(re_max, fmax(fabs(a0), fabs(a1)));
+                im_max = fmax(im_max, fmax(magnitude(i0), magnitude(i1)));
+                re_max = fmax(re_max, fmax(magnitude(a0), magnitude(a1)));
             }
             if (u != nullptr) {
                 __stcs(reinterpret_cast<float2*>(u + v * 2), make_float2((float)a0, (float)a1));
@@ -140,8 +143,8 @@ cyc_recover_kernel(const float2* __restrict__ R, int64_t len, int64_t ld, const 
                     }
             }
             if (sampled) {
-                im_max = fmax(im_max, fabs(i0));
-                re_max = fmax(re_max, fabs(a0));
+                im_max = fmax(im_max, magnitude(i0));
+                re_max = fmax(re_max, magnitude(a0));
             }
             if (u != nullptr) {
                 u[i] = (float)a0;
@@ -158,9 +161,7 @@ cyc_recover_kernel(const float2* __restrict__ R, int64_t len, int64_t ld, const 
         }
     }
     if (!PACKED) {
-        // non-negative doubles order like their bit patterns; NaN (an adversary may send it) counts as the largest
-        if (!(im_max == im_max)) im_max = __longlong_as_double(0x7ff0000000000000ll);
-        if (!(re_max == re_max)) re_max = __longlong_as_double(0x7ff0000000000000ll);
+        // non-negative doubles order like their bit patterns
 #pragma unroll
         for (int off = 16; off > 0; off >>= 1) {
             im_max = fmax(im_max, __shfl_xor_sync(0xffffffffu, im_max, off));
@@ -241,7 +242,7 @@ cyc_recover_short_kernel(const float2* __restrict__ R, int64_t len, int64_t ld, 
         if (w != nullptr) w[at] = fmaf(-scale, (float)a, w[at]);
     }
     if (sampled) {
-        double m = in ? fmax(0.0, fabs(a)) : 0.0;
+        double m = in ? magnitude(a) : 0.0;
 #pragma unroll
         for (int off = 16; off > 0; off >>= 1) m = fmax(m, __shfl_xor_sync(0xffffffffu, m, off));
         if (lane == 0 && m > 0.0) atomicMax(imag ? &info->im_residual_bits : &info->re_max_bits, (unsigned long long)__double_as_longlong(m));

@@ -4,6 +4,7 @@
 #include <stdlib.h>
 #include <string.h>
 
+#include <cmath>
 #include <complex>
 #include <new>
 #include <vector>
@@ -327,11 +328,12 @@ int draco_get_info(draco_plan* plan, draco_info* info, void* stream) {
     memcpy(&info->im_residual, &h.im_residual_bits, sizeof(double));
     memcpy(&info->re_max, &h.re_max_bits, sizeof(double));
     // The recovery kernel's blocks only merge their maxima; the verdict on them is formed here.  u-hat = G 1_P is
-    // real: an imaginary part beyond rounding means an adversary is still among the rows that were combined.
-    // (NaN from an adversary compares false with everything and so counts as a failed check.)
+    // real: an imaginary part beyond rounding means an adversary is still among the rows that were combined, and so does a
+    // maximum that is not finite (NaN counts as infinity there).
     if (is_cyc(plan) && (info->status == DRACO_OK || info->status == DRACO_EUNSURE)) {
-        const bool decoded = info->re_max > 0.0 || info->im_residual > 0.0 || info->re_max != info->re_max;   // since the last locate
-        const bool residual_ok = info->im_residual <= kImResidualBar * info->re_max;
+        const bool decoded = info->re_max > 0.0 || info->im_residual > 0.0;   // since the last locate
+        const bool residual_ok = std::isfinite(info->re_max) && std::isfinite(info->im_residual) &&
+                                 info->im_residual <= kImResidualBar * info->re_max;
         if (decoded && !residual_ok) {
             info->status = DRACO_EUNSURE;
         } else if (decoded && info->status == DRACO_EUNSURE && info->svd_sweeps >= 0 && !is_packed(plan)) {

@@ -595,6 +595,29 @@ def test_adversaries_sending_nan_or_infinities(n, s, d):
     assert normwise(host(u), G.astype(np.float64).sum(axis=0)) <= (1e-4 if n <= 15 else 1e-2)
 
 
+@pytest.mark.parametrize("d", [6150, 6151, 100_000, 100_003])          # the short and the long recovery, adjacent and odd rows
+@pytest.mark.parametrize("value", [np.nan, np.inf, -np.inf])
+@pytest.mark.parametrize("where", ["row", "entry"])
+def test_nan_or_infinity_left_among_the_rows_fails_the_self_check(d, value, where):
+    """decode with flags that leave a node's NaN or infinities in U: the sum is not finite, and the status says so, whether every
+    sampled coordinate is affected or one of them (all others then look clean)."""
+    import paper_1803_09877_b200 as dr
+    n, s = 15, 2
+    plan = dr.Plan(n, s, d, dr.CYC)
+    R = orc.cyc_encode(di.gradient_rows(7100 + d, n, d), n, s)
+    f = dev(di.projection_vector(7101 + d, d))
+    flags = torch.empty(n, dtype=torch.uint8, device="cuda")
+    u = torch.empty(d, dtype=torch.float32, device="cuda")
+    plan.locate_decode(dev(R), f, flags, u)
+    assert plan.info()["status"] == dr.binding.OK and np.isfinite(host(u)).all() and not host(flags).any()
+    R[4, slice(None) if where == "row" else 513] = value                # 513: in a sampled run, floor(513 / 64) mod 8 = 0
+    plan.decode(dev(R), flags, u)
+    info = plan.info()
+    assert not np.isfinite(host(u)[513])
+    assert info["status"] == dr.binding.EUNSURE
+    assert not np.isfinite(info["im_residual"]) or not np.isfinite(info["re_max"])
+
+
 def test_host_pipeline_over_several_column_chunks():
     """d large enough that draco_pipeline_host streams G in three column chunks (the last one ragged): the projection
     then accumulates over the chunks' launches.  Same worker vectors, flags and sum as the device-resident path."""
