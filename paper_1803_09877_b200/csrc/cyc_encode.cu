@@ -29,8 +29,9 @@
 // encoder at the accuracy floor of complex64 transport (2 n (2 s + 1) FMA per coordinate,
 // of which 5 n + 4 n in fp64).
 //
-// Packed mode filters complex inputs: the two halves' sums are combined before the rotation, which halves its cost and the
-// conversions of the results, and up to s = 4 everything runs in fp64 (each fp32 partial sum costs a conversion of 8 cycles, a
+// Packed mode filters complex inputs: the two halves' sums are combined before the rotation (s = 0, where there is nothing
+// to sum, after it: n = 15, d = 11.7 M 286 us, 238 so), which halves its cost and the conversions of the results, and up to
+// s = 4 everything runs in fp64 (each fp32 partial sum costs a conversion of 8 cycles, a
 // fp64 multiply-add 2).  n = 45, d = 60.2 M: s = 5 5.64 -> 5.31 ms, s = 3 5.06 -> 4.34 ms, s = 4 5.44 -> 5.2 ms; n = 15, s = 2
 // 1.35 -> 1.21 ms; s = 7, d = 30 M 3.24 -> 2.98 ms; error against fp64 at s <= 4 2.7e-8 -> 2.53e-8, elsewhere unchanged.  All of
 // s = 5 in fp64 measured 5.79 ms, five fp64 taps 6.02 ms.  The real centre tap (one fp64 operation per coordinate less) took
@@ -132,9 +133,10 @@ struct Cursor {
 
 // One step of the walk: bring row vv of the strip into window slot P (from the ring, or from the stash once
 // the circle has closed), emit z_{vv mod n} when the window is full, and refill the ring slot.
+// REALC: the centre tap's imaginary part, which is zero, is left out.
 // MODE 0: first SL steps of a strip (all rows from the ring; outputs from step 2 S on);
 // MODE 1: steady state (ring row + output);  MODE 2: anything (run-time guards).
-template <int S, int P, int MODE, bool PACKED>
+template <int S, int P, int MODE, bool PACKED, bool REALC>
 __device__ __forceinline__ void encode_step(Window<S, PACKED>& w, Cursor& cur, Fetcher<PACKED>& f, int vv, int n, int64_t ldz,
                                             uint32_t stash0, float2* zcol, bool act0, bool act1,
                                             const EncodeTaps& taps, const EncodeTaps64& taps64,
@@ -179,9 +181,10 @@ __device__ __forceinline__ void encode_step(Window<S, PACKED>& w, Cursor& cur, F
             ar[2] = fmaf(cr, g.z, ar[2]); ai[2] = fmaf(ci, g.z, ai[2]);
             ar[3] = fmaf(cr, g.w, ar[3]); ai[3] = fmaf(ci, g.w, ai[3]);
         }
-        constexpr int NOUT = PACKED ? 2 : 4;             // complex outputs of this thread
+        constexpr bool kJoin = PACKED && S > 0;          // the two halves' sums are joined before the rotation
+        constexpr int NOUT = kJoin ? 2 : 4;              // rotations of this thread
         double dr[NOUT], di[NOUT];
-        if constexpr (PACKED) {
+        if constexpr (kJoin) {
             // components 0, 1 of a row are the real parts of two complex coordinates, 2, 3 their imaginary parts
 #pragma unroll
             for (int c = 0; c < 2; ++c) {
@@ -213,7 +216,7 @@ __device__ __forceinline__ void encode_step(Window<S, PACKED>& w, Cursor& cur, F
 #pragma unroll
                 for (int c = 0; c < 4; ++c) {
                     dr[c] = fma(cr, w.cw[q][c], dr[c]);
-                    if (t != S) di[c] = fma(ci, w.cw[q][c], di[c]);
+                    if (!REALC || t != S) di[c] = fma(ci, w.cw[q][c], di[c]);
                 }
             }
         }
@@ -231,8 +234,13 @@ __device__ __forceinline__ void encode_step(Window<S, PACKED>& w, Cursor& cur, F
             dst = cur.zout;
             cur.zout += ldz;
         }
-        if constexpr (PACKED) {
+        if constexpr (kJoin) {
             if (act0) __stcs(reinterpret_cast<float4*>(dst), make_float4((float)xr[0], (float)xi[0], (float)xr[1], (float)xi[1]));
+        } else if constexpr (PACKED) {
+            // components 0, 1 filtered the real parts (X), 2, 3 the imaginary parts (Y): z = X + i Y
+            if (act0)
+                __stcs(reinterpret_cast<float4*>(dst), make_float4((float)(xr[0] - xi[2]), (float)(xi[0] + xr[2]),
+                                                                   (float)(xr[1] - xi[3]), (float)(xi[1] + xr[3])));
         } else {
             // A lane's two 16-byte stores are 512 bytes apart, so that each store instruction of the warp
             // covers 512 contiguous bytes (whole 32-byte sectors).  With the 4 coordinates of a lane adjacent,
@@ -251,21 +259,21 @@ __device__ __forceinline__ void encode_step(Window<S, PACKED>& w, Cursor& cur, F
     }
 }
 
-template <int S, int MODE, bool PACKED, int P = 0>
+template <int S, int MODE, bool PACKED, bool REALC, int P = 0>
 __device__ __forceinline__ void encode_chunk(Window<S, PACKED>& w, Cursor& cur, Fetcher<PACKED>& f, int v0, int n, int64_t ldz,
                                              uint32_t stash0, float2* zcol, bool act0, bool act1,
                                              const EncodeTaps& taps, const EncodeTaps64& taps64,
                                              const EncodePhase64& ph64) {
     if constexpr (P < StreamCfg<S, PACKED>::SL) {
-        encode_step<S, P, MODE, PACKED>(w, cur, f, v0 + P, n, ldz, stash0, zcol, act0, act1, taps, taps64, ph64);
-        encode_chunk<S, MODE, PACKED, P + 1>(w, cur, f, v0, n, ldz, stash0, zcol, act0, act1, taps, taps64, ph64);
+        encode_step<S, P, MODE, PACKED, REALC>(w, cur, f, v0 + P, n, ldz, stash0, zcol, act0, act1, taps, taps64, ph64);
+        encode_chunk<S, MODE, PACKED, REALC, P + 1>(w, cur, f, v0, n, ldz, stash0, zcol, act0, act1, taps, taps64, ph64);
     }
 }
 
 // PACKED: the real -> complex packing of Section 3's last paragraph.  `len` then counts complex
 // coordinates, a strip holds 64 of them, and a lane receives two pairs of each row:
 // G[r][c], G[r][c + 1] (real parts) and G[r][half + c], G[r][half + c + 1] (imaginary parts).
-template <int S, bool PACKED>
+template <int S, bool PACKED, bool REALC>
 __global__ void __launch_bounds__(StreamCfg<S, PACKED>::kThreads, 1)
 cyc_encode_stream_kernel(const float* __restrict__ G, float2* __restrict__ Z, int64_t len, int64_t ldg, int64_t ldz,
                          int64_t half, int n,
@@ -301,12 +309,12 @@ cyc_encode_stream_kernel(const float* __restrict__ G, float2* __restrict__ Z, in
         cur.zout = zcol + (int64_t)(2 * S) * ldz;
         int v0 = 0;
         if (n >= SL && S > 0) {
-            encode_chunk<S, 0, PACKED>(w, cur, f, 0, n, ldz, stash0, zcol, act0, act1, taps, taps64, ph64);
+            encode_chunk<S, 0, PACKED, REALC>(w, cur, f, 0, n, ldz, stash0, zcol, act0, act1, taps, taps64, ph64);
             for (v0 = SL; v0 + SL <= n; v0 += SL)
-                encode_chunk<S, 1, PACKED>(w, cur, f, v0, n, ldz, stash0, zcol, act0, act1, taps, taps64, ph64);
+                encode_chunk<S, 1, PACKED, REALC>(w, cur, f, v0, n, ldz, stash0, zcol, act0, act1, taps, taps64, ph64);
         }
         for (; v0 < total; v0 += SL)
-            encode_chunk<S, 2, PACKED>(w, cur, f, v0, n, ldz, stash0, zcol, act0, act1, taps, taps64, ph64);
+            encode_chunk<S, 2, PACKED, REALC>(w, cur, f, v0, n, ldz, stash0, zcol, act0, act1, taps, taps64, ph64);
     }
     cp_async_wait<0>();
 }
@@ -495,12 +503,12 @@ cyc_encode_generic_kernel(const float* __restrict__ G, float2* __restrict__ Z, i
     }
 }
 
-template <int S, bool PACKED>
+template <int S, bool PACKED, bool REALC = true>
 int launch_stream(const draco_plan* p, const float* G, float2* Z, int64_t len, int64_t ldg, int64_t ldz, int64_t half,
                   cudaStream_t st) {
     using Cfg = StreamCfg<S, PACKED>;
     constexpr int kThreads = Cfg::kThreads;
-    auto kern = cyc_encode_stream_kernel<S, PACKED>;
+    auto kern = cyc_encode_stream_kernel<S, PACKED, REALC>;
     static bool configured[64] = {};
     int dev = p->device;
     if (dev < 0 || dev >= 64) dev = 0;
@@ -533,7 +541,12 @@ int launch_stream_any(const draco_plan* p, const float* G, float2* Z, int64_t le
         case 4: return launch_stream<4, PACKED>(p, G, Z, len, ldg, ldz, half, st);
         case 5: return launch_stream<5, PACKED>(p, G, Z, len, ldg, ldz, half, st);
         case 6: return launch_stream<6, PACKED>(p, G, Z, len, ldg, ldz, half, st);
-        default: return launch_stream<7, PACKED>(p, G, Z, len, ldg, ldz, half, st);
+        default:
+            // a walk of fewer than 2 R rows is all head and tail, whose code is the slower one without the zero term (n = 15,
+            // s = 7, d = 1 M 52.3 us, 49.2 with it, 30 M 1196 and 1172; n = 29 2298 and 2247; but n = 30 2358 and 2365, n = 45
+            // 7195 and 7313 at 60.2 M)
+            if (!PACKED && p->n < 2 * StreamCfg<7, PACKED>::R) return launch_stream<7, PACKED, PACKED>(p, G, Z, len, ldg, ldz, half, st);
+            return launch_stream<7, PACKED>(p, G, Z, len, ldg, ldz, half, st);
     }
 }
 

@@ -365,6 +365,23 @@ def test_packed_encode_parity(n, s, d):
         assert np.abs(Zg[j] - Zo[j]).max() <= 1e-6 * np.abs(Zo[j]).max(), j
 
 
+# the streaming encoder's variants of their own: s = 7 with fewer than two filter lengths of rows (n = 15, 29; 30 is the first
+# with two), packed vectors without redundancy
+@pytest.mark.parametrize("code,n,s,d", [("CYC", 15, 7, 260), ("CYC", 16, 7, 4100), ("CYC", 29, 7, 1028), ("CYC", 30, 7, 1028), ("CYC", 31, 7, 260),
+                                        ("CYC_PACKED", 1, 0, 8), ("CYC_PACKED", 3, 0, 1000), ("CYC_PACKED", 15, 0, 20_008)])
+def test_encode_parity_of_the_streaming_variants(code, n, s, d):
+    import paper_1803_09877_b200 as dr
+    packed = code == "CYC_PACKED"
+    plan = dr.Plan(n, s, d, getattr(dr, code))
+    G = di.gradient_rows(0xD2B00 + n + s, n, d)
+    Z = torch.empty((n, d if packed else 2 * d), dtype=torch.float32, device="cuda")
+    plan.encode(dev(G), Z)
+    Zg = host(Z, complex64=True)
+    Zo = (orc.cyc_encode_packed if packed else orc.cyc_encode)(G, n, s, dtype=np.complex128)
+    for j in range(n):
+        assert np.abs(Zg[j] - Zo[j]).max() <= 1e-6 * np.abs(Zo[j]).max(), j     # the bar of test_encode_parity
+
+
 @pytest.mark.parametrize("n,s,d", PACKED_SHAPES)
 def test_packed_locate_decode_parity_and_exact_sum(n, s, d):
     dr, plan = _packed_plan(n, s, d)
