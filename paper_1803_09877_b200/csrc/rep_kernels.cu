@@ -77,7 +77,8 @@ struct Columns {
 
 // ---------------------------------------------------------------- encode
 // MMAX > 0: groups of at most MMAX members, GB groups fetched together so that about 16 rows are in flight per
-// thread whatever the group size (as in the vote kernel); MMAX == 0: larger groups, members streamed, eight at a time.
+// thread whatever the group size (as in the vote kernel); MMAX == 0: larger groups, members streamed, eight at a time (off the
+// 16-byte grid four: eight at n = 128, s = 20, d = 12,000,001 3802 us, four 3135).
 // Groups do not depend on one another: where the columns alone give few blocks, gridDim.y blocks share the groups of a column
 // range.  A thread that walks all of them is a chain of latencies (n = 45, s = 3, d = 100,000: 15.6 us so, 4.7 us shared; with
 // rows off the grid, d = 100,003, 19.1 and 8.9; streamed groups, n = 42, s = 10, d = 100,003, 41 and 10.7).
@@ -129,13 +130,14 @@ rep_encode_kernel(const float* __restrict__ G, float* __restrict__ Z, int64_t le
             for (int g = (int)blockIdx.y; g < gt.num_groups; g += (int)gridDim.y) {
                 const int first = gt.first[g], m = gt.size[g];
                 float acc[4];
-                for (int k0 = 0; k0 < m; k0 += kStreamBatch) {
-                    Pack x[kStreamBatch];
+                constexpr int kBatch = ADJ ? kStreamBatch : kStreamBatch / 2;
+                for (int k0 = 0; k0 < m; k0 += kBatch) {
+                    Pack x[kBatch];
 #pragma unroll
-                    for (int q = 0; q < kStreamBatch; ++q)
+                    for (int q = 0; q < kBatch; ++q)
                         if (k0 + q < m) cols.load(x[q], Gb + (int64_t)(first + k0 + q) * ldg);
 #pragma unroll
-                    for (int q = 0; q < kStreamBatch; ++q)
+                    for (int q = 0; q < kBatch; ++q)
                         if (k0 + q < m) {
 #pragma unroll
                             for (int c = 0; c < 4; ++c) {
