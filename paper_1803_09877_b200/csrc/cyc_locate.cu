@@ -127,6 +127,17 @@ cyc_project_kernel(const float2* __restrict__ R, const float* __restrict__ f, in
                             eq = fma(x1, x1, eq); eq = fma(y1, y1, eq);
                         }
                     }
+                } else if (RPW == 4 && TILE == kProjectTile) {
+                    // Up to four rows per warp, full tiles, rows off the 16-byte grid: left to the compiler's order of loads.  Sixteen at
+                    // a time, as below, cost 12 % (n = 17, d = 12,000,001 327 us, 280 so; n = 32 505 and 461), eight or four no less;
+                    // with more rows per warp they gain (n = 45 757 us so, 707).
+                    for (int i = lane; i < cnt; i += 32) {
+                        const float2 v = __ldcs(row + i);
+                        const double ff = fs[i], x0 = (double)v.x, y0 = (double)v.y;
+                        ar = fma(ff, x0, ar);
+                        ai = fma(ff, y0, ai);
+                        eq = fma(y0, y0, fma(x0, x0, eq));
+                    }
                 } else {
                     // 8-byte loads, which any row start allows; entries beyond the vector count as zero (and fs is zero there)
 #pragma unroll 1

@@ -82,6 +82,7 @@ def test_repetition_rows_off_the_grid(n, s, d):
 DECODE = [(code, n, s, d) for code in ("CYC", "CYC_PACKED")
           for n, s, d in [(5, 1, 1), (15, 2, 511), (15, 2, 513), (16, 3, 4097), (15, 2, 8200), (17, 2, 513), (45, 5, 2047),
                           (45, 5, 4100), (45, 5, 32_767), (45, 5, 32_770), (45, 5, 65_539), (70, 2, 1025), (105, 2, 33_001), (15, 2, 94_720), (15, 2, 94_722), (15, 2, 95_003), (15, 2, 189_447)]]
+DECODE += [("CYC", 17, 2, 40_003), ("CYC", 32, 5, 50_001), ("CYC_PACKED", 24, 4, 100_003)]
 
 
 @pytest.mark.parametrize("code,n,s,d", DECODE)
