@@ -113,9 +113,8 @@ int cuda_fail(cudaError_t err, const char* what);
 // Launch whose blocks may be set up while the kernel before it in the stream is still running (programmatic dependent launch).
 // Every kernel launched so begins with pdl_begin(): it lets the kernel after it be set up in turn (one of them does so at its
 // end), and waits until everything before it in the stream is complete and visible, before it touches global memory that another
-// kernel writes.  Saves the launch
-// gap, 1 - 2 us a kernel: n = 45, s = 5, d = 4096, locate and decode (three kernels) 37.8 -> 31.8 us; n = 15, s = 2, d = 1 M
-// 68.7 -> 63.5 us; a repetition encode of 100,000 coordinates costs the caller 3.8 instead of 4.4 us.
+// kernel writes.  Saves the launch gap, 1 - 2 us a kernel: n = 45, s = 5, d = 4096, locate and decode (three kernels) 37.8 -> 31.8
+// us; n = 15, s = 2, d = 1 M 68.7 -> 63.5 us; a repetition encode of 100,000 coordinates costs the caller 3.8 instead of 4.4 us.
 template <typename... Params, typename... Args>
 void launch_dependent(void (*kernel)(Params...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, Args... args) {
     cudaLaunchAttribute attr = {};
