@@ -137,7 +137,9 @@ void free_plan(draco_plan* p) {
 using namespace draco;
 
 namespace {
-constexpr int64_t kSplitBytes = (int64_t)2 << 20;    // chunks of G below this are not split: their kernels take no longer than a launch
+// Chunks of G below this (packed plans: of its first half, one of the chunk's two copies) are not split: their kernels take no
+// longer than a launch.
+constexpr int64_t kSplitBytes = (int64_t)2 << 20;
 }
 
 extern "C" {

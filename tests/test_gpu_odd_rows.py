@@ -141,10 +141,13 @@ def test_adversary_rows_of_any_alignment(code, d):
     np.testing.assert_array_equal(np.ascontiguousarray(got).view(np.uint32), np.ascontiguousarray(want).view(np.uint32))
 
 
-@pytest.mark.parametrize("code", ["REP", "CYC", "CYC_PACKED"])
-@pytest.mark.parametrize("d", [39_999, 40_000, 40_002, 65_536])
+# the second piece has what is left after a multiple of 4096 entries, an eighth of the vector or a little more: odd, a multiple of
+# 2, 4 or more, for packed plans also a shorter second half (d odd); packed plans below 70,000 make one copy
+@pytest.mark.parametrize("code,d", [(code, d) for code in ("REP", "CYC", "CYC_PACKED") for d in (39_999, 40_000, 40_002, 65_536)]
+                         + [("CYC_PACKED", d) for d in (79_999, 80_000, 80_002, 80_004, 131_073)])
 def test_host_pipeline_with_a_split_last_chunk(code, d):
-    """More than 2 MB of G: the call copies it in two pieces, and gives the bits of the device-resident path."""
+    """More than 2 MB of G (packed plans: of its first half): the call copies it in two pieces, and gives the bits of the
+    device-resident path."""
     import paper_1803_09877_b200 as dr
     n, s = 15, 2
     cyc, v = code != "REP", (d + 1) // 2 if code == "CYC_PACKED" else d
