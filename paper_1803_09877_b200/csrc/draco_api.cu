@@ -97,12 +97,10 @@ int build_cyclic_tables(draco_plan* p, std::vector<double2>* taps_full, std::vec
             p->taps64.tap[t] = (*taps_full)[t];
         }
     }
-    memset(&p->phase, 0, sizeof(p->phase));
     twiddle->resize(kMaxN);
     for (int j = 0; j < kMaxN; ++j) (*twiddle)[j] = make_double2(0.0, 0.0);
     for (int j = 0; j < n; ++j) {
         const cld ph = root_of_unity(n, (long long)j * M) * unit;
-        p->phase.phase[j] = make_float2((float)ph.real(), (float)ph.imag());
         p->phase64.phase[j] = make_double2((double)ph.real(), (double)ph.imag());
         const cld tw = root_of_unity(n, j);
         (*twiddle)[j] = make_double2((double)tw.real(), (double)tw.imag());

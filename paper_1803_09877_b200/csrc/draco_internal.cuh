@@ -28,10 +28,6 @@ struct EncodeTaps {                   // cyclic encoder: z_j = phase[j] * sum_t 
     float2 tap[kMaxTaps];
 };
 
-struct EncodePhase {
-    float2 phase[kMaxN];
-};
-
 struct EncodeTaps64 {                 // the same taps / phases in fp64 (centre taps and the final rotation)
     double2 tap[kMaxTaps];
 };
@@ -78,7 +74,6 @@ struct draco_plan {
     // cyclic (host copies)
     double* W_host;                   // [n][n][2]
     draco::EncodeTaps taps;
-    draco::EncodePhase phase;
     draco::EncodeTaps64 taps64;
     draco::EncodePhase64 phase64;
     double2* taps_full_dev;           // generic encoder: fp64 taps for any s, device [2s+1]
