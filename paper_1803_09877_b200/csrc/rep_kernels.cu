@@ -485,16 +485,31 @@ int launch_rep_encode(const draco_plan* p, const float* G, float* Z, int64_t len
                       cudaStream_t st) {
     const GroupTable& gt = p->groups;
     const bool adj = (len % 4 == 0) && (ldg % 4 == 0) && (ldz % 4 == 0);
-    const int64_t quads = (len + 3) / 4;
-    const int grid = grid_for(quads, kThreads, (int64_t)p->sm_count * 8);
-    // blocks that share the groups of a column range: as many as make sixteen blocks per SM (aligned rows) or eight.  More for
-    // the others costs where the shares are unequal: n = 15, s = 2, d = 1,000,003, two shares of three groups, 21.9 -> 24.4 us.
-    const int64_t room = (int64_t)p->sm_count * (adj ? 16 : 8) / grid;
-    auto blocks = [&](int gb) {
-        const int64_t steps = (gt.num_groups + gb - 1) / gb, share = room < steps ? room : steps;
-        return dim3(grid, share < 1 ? 1 : (unsigned)share);
+    struct Shape {
+        dim3 grid;
+        int threads;
     };
-#define DRACO_ENC(MM, AA, GG) launch_dependent(rep_encode_kernel<MM, AA, GG>, blocks(GG), kThreads, 0, st, G, Z, len, ldg, ldz, gt)
+    auto shape = [&](int gb) {
+        const int64_t steps = (gt.num_groups + gb - 1) / gb, sms = p->sm_count;
+        auto tiles = [&](int threads) {                    // column ranges of that many threads
+            const int64_t tile = 4 * threads - (adj ? 0 : kSector);
+            return (len + tile - 1) / tile;
+        };
+        // the kernel's limit, fewer where that would not give every SM two blocks (n = 15, s = 5, d = 48,827: 256 threads 7.0 us,
+        // 64 3.9); a block more than there are ranges short is a second range for some (100,003: 7.6 us, 3.9 without)
+        int threads = kThreads;
+        while (threads > 64 && tiles(threads) * steps < 2 * sms) threads /= 2;
+        const int64_t cap = sms * 8 * (kThreads / threads), x = tiles(threads) < cap ? tiles(threads) : cap;
+        // blocks that share the groups of a column range: as many as make sixteen blocks per SM (aligned rows) or eight.  More for
+        // the others costs where the shares are unequal: n = 15, s = 2, d = 1,000,003, two shares of three groups, 21.9 -> 24.4 us.
+        const int64_t room = sms * (adj ? 16 : 8) * (kThreads / threads) / x, share = room < steps ? room : steps;
+        return Shape{dim3((unsigned)x, share < 1 ? 1 : (unsigned)share), threads};
+    };
+#define DRACO_ENC(MM, AA, GG)                                                                                     \
+    do {                                                                                                          \
+        const Shape sh = shape(GG);                                                                               \
+        launch_dependent(rep_encode_kernel<MM, AA, GG>, sh.grid, sh.threads, 0, st, G, Z, len, ldg, ldz, gt);     \
+    } while (0)
 #define DRACO_ENC_BY_SIZE(AA)                                      \
     do {                                                           \
         if (gt.max_size <= 3) DRACO_ENC(3, AA, 5);                 \
