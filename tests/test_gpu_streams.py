@@ -46,3 +46,51 @@ def test_first_call_on_a_new_plan_on_a_side_stream(code, n, s, d):
         assert normwise(host(u), ref) <= 1e-6
         honest = [j for j in range(n) if j not in adv]
         assert normwise(host(Z).reshape(n, -1)[honest], np.ascontiguousarray(R[honest]).view(np.float32)) <= 1e-6
+
+
+@pytest.mark.parametrize("code,n,s,d", [("REP", 15, 2, 20_003), ("REP", 42, 10, 4096), ("CYC", 20, 8, 3001), ("CYC", 15, 7, 4100),
+                                        ("CYC_PACKED", 15, 2, 8002)])
+def test_two_chains_captured_on_forked_streams(code, n, s, d):
+    """Copies, encodes, adversaries and decodes of two plans in one graph, on two streams that fork and join: replays give the bits of
+    the eager calls (kernels set up early, kernels launched in the ordinary way and copies follow one another in it)."""
+    import paper_1803_09877_b200 as dr
+    cyc, packed = code != "REP", code == "CYC_PACKED"
+    v = (d + 1) // 2 if packed else d
+    adv = di.choose_adversaries(5400 + n, n, s)
+    fd = dev(di.projection_vector(5500 + n, v)) if cyc else None
+
+    class Chain:
+        def __init__(self, seed):
+            self.plan = dr.Plan(n, s, d, getattr(dr, code))
+            self.src = dev(di.gradient_rows(seed, n, d))
+            self.G = torch.empty_like(self.src)
+            self.Z = torch.empty((n, 2 * v if cyc else v), dtype=torch.float32, device="cuda")
+            self.flags = torch.empty(n, dtype=torch.uint8, device="cuda")
+            self.u = torch.empty(d, dtype=torch.float32, device="cuda")
+            self.outputs = (self.Z, self.flags, self.u)
+
+        def run(self):
+            self.G.copy_(self.src)
+            self.plan.encode(self.G, self.Z)
+            self.plan.corrupt(self.Z, adv, [di.ADV_REVGRAD] * s, [100.0] * s, seed=3)
+            self.plan.locate_decode(self.Z, fd, self.flags, self.u)
+
+    a, b = Chain(5600 + n), Chain(5700 + n)
+    a.run()
+    b.run()
+    torch.cuda.synchronize()
+    want = [t.clone() for t in a.outputs + b.outputs]
+    main, side, graph = torch.cuda.Stream(), torch.cuda.Stream(), torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph, stream=main):
+        side.wait_stream(main)
+        a.run()
+        with torch.cuda.stream(side):
+            b.run()
+        main.wait_stream(side)
+    for _ in range(2):
+        for t in (a.G, b.G) + a.outputs + b.outputs:
+            t.fill_(3)
+        graph.replay()
+        torch.cuda.synchronize()
+        for got, ref in zip(a.outputs + b.outputs, want):
+            assert torch.equal(got, ref)
