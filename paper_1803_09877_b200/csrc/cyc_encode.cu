@@ -31,11 +31,12 @@
 //
 // Packed mode filters complex inputs: the two halves' sums are combined before the rotation (s = 0, where there is nothing
 // to sum, after it: n = 15, d = 11.7 M 286 us, 238 so), which halves its cost and the conversions of the results, and up to
-// s = 4 everything runs in fp64 (each fp32 partial sum costs a conversion of 8 cycles, a
-// fp64 multiply-add 2).  n = 45, d = 60.2 M: s = 5 5.64 -> 5.31 ms, s = 3 5.06 -> 4.34 ms, s = 4 5.44 -> 5.2 ms; n = 15, s = 2
-// 1.35 -> 1.21 ms; s = 7, d = 30 M 3.24 -> 2.98 ms; error against fp64 at s <= 4 2.7e-8 -> 2.53e-8, elsewhere unchanged.  All of
-// s = 5 in fp64 measured 5.79 ms, five fp64 taps 6.02 ms.  The real centre tap (one fp64 operation per coordinate less) took
-// the unpacked encoder from 6.29 to 6.24 ms at s = 5 and from 3.64 to 3.45 ms at s = 7, d = 30 M.
+// s = 4 everything runs in fp64 (each fp32 partial sum costs a conversion of 8 cycles, a fp64 multiply-add 2).  Against the sums
+// kept apart, both timed in turn: n = 45, d = 60.2 M: s = 5 5.79 -> 5.17 ms, s = 3 5.30 -> 4.44 ms, s = 7 6.52 -> 5.91 ms; n = 15,
+// s = 2 1.45 -> 1.20 ms; error against fp64 at s <= 4 2.7e-8 -> 2.53e-8, elsewhere unchanged.  All of s = 5 in fp64 measured
+// 5.79 ms, five fp64 taps 6.02 ms.  The real centre tap (one fp64 operation per coordinate less) took the unpacked encoder from
+// 6.21 to 6.13 ms at s = 5 and from 7.39 to 7.27 ms at s = 7.  In a loop of launches the power cap lowers the clock: unpacked,
+// s = 5, 5.6 ms at 1965 MHz, 6.3 at 1665; packed 5.0 and 5.4 at 1820.
 #include "draco_internal.cuh"
 
 namespace draco {

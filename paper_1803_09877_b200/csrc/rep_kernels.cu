@@ -496,7 +496,7 @@ int launch_rep_encode(const draco_plan* p, const float* G, float* Z, int64_t len
             return (len + tile - 1) / tile;
         };
         // the kernel's limit, fewer where that would not give every SM two blocks (n = 15, s = 5, d = 48,827: 256 threads 7.0 us,
-        // 64 3.9); a block more than there are ranges short is a second range for some (100,003: 7.6 us, 3.9 without)
+        // 64 3.9); the grid counts ranges and not coordinates per thread, so that no block has a second one (100,003: 7.6 and 3.9)
         int threads = kThreads;
         while (threads > 64 && tiles(threads) * steps < 2 * sms) threads /= 2;
         const int64_t cap = sms * 8 * (kThreads / threads), x = tiles(threads) < cap ? tiles(threads) : cap;
