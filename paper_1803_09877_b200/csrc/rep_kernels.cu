@@ -247,40 +247,45 @@ __device__ __forceinline__ void vote_step(uint32_t x, uint32_t& ma, int& counter
 template <int MMAX>
 __device__ __forceinline__ void vote_group(const Pack (&val)[MMAX], int m, uint32_t in, uint32_t (&sel)[4], uint32_t& dis,
                                            unsigned int& nomaj) {
-    // Small groups: nearly all of them agree bit for bit, which is cheaper to see than to count (n = 45, s = 1, d = 60.2 M 1843
-    // -> 1675 us, rows off the 16-byte grid, 11.7 M + 1, 383 -> 348; from six members on the count below is as cheap, n = 45,
-    // s = 5, 60.2 M 1691 us without and 1912 with this).
-    if constexpr (MMAX <= 5) {
-        uint32_t differ = 0;
-#pragma unroll
-        for (int k = 1; k < MMAX; ++k)
-            if (k < m) {
-#pragma unroll
-                for (int c = 0; c < 4; ++c) differ |= val[k].get(c) ^ val[0].get(c);
-            }
-        if (differ == 0) {
-#pragma unroll
-            for (int c = 0; c < 4; ++c) sel[c] = val[0].get(c);
-            return;
-        }
-    }
     // A value held by strictly more than half of the group IS what Algorithm 2 returns.  So count first the members that equal
     // member 0 in all four columns (five logic operations each), then those that equal member 1 (member 0 may be the
     // adversary); only if neither has a strict majority is the streaming vote itself run, column by column.  Counting column by
     // column at once took about twice the instructions and left large groups bound by them (n = 45, d = 5 M: s = 7 244 us, now
     // 188; s = 5 162 us, now 141).
+    // Nearly all groups agree bit for bit: up to eight members the differences from member 0 are looked at together before they are
+    // counted (n = 45, s = 1, d = 20 M 617 us without, 560 so; n = 64, s = 2 873 and 788; every group with an adversary, n = 10, s = 2
+    // 145 and 144).  Larger groups have no registers to keep them (n = 9, s = 4, 20 M 251 us, 282 so).
     bool settled = false;
 #pragma unroll
     for (int ref = 0; ref < 2 && ref < MMAX; ++ref) {
         if (!settled && ref < m) {
             const uint4 r = val[ref].v;
+            auto apart = [&](int k) {                      // non-zero where member k differs from `ref`
+                const uint4 x = val[k].v;
+                return (x.x ^ r.x) | (x.y ^ r.y) | (x.z ^ r.z) | (x.w ^ r.w);
+            };
             uint32_t ne = 0;
+            if constexpr (MMAX <= 8) {
+                uint32_t diff[MMAX], any = 0;
 #pragma unroll
-            for (int k = 0; k < MMAX; ++k)
-                if (k != ref && k < m) {
-                    const uint4 x = val[k].v;
-                    ne |= (((x.x ^ r.x) | (x.y ^ r.y) | (x.z ^ r.z) | (x.w ^ r.w)) != 0u ? 1u : 0u) << k;
+                for (int k = 0; k < MMAX; ++k)
+                    if (k != ref && k < m) {
+                        diff[k] = apart(k);
+                        any |= diff[k];
+                    }
+                if (ref == 0 && any == 0u) {
+#pragma unroll
+                    for (int c = 0; c < 4; ++c) sel[c] = val[0].get(c);
+                    return;
                 }
+#pragma unroll
+                for (int k = 0; k < MMAX; ++k)
+                    if (k != ref && k < m) ne |= (diff[k] != 0u ? 1u : 0u) << k;
+            } else {
+#pragma unroll
+                for (int k = 0; k < MMAX; ++k)
+                    if (k != ref && k < m) ne |= (apart(k) != 0u ? 1u : 0u) << k;
+            }
             if (2 * (m - __popc(ne)) > m) {
 #pragma unroll
                 for (int c = 0; c < 4; ++c) sel[c] = val[ref].get(c);
