@@ -19,7 +19,8 @@ namespace {
 
 constexpr int kThreads = 256;
 constexpr int kUnroll = 8;
-constexpr int kShortCoordinates = 640;   // per SM: up to this length the short kernel is the faster one
+constexpr int kShortCoordinates = 300;   // per SM: up to this length the short kernel is the faster one ..
+constexpr int kShortFewRows = 140;       // .. and with at most 16 rows
 
 // |a| for the self-check's maxima; NaN, which a node may send and fmax would drop, counts as infinity
 __device__ __forceinline__ double magnitude(double a) { return a == a ? fabs(a) : __longlong_as_double(0x7ff0000000000000ll); }
@@ -176,7 +177,9 @@ cyc_recover_kernel(const float2* __restrict__ R, int64_t len, int64_t ld, const 
 
 // The same for short vectors, whose time is a chain of load latencies (five batches of eight rows one after the other at
 // n = 45): a block takes 64 coordinates, its warps the rows w, w + 8, .., all loads of a warp in flight together; the
-// warps' sums are added in ascending order.  n = 45, s = 5, d = 4096: locate and decode 39.9 -> 37.8 us; d = 100,000 48.2 us with either kernel.
+// warps' sums are added in ascending order.  Where the lines lie, locate and decode, the other kernel / this one in us: n = 45,
+// s = 5, d = 10,000 22.0 / 21.6, 20,000 26.9 / 24.3, 40,000 34.5 / 31.6, but 50,000 34.4 / 37.0, 94,000 46 / 58; n = 105, s = 2,
+// 31,000 53 / 50, 60,000 73 / 88, 94,000 96 / 125; n = 15, s = 2, 20,000 17.0 / 17.2, 31,000 17.4 / 19.7, 94,000 21.5 / 27.5.
 constexpr int kShortBatch = 8;
 template <bool VEC2, bool PACKED>
 __global__ void __launch_bounds__(kThreads)
@@ -266,7 +269,7 @@ int launch_cyc_recover(draco_plan* p, const float2* R, int64_t len, int64_t ld, 
 #define DRACO_REC_SHORT(V2, PK)                                                                                                    \
     launch_dependent(cyc_recover_short_kernel<V2, PK>, (int)((len + 63) / 64), kThreads, 0, st, R, len, ld, p->cyc_dev, p->info_dev, u, d_packed, w, \
                                                                                   scale)
-    if (len <= (int64_t)p->sm_count * kShortCoordinates) {
+    if (len <= (int64_t)p->sm_count * (p->n <= 16 ? kShortFewRows : kShortCoordinates)) {
         if (vec2) {
             if (packed) DRACO_REC_SHORT(true, true); else DRACO_REC_SHORT(true, false);
         } else {

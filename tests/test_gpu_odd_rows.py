@@ -80,10 +80,12 @@ def test_repetition_rows_off_the_grid(n, s, d):
 # The few-rows projection takes 512 coordinates per warp and splits the rows of short vectors over blocks.  The tile kernel takes 512
 # coordinates per block up to 32,768, and also where full tiles would leave more partials than the locator adds up itself (3 n per
 # tile, 8192) and small ones are at most two rounds of blocks (four per SM): n = 45 from 122,881 to 606,208 on 148 SMs, n = 105 from
-# 53,249, n = 17 from 327,681; 2048 otherwise.  The recovery takes 64 per block up to 640 per SM, then 512.
+# 53,249, n = 17 from 327,681; 2048 otherwise.  The recovery takes 64 per block
+# up to 300 per SM (44,400), with at most 16 rows 140 (20,720), then 512.
 DECODE = [(code, n, s, d) for code in ("CYC", "CYC_PACKED")
           for n, s, d in [(5, 1, 1), (15, 2, 511), (15, 2, 513), (16, 3, 4097), (15, 2, 8200), (17, 2, 513), (45, 5, 2047),
                           (45, 5, 4100), (45, 5, 32_767), (45, 5, 32_770), (45, 5, 65_539), (70, 2, 1025), (105, 2, 33_001), (15, 2, 94_720), (15, 2, 94_722), (15, 2, 95_003), (15, 2, 189_447)]]
+DECODE += [(code, n, s, k * d + r) for code, k in (("CYC", 1), ("CYC_PACKED", 2)) for n, s, d in [(15, 2, 20_720), (17, 2, 44_400)] for r in (-1, 0, 1, 2)]
 DECODE += [("CYC", n, s, d) for n, s, d in [(45, 5, 122_879), (45, 5, 122_883), (45, 5, 200_003), (45, 5, 303_203), (45, 2, 606_207), (45, 2, 606_211),
                                             (105, 2, 53_249), (105, 2, 100_001), (17, 2, 40_003), (32, 5, 50_001), (24, 4, 100_000), (17, 2, 400_003)]]
 DECODE += [("CYC_PACKED", n, s, d) for n, s, d in [(45, 5, 245_767), (45, 5, 400_006), (105, 2, 200_003), (24, 4, 100_003), (45, 2, 1_212_421)]]
