@@ -815,6 +815,24 @@ __device__ __noinline__ void run_recurrence(double2* h, int n, int count, const 
     }
 }
 
+// The same for more than kRegSystem unknowns, the terms left to the compiler's unrolling: their loads are most of a step (n = 128,
+// s = 20, locate 1295 us rolled, 1231 so).  A function of its own, so that its instructions do not lie between those of the small
+// systems (in their midst: n = 15, s = 2, d = 4096, locate and decode 16.4 us, 15.9 so).
+__device__ __noinline__ void run_recurrence_any(double2* h, int n, int count, int S, const double2* beta) {
+#pragma unroll 1
+    for (int l = 0; l < count; ++l) {
+        double a = 0.0, b = 0.0;
+        for (int u = 0; u < S; ++u) {
+            int idx = l + u - S;
+            if (idx < 0) idx += n;
+            const double2 q = cmul(beta[u], h[idx]);
+            a += q.x;
+            b += q.y;
+        }
+        h[l] = make_double2(a, b);
+    }
+}
+
 #define DRACO_BY_SIZE(size, CALL)                                                                            \
     switch (size) {                                                                                          \
         case 1: CALL(1); break;                                                                              \
@@ -1251,19 +1269,7 @@ cyc_solve_kernel(CycDevice* cd, const double2* __restrict__ e_in, const double2*
                 DRACO_BY_SIZE(s2, DRACO_RECUR)
 #undef DRACO_RECUR
             } else {
-#pragma unroll 1
-                for (int l = 0; l < count; ++l) {
-                    double a = 0.0, b = 0.0;
-                    // (not kept rolled: the terms' loads are most of a step; n = 128, s = 20, locate 1173 us rolled, 1116 so)
-                    for (int u = 0; u < s2; ++u) {
-                        int idx = l + u - s2;
-                        if (idx < 0) idx += n;
-                        const double2 q = cmul(beta_s[u], h[idx]);
-                        a += q.x;
-                        b += q.y;
-                    }
-                    h[l] = make_double2(a, b);
-                }
+                run_recurrence_any(h, n, count, s2, beta_s);
             }
         }
         __syncthreads();
