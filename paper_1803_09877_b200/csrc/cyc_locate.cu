@@ -63,7 +63,7 @@ __device__ __forceinline__ double* q_partials(double2* partial, int cap, int n) 
     return reinterpret_cast<double*>(partial + (int64_t)cap * n);
 }
 // Block = 8 warps over one tile of coordinates; warp w owns rows row0 + w, row0 + w + 8, ... of the
-// launch's nrows <= 8 RPW rows; f for the tile sits in shared memory as fp64 (converted once per tile, used by
+// launch's nrows <= 8 RPW rows; every: 1, or only each `every`-th tile is read; f for the tile sits in shared memory as fp64 (converted once per tile, used by
 // every row).  More than 64 rows take two launches of half the rows each (rows are
 // independent; f is read twice, 1 % more traffic): 16 rows per warp in registers halve the blocks per SM
 // (0.79 of the copy bandwidth at n = 105), and per-lane sums in shared memory left the compiler too few
@@ -71,7 +71,7 @@ __device__ __forceinline__ double* q_partials(double2* partial, int cap, int n) 
 template <int RPW, bool VEC2, int TILE>
 __global__ void __launch_bounds__(kThreads, 4)
 cyc_project_kernel(const float2* __restrict__ R, const float* __restrict__ f, int64_t len, int64_t ld, int n,
-                   int row0, int nrows, double2* __restrict__ partial, int cap, int accumulate) {
+                   int row0, int nrows, double2* __restrict__ partial, int cap, int accumulate, int every) {
     pdl_begin();
     __shared__ __align__(16) double fs[TILE];
     // Running sums of row warp + r * 8 over this block's tiles, kept by lane 0 of the row's warp: after every tile
@@ -98,7 +98,7 @@ cyc_project_kernel(const float2* __restrict__ R, const float* __restrict__ f, in
     }
 
     const int64_t ntiles = (len + TILE - 1) / TILE;
-    for (int64_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
+    for (int64_t tile = (int64_t)blockIdx.x * every; tile < ntiles; tile += (int64_t)gridDim.x * every) {
         const int64_t c0 = tile * TILE;
         const int cnt = (int)((len - c0) < TILE ? (len - c0) : TILE);
         for (int i = threadIdx.x; i < TILE; i += kThreads) fs[i] = (i < cnt) ? (double)__ldcs(f + c0 + i) : 0.0;
@@ -200,7 +200,7 @@ constexpr int kFewRows = 16;
 template <bool VEC2, bool SPLIT>
 __global__ void __launch_bounds__(kThreads, 3)
 cyc_project_fewrows_kernel(const float2* __restrict__ R, const float* __restrict__ f, int64_t len, int64_t ld, int n,
-                           double2* __restrict__ partial, int cap, int accumulate) {
+                           double2* __restrict__ partial, int cap, int accumulate, int every) {
     pdl_begin();
     constexpr int CH = kProjectChunk;
     __shared__ double2 es[kProjectWarps][kFewRows];
@@ -230,8 +230,8 @@ cyc_project_fewrows_kernel(const float2* __restrict__ R, const float* __restrict
         nrows = (n - row0) < per ? (n - row0) : per;
     }
     const int64_t nchunks = (len + CH - 1) / CH;
-    const int64_t nwarps = (int64_t)gridDim.x * kProjectWarps;
-    for (int64_t chunk = (int64_t)blockIdx.x * kProjectWarps + warp; chunk < nchunks; chunk += nwarps) {
+    const int64_t nwarps = (int64_t)gridDim.x * kProjectWarps * every;
+    for (int64_t chunk = ((int64_t)blockIdx.x * kProjectWarps + warp) * every; chunk < nchunks; chunk += nwarps) {
         const int64_t c0 = chunk * CH;
         const int cnt = (int)((len - c0) < CH ? (len - c0) : CH);
         if (VEC2 && cnt == CH) {
@@ -895,9 +895,9 @@ __device__ void decode_vector_body(CycDevice* cd, const uint8_t* fl, const doubl
     const int a = list_flagged(fl, n, vlist, bits);
     if (a > 2 * s) {                                       // fewer than n - 2 s rows left: no b exists
         if (tid < n) cd->b[tid] = make_double2(0.0, 0.0);
-        if (tid == 0) {
+        if (tid == kSolveThreads - 1) {
             info->n_active = 0; info->n_flagged = a; info->status = DRACO_ETOOMANY;
-            info->im_residual_bits = 0ull; info->re_max_bits = 0ull;
+            info->im_residual_bits = 0ull; info->re_max_bits = 0ull; info->combine = 0;
         }
         return;
     }
@@ -992,6 +992,7 @@ __device__ void decode_vector_body(CycDevice* cd, const uint8_t* fl, const doubl
         info->n_flagged = a;
         info->im_residual_bits = 0ull;                     // the recovery kernel's blocks merge their maxima into these
         info->re_max_bits = 0ull;
+        info->combine = n - a;
         if (info->status == DRACO_ETOOMANY) info->status = DRACO_OK;
     }
 }
@@ -1019,7 +1020,8 @@ cyc_decode_vector_kernel(CycDevice* cd, const uint8_t* __restrict__ flags, int n
 // decode vector included: 47 us with a thread per sum, one-thread list building and the singular-value iteration.
 __global__ void __launch_bounds__(kSolveThreads)
 cyc_solve_kernel(CycDevice* cd, const double2* __restrict__ e_in, const double2* __restrict__ partial, int used, int cap,
-                 int n, int s, double theta, ModN mod, double rsn, uint8_t* flags, uint8_t* flags2, DeviceInfo* info, int with_b) {
+                 int n, int s, double theta, ModN mod, double rsn, uint8_t* flags, uint8_t* flags2, DeviceInfo* info, int with_b,
+                 const uint8_t* sample_flags, const DeviceInfo* sample) {
     __shared__ double2 e[kMaxN], h[kMaxN + 1], tw[kMaxN];
     __shared__ double2 As[kSmallDim * kSmallDim], Vs[kSmallDim * kSmallDim];
     __shared__ double2 rhs_s[kMaxN / 2], beta_s[kMaxN / 2], coef_s[kMaxN / 2];
@@ -1335,6 +1337,14 @@ cyc_solve_kernel(CycDevice* cd, const double2* __restrict__ e_in, const double2*
     if (with_b) {                                          // the decode vector for the V just found, same launch
         __syncthreads();
         decode_vector_body(cd, fl_s, tw, n, s, mod, rsn, info);
+        if (sample != nullptr) {                           // u has been written for the sample's V, if that was beyond doubt
+            const int differ = __syncthreads_count(tid < n && fl_s[tid] != sample_flags[tid]);
+            if (tid == kSolveThreads - 1 && differ == 0 && sample->status == DRACO_OK) {
+                info->im_residual_bits = sample->im_residual_bits;
+                info->re_max_bits = sample->re_max_bits;
+                info->combine = -1;
+            }
+        }
     }
 }
 
@@ -1379,12 +1389,12 @@ static ProjectShape project_shape(int cap, int sm_count, int64_t len, int n) {
 // All launches of one projection: n <= 16 the few-rows kernel, n <= 64 one launch of the tile kernel, otherwise two
 // launches of it over half the rows each.  partial: [cap][n] double2 followed by [cap][n] double.
 static cudaError_t launch_project_kernels(int cap, const ProjectShape& shape, cudaStream_t st, const float2* R, const float* f,
-                                          int64_t len, int64_t ld, int n, double2* partial, int accumulate) {
+                                          int64_t len, int64_t ld, int n, double2* partial, int accumulate, int every = 1) {
     const bool vec2 = (ld % 2 == 0);
     const int grid = shape.grid, tile = shape.tile;
     if (n <= kFewRows) {
         const dim3 grid2(grid, shape.gridy);
-#define DRACO_FEW(VV, SS) launch_dependent(cyc_project_fewrows_kernel<VV, SS>, grid2, kThreads, 0, st, R, f, len, ld, n, partial, cap, accumulate)
+#define DRACO_FEW(VV, SS) launch_dependent(cyc_project_fewrows_kernel<VV, SS>, grid2, kThreads, 0, st, R, f, len, ld, n, partial, cap, accumulate, every)
         if (shape.gridy > 1) {
             if (vec2) DRACO_FEW(true, true); else DRACO_FEW(false, true);
         } else {
@@ -1405,7 +1415,7 @@ static cudaError_t launch_project_kernels(int cap, const ProjectShape& shape, cu
     }
     const dim3 grid2(grid, ysplit);
 #define DRACO_PROJECT(RR, VV, TT) \
-    launch_dependent(cyc_project_kernel<RR, VV, TT>, grid2, kThreads, 0, st, R, f, len, ld, n, row0, nrows, partial, cap, accumulate)
+    launch_dependent(cyc_project_kernel<RR, VV, TT>, grid2, kThreads, 0, st, R, f, len, ld, n, row0, nrows, partial, cap, accumulate, every)
 #define DRACO_PROJECT_TILE(RR, VV)                                           \
     do {                                                                     \
         if (tile == kProjectTile) DRACO_PROJECT(RR, VV, kProjectTile);       \
@@ -1448,6 +1458,26 @@ int launch_cyc_project(draco_plan* p, const float2* R, const float* f, int64_t l
     return DRACO_OK;
 }
 
+static ModN mod_n(int n) { return ModN{(uint32_t)n, (uint32_t)(((1ull << 32) + (uint64_t)n - 1) / (uint64_t)n)}; }
+
+// The locator and the decode vector from a sample of R's columns, tiles spread over the whole length: the flags to the second half
+// of flags_dev, the status to info_dev[1].  As many tiles as the locator kernel adds up itself, 48 at most (24,576 coordinates),
+// n <= 16: sixteen blocks (65,536); the sums over them are as telling as those of a vector of that length.
+int launch_cyc_sample(draco_plan* p, const float2* R, const float* f, int64_t len, int64_t ld, cudaStream_t st) {
+    const int n = p->n, cap = p->project_grid;
+    const bool few = n <= kFewRows;
+    int blocks = few ? 16 : kFusedReduceMax / (3 * n);
+    if (blocks > 48) blocks = 48;
+    const int64_t sample = (int64_t)blocks * (few ? kProjectChunk * kProjectWarps : kProjectTileShort);
+    const int64_t every = len < sample ? 1 : len / sample;
+    const ProjectShape shape = {blocks, few ? n : 1, kProjectTileShort};
+    DRACO_CUDA(launch_project_kernels(cap, shape, st, R, f, len, ld, n, p->partial_dev, 0, (int)every));
+    launch_dependent(cyc_solve_kernel, 1, kSolveThreads, 0, st, p->cyc_dev, nullptr, p->partial_dev, blocks, cap, n, p->s, p->theta,
+                     mod_n(n), 1.0 / sqrt((double)n), nullptr, p->flags_dev + kMaxN, p->info_dev + 1, 1, nullptr, nullptr);
+    DRACO_CUDA(cudaGetLastError());
+    return DRACO_OK;
+}
+
 int launch_cyc_project_finish(draco_plan* p, double2* e_out, cudaStream_t st) {
     launch_dependent(cyc_reduce_partials_kernel, p->n, kReduceThreads, 0, st, p->partial_dev, p->project_used,
                      p->project_grid, p->n, reinterpret_cast<double*>(e_out));
@@ -1455,12 +1485,10 @@ int launch_cyc_project_finish(draco_plan* p, double2* e_out, cudaStream_t st) {
     return DRACO_OK;
 }
 
-static ModN mod_n(int n) { return ModN{(uint32_t)n, (uint32_t)(((1ull << 32) + (uint64_t)n - 1) / (uint64_t)n)}; }
-
 // e == nullptr: the record of the plan's own projection (launch_cyc_project) is formed first: by the locator kernel
 // itself when the projection left few block partials (short vectors, where every launch counts), by the reduction
 // kernel otherwise.  with_b: the decode vector for the set V just found is formed in the same launch.
-int launch_cyc_solve(draco_plan* p, const double2* e, uint8_t* flags, bool with_b, cudaStream_t st) {
+int launch_cyc_solve(draco_plan* p, const double2* e, uint8_t* flags, bool with_b, cudaStream_t st, bool sampled) {
     const double2* partial = nullptr;
     int used = 0;
     if (!e) {
@@ -1475,7 +1503,8 @@ int launch_cyc_solve(draco_plan* p, const double2* e, uint8_t* flags, bool with_
         }
     }
     launch_dependent(cyc_solve_kernel, 1, kSolveThreads, 0, st, p->cyc_dev, e, partial, used, p->project_grid, p->n, p->s,
-                     p->theta, mod_n(p->n), 1.0 / sqrt((double)p->n), flags, p->flags_dev, p->info_dev, with_b ? 1 : 0);
+                     p->theta, mod_n(p->n), 1.0 / sqrt((double)p->n), flags, p->flags_dev, p->info_dev, with_b ? 1 : 0,
+                     sampled ? p->flags_dev + kMaxN : nullptr, sampled ? p->info_dev + 1 : nullptr);
     DRACO_CUDA(cudaGetLastError());
     return DRACO_OK;
 }

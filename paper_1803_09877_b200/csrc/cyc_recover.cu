@@ -30,14 +30,16 @@ __device__ __forceinline__ double magnitude(double a) { return a == a ? fabs(a) 
 // VEC2: a thread owns two neighbouring coordinates, one 16-byte load per row.  Otherwise (odd row starts) two coordinates
 // kThreads apart and two 8-byte loads per row, so that a warp's loads are contiguous and as many bytes are in flight (one
 // coordinate per thread and no batch of rows: n = 45, d = 20,000,001 1589 us with the decode vector, now 1107).
-template <bool VEC2, bool PACKED>
+// ONCE: u may have been written already, beside the projection; the others do without the look (1 % of 1 M coordinates).
+template <bool VEC2, bool PACKED, bool ONCE>
 __global__ void __launch_bounds__(kThreads)
 cyc_recover_kernel(const float2* __restrict__ R, int64_t len, int64_t ld, const CycDevice* __restrict__ cd,
                    DeviceInfo* info, float* __restrict__ u, int64_t d_packed, float* __restrict__ w, float scale) {
     pdl_begin();
     __shared__ double2 bs[kMaxN];
     __shared__ int rows[kMaxN];
-    const int count = info->n_active;
+    const int count = ONCE ? info->combine : info->n_active;
+    if (ONCE && count < 0) return;
     double im_max = 0.0, re_max = 0.0;                    // over this thread's sampled coordinates
     for (int k = threadIdx.x; k < count; k += kThreads) {
         bs[k] = cd->b_active[k];
@@ -255,7 +257,7 @@ cyc_recover_short_kernel(const float2* __restrict__ R, int64_t len, int64_t ld, 
 }  // namespace
 
 int launch_cyc_recover(draco_plan* p, const float2* R, int64_t len, int64_t ld, float* u, int64_t d_packed,
-                       cudaStream_t st, float* w, float scale) {
+                       cudaStream_t st, float* w, float scale, bool once) {
     const bool packed = d_packed > 0;
     // 64-bit stores of u need len even; in packed mode the second half starts at u + len and must cover it fully
     const bool vec2 = (len % 2 == 0) && (ld % 2 == 0) && (!packed || d_packed == 2 * len);
@@ -264,12 +266,16 @@ int launch_cyc_recover(draco_plan* p, const float2* R, int64_t len, int64_t ld, 
     const int64_t cap = (int64_t)p->sm_count * 16;
     if (want > cap) want = cap;
     if (want < 1) want = 1;
-#define DRACO_REC(V2, PK) \
-    launch_dependent(cyc_recover_kernel<V2, PK>, (int)want, kThreads, 0, st, R, len, ld, p->cyc_dev, p->info_dev, u, d_packed, w, scale)
+#define DRACO_REC_ONCE(V2, PK, ONCE) \
+    launch_dependent(cyc_recover_kernel<V2, PK, ONCE>, (int)want, kThreads, 0, st, R, len, ld, p->cyc_dev, p->info_dev, u, d_packed, w, scale)
+#define DRACO_REC(V2, PK)                                                                    \
+    do {                                                                                     \
+        if (once) DRACO_REC_ONCE(V2, PK, true); else DRACO_REC_ONCE(V2, PK, false);          \
+    } while (0)
 #define DRACO_REC_SHORT(V2, PK)                                                                                                    \
     launch_dependent(cyc_recover_short_kernel<V2, PK>, (int)((len + 63) / 64), kThreads, 0, st, R, len, ld, p->cyc_dev, p->info_dev, u, d_packed, w, \
                                                                                   scale)
-    if (len <= (int64_t)p->sm_count * (p->n <= 16 ? kShortFewRows : kShortCoordinates)) {
+    if (!once && len <= (int64_t)p->sm_count * (p->n <= 16 ? kShortFewRows : kShortCoordinates)) {
         if (vec2) {
             if (packed) DRACO_REC_SHORT(true, true); else DRACO_REC_SHORT(true, false);
         } else {
@@ -280,6 +286,7 @@ int launch_cyc_recover(draco_plan* p, const float2* R, int64_t len, int64_t ld, 
     } else {
         if (packed) DRACO_REC(false, true); else DRACO_REC(false, false);
     }
+#undef DRACO_REC_ONCE
 #undef DRACO_REC
 #undef DRACO_REC_SHORT
     DRACO_CUDA(cudaGetLastError());

@@ -138,6 +138,12 @@ namespace {
 // Chunks of G below this (packed plans: of its first half, one of the chunk's two copies) are not split: their kernels take no
 // longer than a launch.
 constexpr int64_t kSplitBytes = (int64_t)2 << 20;
+// Received matrices from this size on are located and decoded with one read: what the read saves has to pay for a run of the locator
+// on the sample, about 25 us.  Packed vectors need twice the fp64 operations per byte for the sum, and half as many coordinates
+// share the additions over the lanes: two reads / one, us: n = 45, s = 5, d = 500 k 83 / 85, 800 k 115 / 108, 1.5 M 193 / 147; n = 15,
+// s = 2, 1 M 59 / 67, 2 M 96 / 89, 4 M 160 / 126; n = 105, s = 2, 200 k 93 / 139, 400 k 147 / 132; packed n = 45, 2 M 126 / 133, 4 M
+// 233 / 192; and 60.2 M 6150 / 3490, packed 3180 / 2150.
+constexpr int64_t kOnePassBytes = (int64_t)256 << 20, kOnePassBytesPacked = (int64_t)512 << 20;
 }
 
 extern "C" {
@@ -169,10 +175,10 @@ int draco_plan_create(int n, int s, int64_t d, int code, draco_plan** out) {
         cudaError_t e__ = (call);                                                \
         if (e__ != cudaSuccess) { free_plan(p); return cuda_fail(e__, #call); }  \
     } while (0)
-    DRACO_TRY(cudaMalloc(&p->info_dev, sizeof(DeviceInfo)));
-    DRACO_TRY(cudaMemset(p->info_dev, 0, sizeof(DeviceInfo)));
-    DRACO_TRY(cudaMalloc(&p->flags_dev, kMaxN));
-    DRACO_TRY(cudaMemset(p->flags_dev, 0, kMaxN));
+    DRACO_TRY(cudaMalloc(&p->info_dev, 2 * sizeof(DeviceInfo)));
+    DRACO_TRY(cudaMemset(p->info_dev, 0, 2 * sizeof(DeviceInfo)));
+    DRACO_TRY(cudaMalloc(&p->flags_dev, 2 * kMaxN));
+    DRACO_TRY(cudaMemset(p->flags_dev, 0, 2 * kMaxN));
     if (code == DRACO_REP) {
         DRACO_TRY(cudaMalloc(&p->mask_dev, rep_scratch_bytes()));
         DRACO_TRY(cudaMemset(p->mask_dev, 0, rep_scratch_bytes()));
@@ -295,10 +301,18 @@ int draco_locate_decode(draco_plan* plan, const void* R, const float* f, uint8_t
         return launch_rep_vote(plan, (const float*)R, plan->d, plan->d, u, nullptr, flags, st);
     // projection, then syndromes / solve / support / decode vector in one launch, then the recovery
     if (!f || !aligned16(f)) return DRACO_EINVAL;
-    int rc = launch_cyc_project(plan, (const float2*)R, f, vec_len(plan), vec_len(plan), false, st);
-    if (rc == DRACO_OK) rc = launch_cyc_solve(plan, nullptr, flags, true, st);
+    const int64_t len = vec_len(plan);
+    const bool once = 8 * plan->n * len >= (is_packed(plan) ? kOnePassBytesPacked : kOnePassBytes);      // the projection and, most probably, the recovery in one
+    int rc;
+    if (once) {
+        rc = launch_cyc_sample(plan, (const float2*)R, f, len, len, st);
+        if (rc == DRACO_OK) rc = launch_cyc_onepass(plan, (const float2*)R, f, len, len, u, is_packed(plan) ? plan->d : 0, st);
+    } else {
+        rc = launch_cyc_project(plan, (const float2*)R, f, len, len, false, st);
+    }
+    if (rc == DRACO_OK) rc = launch_cyc_solve(plan, nullptr, flags, true, st, once);
     if (rc != DRACO_OK) return rc;
-    return launch_cyc_recover(plan, (const float2*)R, vec_len(plan), vec_len(plan), u, is_packed(plan) ? plan->d : 0, st);
+    return launch_cyc_recover(plan, (const float2*)R, len, len, u, is_packed(plan) ? plan->d : 0, st, nullptr, 0.0f, once);
 }
 
 int draco_cyc_decode_vector(draco_plan* plan, double* b_host, void* stream) {

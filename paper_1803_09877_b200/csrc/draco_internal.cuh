@@ -59,6 +59,7 @@ struct DeviceInfo {                   // mirrors draco_info
     double locator_margin;
     unsigned long long im_residual_bits;   // bit patterns of non-negative doubles: they order like integers, so the
     unsigned long long re_max_bits;        // blocks of the recovery kernel merge their maxima with atomicMax
+    int32_t combine;                  // not in draco_info: n_active, or -1: u has been written, the recovery returns at once
 };
 
 }  // namespace draco
@@ -79,11 +80,11 @@ struct draco_plan {
     double2* taps_full_dev;           // generic encoder: fp64 taps for any s, device [2s+1]
     // device scratch
     draco::CycDevice* cyc_dev;
-    draco::DeviceInfo* info_dev;
+    draco::DeviceInfo* info_dev;      // [2]: the plan's, and that of the locator's run on a sample
     double2* partial_dev;             // [project_grid][n]
     int project_grid;                 // capacity of partial_dev in blocks
     int project_used;                 // blocks whose partials the plan's last projection (all its chunks) filled
-    uint8_t* flags_dev;               // [n] internal flags
+    uint8_t* flags_dev;               // [2 kMaxN] internal flags, and those of the sample
     uint32_t* mask_dev;               // repetition: the vote's scratch, zero between calls
     // host-buffer pipeline (allocated on its first call)
     float* stage_dev;                 // two [n][stage_chunk] slices of G (double buffer)
@@ -141,10 +142,15 @@ int launch_cyc_encode(const draco_plan* p, const float* G, float2* Z, int64_t le
 int launch_cyc_project(draco_plan* p, const float2* R, const float* f, int64_t len, int64_t ld, bool accumulate,
                        cudaStream_t st);
 int launch_cyc_project_finish(draco_plan* p, double2* e_out, cudaStream_t st);
-int launch_cyc_solve(draco_plan* p, const double2* e, uint8_t* flags, bool with_b, cudaStream_t st);
+int launch_cyc_sample(draco_plan* p, const float2* R, const float* f, int64_t len, int64_t ld, cudaStream_t st);
+int launch_cyc_onepass(draco_plan* p, const float2* R, const float* f, int64_t len, int64_t ld, float* u, int64_t d_packed,
+                       cudaStream_t st);
+// with_b: the decode vector too; sampled: the flags are compared with those that launch_cyc_sample found
+int launch_cyc_solve(draco_plan* p, const double2* e, uint8_t* flags, bool with_b, cudaStream_t st, bool sampled = false);
 int launch_cyc_decode_vector(draco_plan* p, const uint8_t* flags, cudaStream_t st);
+// once: after launch_cyc_onepass, whose sum stands where the sample's V was the right one
 int launch_cyc_recover(draco_plan* p, const float2* R, int64_t len, int64_t ld, float* u, int64_t d_packed,
-                       cudaStream_t st, float* w = nullptr, float scale = 0.0f);
+                       cudaStream_t st, float* w = nullptr, float scale = 0.0f, bool once = false);
 int launch_generate(float* out, int rows, int64_t len, int64_t ld, int64_t i0, int row0, float mean, float std,
                     uint64_t seed, cudaStream_t st);
 int launch_corrupt(float* R, int64_t row_pitch, int64_t nvals, int64_t v0, const int* node, const int* model,

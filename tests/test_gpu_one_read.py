@@ -1,0 +1,90 @@
+"""locate_decode of matrices large enough to be read once (a sample of the columns gives a provisional V, one pass projects and
+combines, the whole projection decides) against the separate locate and decode calls and the fp64 sum of the gradients."""
+import pytest
+import torch
+
+pytestmark = pytest.mark.gpu
+
+# just above the size from which on one read is tried; rows on and off the 16-byte grid, ragged last chunks, few and many rows
+SHAPES = [("CYC", 15, 2, 2_240_000), ("CYC", 15, 2, 2_240_003), ("CYC", 3, 1, 11_300_130), ("CYC", 45, 5, 746_002), ("CYC", 45, 3, 746_001),
+          ("CYC", 105, 2, 320_300), ("CYC", 128, 1, 263_001), ("CYC_PACKED", 15, 2, 8_960_008), ("CYC_PACKED", 45, 3, 2_984_003),
+          ("CYC_PACKED", 45, 3, 2_984_130)]
+
+
+def _setup(code, n, s, d, seed):
+    import paper_1803_09877_b200 as dr
+    plan = dr.Plan(n, s, d, getattr(dr, code))
+    v = (d + 1) // 2 if code == "CYC_PACKED" else d
+    gen = torch.Generator(device="cuda").manual_seed(seed)
+    G = torch.empty((n, d), dtype=torch.float32, device="cuda").normal_(generator=gen)
+    Z = torch.empty((n, 2 * v), dtype=torch.float32, device="cuda")
+    plan.encode(G, Z)
+    f = torch.randn(v, generator=gen, device="cuda") + 1.0
+    nodes = torch.randperm(n, generator=torch.Generator().manual_seed(seed))[:s].sort().values.tolist()
+    return dr, plan, G, Z, f, nodes, v
+
+
+def _same(u, u2):
+    """Both sum in fp64 and round once: an entry may fall on either side of a rounding boundary, 2^-23 of it."""
+    return bool(((u - u2).abs() <= 2.0 ** -23 * u2.abs() + 1e-12 * u2.abs().max()).all())
+
+
+@pytest.mark.parametrize("code,n,s,d", SHAPES)
+# "hidden": adversaries that alter one coordinate only, which the sample does not hold; "nan": the same with NaN
+@pytest.mark.parametrize("attack", ["none", "all", "hidden", "nan"])
+def test_one_read_is_the_separate_calls(code, n, s, d, attack):
+    dr, plan, G, Z, f, nodes, v = _setup(code, n, s, d, 11 * n + s)
+    if attack == "none":
+        nodes = []
+    elif attack == "all":
+        plan.corrupt(Z, nodes, [dr.ADV_REVGRAD] * s, [100.0] * s)
+    else:
+        Z[nodes, 2 * v - 2] = 1e9 if attack == "hidden" else float("nan")
+    flags = torch.full((n,), 7, dtype=torch.uint8, device="cuda")
+    buf = torch.full((d + 64,), 7.0, dtype=torch.float32, device="cuda")
+    u = buf[32:32 + d]
+    plan.locate_decode(Z, f, flags, u)
+    info, b = plan.info(), plan.cyc_decode_vector()
+    assert torch.nonzero(flags).flatten().tolist() == nodes
+    assert (buf[:32] == 7.0).all() and (buf[32 + d:] == 7.0).all()
+    other = dr.Plan(n, s, d, plan.code)
+    flags2, u2 = torch.empty_like(flags), torch.empty(d, dtype=torch.float32, device="cuda")
+    other.locate(Z, f, flags2)
+    other.decode(Z, flags2, u2)
+    info2 = other.info()
+    assert torch.equal(flags, flags2) and abs(b - other.cyc_decode_vector()).max() == 0.0
+    assert _same(u, u2)
+    for key in ("status", "n_flagged", "locator_rank", "n_active", "svd_sweeps"):
+        assert info[key] == info2[key]
+    # the same coordinates, whose imaginary parts are rounding residue of one size
+    assert abs(info["re_max"] - info2["re_max"]) <= 1e-9 * info2["re_max"]
+    assert abs(info["im_residual"] - info2["im_residual"]) <= 1e-6 * info2["re_max"]
+    plan.decode(Z, None, u2)                                # the plan goes on as after any locate
+    assert _same(u, u2)
+    if n == 15:
+        sums = G.double().sum(0)
+        assert float((u.double() - sums).abs().max() / sums.abs().max()) <= 1e-5
+
+
+def test_one_read_replays_from_a_graph_with_other_adversaries():
+    code, n, s, d = "CYC", 15, 2, 2_240_000
+    dr, plan, G, Z, f, _, v = _setup(code, n, s, d, 5)
+    flags = torch.zeros(n, dtype=torch.uint8, device="cuda")
+    u, R = torch.zeros(d, dtype=torch.float32, device="cuda"), Z.clone()
+    plan.locate_decode(R, f, flags, u)
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        plan.locate_decode(R, f, flags, u)
+    sums = G.double().sum(0)
+    for nodes, hidden in (([3, 9], False), ([], False), ([0, 14], True), ([7], False)):
+        R.copy_(Z)
+        if hidden:
+            R[nodes, 2 * v - 1] = 1e9
+        elif nodes:
+            plan.corrupt(R, nodes, [dr.ADV_CONST] * len(nodes), [1e4] * len(nodes))
+        u.zero_()
+        graph.replay()
+        torch.cuda.synchronize()
+        assert torch.nonzero(flags).flatten().tolist() == nodes
+        assert float((u.double() - sums).abs().max() / sums.abs().max()) <= 1e-5
