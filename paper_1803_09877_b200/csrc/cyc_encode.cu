@@ -90,6 +90,87 @@ struct Window {
     double cw[StreamCfg<S, PACKED>::NBIG][4];              // fp64 copies of the rows under the centre taps
 };
 
+// One output z_j of a thread's coordinates, rotated and stored: win[(P - t) mod SL] = row (j - t) mod n, cw its fp64 copies.
+template <int S, int P, bool PACKED, bool REALC>
+__device__ __forceinline__ void encode_output(const Window<S, PACKED>& w, const double2 rot, float2* dst, bool act0, bool act1,
+                                              const EncodeTaps& taps, const EncodeTaps64& taps64) {
+    using Cfg = StreamCfg<S, PACKED>;
+    constexpr int R = Cfg::R, NBIG = Cfg::NBIG, H = Cfg::H, SL = Cfg::SL;
+    float ar[4] = {0.f, 0.f, 0.f, 0.f}, ai[4] = {0.f, 0.f, 0.f, 0.f};
+    // taps grow towards the middle of the filter: add the outer (small) terms first so the
+    // running sums stay small while most of the fp32 roundings happen
+#pragma unroll
+    for (int k = 0; k < R; ++k) {
+        const int t = (k & 1) ? 2 * S - (k >> 1) : (k >> 1);
+        if (t >= S - H && t <= S + H) continue;
+        const float4 g = w.win[(P - t + 2 * SL) % SL];
+        const float cr = taps.tap[t].x, ci = taps.tap[t].y;
+        ar[0] = fmaf(cr, g.x, ar[0]); ai[0] = fmaf(ci, g.x, ai[0]);
+        ar[1] = fmaf(cr, g.y, ar[1]); ai[1] = fmaf(ci, g.y, ai[1]);
+        ar[2] = fmaf(cr, g.z, ar[2]); ai[2] = fmaf(ci, g.z, ai[2]);
+        ar[3] = fmaf(cr, g.w, ar[3]); ai[3] = fmaf(ci, g.w, ai[3]);
+    }
+    constexpr bool kJoin = PACKED && S > 0;          // the two halves' sums are joined before the rotation
+    constexpr int NOUT = kJoin ? 2 : 4;              // rotations of this thread
+    double dr[NOUT], di[NOUT];
+    if constexpr (kJoin) {
+        // components 0, 1 of a row are the real parts of two complex coordinates, 2, 3 their imaginary parts
+#pragma unroll
+        for (int c = 0; c < 2; ++c) {
+            dr[c] = S > H ? (double)ar[c] - (double)ai[c + 2] : 0.0;
+            di[c] = S > H ? (double)ai[c] + (double)ar[c + 2] : 0.0;
+        }
+#pragma unroll
+        for (int k = 0; k < NBIG; ++k) {
+            const int t = (k & 1) ? S + H - (k >> 1) : S - H + (k >> 1);
+            const double cr = taps64.tap[t].x, ci = taps64.tap[t].y;
+            const double(&g)[4] = w.cw[((P - t + 2 * SL) % SL) % NBIG];
+#pragma unroll
+            for (int c = 0; c < 2; ++c) {
+                dr[c] = fma(cr, g[c], dr[c]);
+                di[c] = fma(cr, g[c + 2], di[c]);
+                if (t != S) {                        // the centre tap is real
+                    dr[c] = fma(-ci, g[c + 2], dr[c]);
+                    di[c] = fma(ci, g[c], di[c]);
+                }
+            }
+        }
+    } else {
+#pragma unroll
+        for (int c = 0; c < 4; ++c) { dr[c] = (double)ar[c]; di[c] = (double)ai[c]; }
+#pragma unroll
+        for (int t = S - H; t <= S + H; ++t) {
+            const int q = ((P - t + 2 * SL) % SL) % NBIG;
+            const double cr = taps64.tap[t].x, ci = taps64.tap[t].y;
+#pragma unroll
+            for (int c = 0; c < 4; ++c) {
+                dr[c] = fma(cr, w.cw[q][c], dr[c]);
+                if (!REALC || t != S) di[c] = fma(ci, w.cw[q][c], di[c]);
+            }
+        }
+    }
+    double xr[NOUT], xi[NOUT];
+#pragma unroll
+    for (int c = 0; c < NOUT; ++c) {
+        xr[c] = fma(dr[c], rot.x, -di[c] * rot.y);
+        xi[c] = fma(dr[c], rot.y, di[c] * rot.x);
+    }
+    if constexpr (kJoin) {
+        if (act0) __stcs(reinterpret_cast<float4*>(dst), make_float4((float)xr[0], (float)xi[0], (float)xr[1], (float)xi[1]));
+    } else if constexpr (PACKED) {
+        // components 0, 1 filtered the real parts (X), 2, 3 the imaginary parts (Y): z = X + i Y
+        if (act0)
+            __stcs(reinterpret_cast<float4*>(dst), make_float4((float)(xr[0] - xi[2]), (float)(xi[0] + xr[2]),
+                                                               (float)(xr[1] - xi[3]), (float)(xi[1] + xr[3])));
+    } else {
+        // A lane's two 16-byte stores are 512 bytes apart, so that each store instruction of the warp
+        // covers 512 contiguous bytes (whole 32-byte sectors).  With the 4 coordinates of a lane adjacent,
+        // every instruction wrote half of 32 sectors and the kernel stopped at 4.9 TB/s.
+        if (act0) __stcs(reinterpret_cast<float4*>(dst), make_float4((float)xr[0], (float)xi[0], (float)xr[1], (float)xi[1]));
+        if (act1) __stcs(reinterpret_cast<float4*>(dst + 64), make_float4((float)xr[2], (float)xi[2], (float)xr[3], (float)xi[3]));
+    }
+}
+
 // The fetch side: the rows of this warp's strips, one after the other, kRing rows ahead of the row being
 // consumed.  A lane copies coordinates 2l, 2l+1 and 64+2l, 64+2l+1 of the strip (packed: complex
 // coordinates 2l, 2l+1, real parts from G[r][c], imaginary parts from G[r][half + c]).
@@ -143,7 +224,7 @@ __device__ __forceinline__ void encode_step(Window<S, PACKED>& w, Cursor& cur, F
                                             const EncodeTaps& taps, const EncodeTaps64& taps64,
                                             const EncodePhase64& ph64) {
     using Cfg = StreamCfg<S, PACKED>;
-    constexpr int R = Cfg::R, NBIG = Cfg::NBIG, H = Cfg::H, SL = Cfg::SL;
+    constexpr int NBIG = Cfg::NBIG, H = Cfg::H, SL = Cfg::SL;
     constexpr uint32_t kRowBytes = Cfg::kRowBytes;
     const int total = n + 2 * S;
     if (MODE == 2 && vv >= total) return;
@@ -168,66 +249,6 @@ __device__ __forceinline__ void encode_step(Window<S, PACKED>& w, Cursor& cur, F
     if (emit) {
         // win[(P - t) mod SL] = row (vv - t) mod n: this output is z_j, j = vv mod n
         const int j = (MODE == 2 && vv >= n) ? vv - n : vv;
-        float ar[4] = {0.f, 0.f, 0.f, 0.f}, ai[4] = {0.f, 0.f, 0.f, 0.f};
-        // taps grow towards the middle of the filter: add the outer (small) terms first so the
-        // running sums stay small while most of the fp32 roundings happen
-#pragma unroll
-        for (int k = 0; k < R; ++k) {
-            const int t = (k & 1) ? 2 * S - (k >> 1) : (k >> 1);
-            if (t >= S - H && t <= S + H) continue;
-            const float4 g = w.win[(P - t + 2 * SL) % SL];
-            const float cr = taps.tap[t].x, ci = taps.tap[t].y;
-            ar[0] = fmaf(cr, g.x, ar[0]); ai[0] = fmaf(ci, g.x, ai[0]);
-            ar[1] = fmaf(cr, g.y, ar[1]); ai[1] = fmaf(ci, g.y, ai[1]);
-            ar[2] = fmaf(cr, g.z, ar[2]); ai[2] = fmaf(ci, g.z, ai[2]);
-            ar[3] = fmaf(cr, g.w, ar[3]); ai[3] = fmaf(ci, g.w, ai[3]);
-        }
-        constexpr bool kJoin = PACKED && S > 0;          // the two halves' sums are joined before the rotation
-        constexpr int NOUT = kJoin ? 2 : 4;              // rotations of this thread
-        double dr[NOUT], di[NOUT];
-        if constexpr (kJoin) {
-            // components 0, 1 of a row are the real parts of two complex coordinates, 2, 3 their imaginary parts
-#pragma unroll
-            for (int c = 0; c < 2; ++c) {
-                dr[c] = S > H ? (double)ar[c] - (double)ai[c + 2] : 0.0;
-                di[c] = S > H ? (double)ai[c] + (double)ar[c + 2] : 0.0;
-            }
-#pragma unroll
-            for (int k = 0; k < NBIG; ++k) {
-                const int t = (k & 1) ? S + H - (k >> 1) : S - H + (k >> 1);
-                const double cr = taps64.tap[t].x, ci = taps64.tap[t].y;
-                const double(&g)[4] = w.cw[((P - t + 2 * SL) % SL) % NBIG];
-#pragma unroll
-                for (int c = 0; c < 2; ++c) {
-                    dr[c] = fma(cr, g[c], dr[c]);
-                    di[c] = fma(cr, g[c + 2], di[c]);
-                    if (t != S) {                        // the centre tap is real
-                        dr[c] = fma(-ci, g[c + 2], dr[c]);
-                        di[c] = fma(ci, g[c], di[c]);
-                    }
-                }
-            }
-        } else {
-#pragma unroll
-            for (int c = 0; c < 4; ++c) { dr[c] = (double)ar[c]; di[c] = (double)ai[c]; }
-#pragma unroll
-            for (int t = S - H; t <= S + H; ++t) {
-                const int q = ((P - t + 2 * SL) % SL) % NBIG;
-                const double cr = taps64.tap[t].x, ci = taps64.tap[t].y;
-#pragma unroll
-                for (int c = 0; c < 4; ++c) {
-                    dr[c] = fma(cr, w.cw[q][c], dr[c]);
-                    if (!REALC || t != S) di[c] = fma(ci, w.cw[q][c], di[c]);
-                }
-            }
-        }
-        const double2 rot = ph64.phase[j];
-        double xr[NOUT], xi[NOUT];
-#pragma unroll
-        for (int c = 0; c < NOUT; ++c) {
-            xr[c] = fma(dr[c], rot.x, -di[c] * rot.y);
-            xi[c] = fma(dr[c], rot.y, di[c] * rot.x);
-        }
         float2* dst;
         if (MODE == 2) {
             dst = zcol + (int64_t)j * ldz;
@@ -235,20 +256,7 @@ __device__ __forceinline__ void encode_step(Window<S, PACKED>& w, Cursor& cur, F
             dst = cur.zout;
             cur.zout += ldz;
         }
-        if constexpr (kJoin) {
-            if (act0) __stcs(reinterpret_cast<float4*>(dst), make_float4((float)xr[0], (float)xi[0], (float)xr[1], (float)xi[1]));
-        } else if constexpr (PACKED) {
-            // components 0, 1 filtered the real parts (X), 2, 3 the imaginary parts (Y): z = X + i Y
-            if (act0)
-                __stcs(reinterpret_cast<float4*>(dst), make_float4((float)(xr[0] - xi[2]), (float)(xi[0] + xr[2]),
-                                                                   (float)(xr[1] - xi[3]), (float)(xi[1] + xr[3])));
-        } else {
-            // A lane's two 16-byte stores are 512 bytes apart, so that each store instruction of the warp
-            // covers 512 contiguous bytes (whole 32-byte sectors).  With the 4 coordinates of a lane adjacent,
-            // every instruction wrote half of 32 sectors and the kernel stopped at 4.9 TB/s.
-            if (act0) __stcs(reinterpret_cast<float4*>(dst), make_float4((float)xr[0], (float)xi[0], (float)xr[1], (float)xi[1]));
-            if (act1) __stcs(reinterpret_cast<float4*>(dst + 64), make_float4((float)xr[2], (float)xi[2], (float)xr[3], (float)xi[3]));
-        }
+        encode_output<S, P, PACKED, REALC>(w, ph64.phase[j], dst, act0, act1, taps, taps64);
     }
     if (from_ring) {
         // The slot just consumed is refilled with the row kRing ahead.  Its read has completed by then: the stash
@@ -318,6 +326,50 @@ cyc_encode_stream_kernel(const float* __restrict__ G, float2* __restrict__ Z, in
             encode_chunk<S, 2, PACKED, REALC>(w, cur, f, v0, n, ldz, stash0, zcol, act0, act1, taps, taps64, ph64);
     }
     cp_async_wait<0>();
+}
+
+// The same for short vectors, where a warp's walk over all rows is a chain of latencies: a warp computes J outputs of its strip and
+// loads their 2 s + J rows at once; the others' rows are re-read through L2.  The same operations on every entry, hence the same bits.
+constexpr int kShortWarps = 4;
+template <int S, bool PACKED, bool REALC, int J>
+__global__ void __launch_bounds__(32 * kShortWarps)
+cyc_encode_short_kernel(const float* __restrict__ G, float2* __restrict__ Z, int64_t len, int64_t ldg, int64_t ldz, int64_t half,
+                        int n, const __grid_constant__ EncodeTaps taps, const __grid_constant__ EncodeTaps64 taps64,
+                        const __grid_constant__ EncodePhase64 ph64) {
+    pdl_begin();
+    using Cfg = StreamCfg<S, PACKED>;
+    constexpr int NBIG = Cfg::NBIG, H = Cfg::H, SL = Cfg::SL, kStrip = PACKED ? 64 : 128;
+    const int64_t c = ((int64_t)blockIdx.x * kShortWarps + (threadIdx.x >> 5)) * kStrip + 2 * (threadIdx.x & 31);
+    const bool act0 = c < len, act1 = PACKED ? act0 : c + 64 < len;
+    if (!act0) return;
+    const int j0 = (int)blockIdx.y * J;
+    const float* g = G + c;
+    const int64_t second = PACKED ? half : act1 ? 64 : 0;
+    float4 x[2 * S + J];
+#pragma unroll
+    for (int q = 0; q < 2 * S + J; ++q) {
+        int r = j0 + q - 2 * S;
+        r = r < 0 ? r + n : r < n ? r : n - 1;             // rows past the last output's are not used
+        const float2 a = *reinterpret_cast<const float2*>(g + (int64_t)r * ldg), b = *reinterpret_cast<const float2*>(g + (int64_t)r * ldg + second);
+        x[q] = make_float4(a.x, a.y, b.x, b.y);
+    }
+#pragma unroll
+    for (int k = 0; k < J; ++k) {
+        if (j0 + k < n) {
+            constexpr int P = 2 * S;
+            Window<S, PACKED> w;
+#pragma unroll
+            for (int q = 0; q < SL; ++q) w.win[q] = x[k + (q < 2 * S ? q : 2 * S)];
+#pragma unroll
+            for (int q = S - H; q <= S + H; ++q) {
+                w.cw[q % NBIG][0] = (double)x[k + q].x;
+                w.cw[q % NBIG][1] = (double)x[k + q].y;
+                w.cw[q % NBIG][2] = (double)x[k + q].z;
+                w.cw[q % NBIG][3] = (double)x[k + q].w;
+            }
+            encode_output<S, P, PACKED, REALC>(w, ph64.phase[j0 + k], Z + (int64_t)(j0 + k) * ldz + c, act0, act1, taps, taps64);
+        }
+    }
 }
 
 // Rows of any alignment and length, 1 <= s <= 7: the same walk with two coordinates kThreads apart (packed: one complex
@@ -469,6 +521,58 @@ cyc_encode_fir_kernel(const float* __restrict__ G, float2* __restrict__ Z, int64
     }
 }
 
+// The same for short vectors: a thread computes J outputs of its coordinates from rows that it loads at once (the same bits).
+template <int S, bool PACKED, int J>
+__global__ void __launch_bounds__(FirCfg<S, PACKED>::kThreads)
+cyc_encode_fir_short_kernel(const float* __restrict__ G, float2* __restrict__ Z, int64_t len, int64_t ldg, int64_t ldz, int64_t half,
+                            int64_t d_real, int n, const __grid_constant__ EncodeTaps64 taps, const __grid_constant__ EncodePhase64 ph) {
+    pdl_begin();
+    using Cfg = FirCfg<S, PACKED>;
+    constexpr int C = Cfg::C, NI = Cfg::NI, kT = Cfg::kThreads;
+    const int64_t c = (int64_t)blockIdx.x * (kT * C) + threadIdx.x;
+    if (c >= len) return;
+    const bool on1 = PACKED ? half + c < d_real : c + kT < len;
+    const int64_t off1 = !on1 ? 0 : PACKED ? half : kT;
+    const int j0 = (int)blockIdx.y * J;
+    float x[2 * S + J][NI];
+#pragma unroll
+    for (int q = 0; q < 2 * S + J; ++q) {
+        int r = j0 + q - 2 * S;
+        r = r < 0 ? r + n : r < n ? r : n - 1;             // rows past the last output's are not used
+        x[q][0] = G[(int64_t)r * ldg + c];
+        x[q][1] = G[(int64_t)r * ldg + c + off1];
+        if (!on1) x[q][1] = 0.0f;
+    }
+#pragma unroll
+    for (int k = 0; k < J; ++k) {
+        if (j0 + k < n) {
+            double ar[C], ai[C];
+#pragma unroll
+            for (int q = 0; q < C; ++q) ar[q] = ai[q] = 0.0;
+#pragma unroll
+            for (int i = 0; i <= 2 * S; ++i) {
+                const int t = (i & 1) ? 2 * S - (i >> 1) : (i >> 1);       // small taps first, as in fir_step
+                const double cr = taps.tap[t].x, ci = taps.tap[t].y;
+                const double y[NI] = {(double)x[k + 2 * S - t][0], (double)x[k + 2 * S - t][1]};
+#pragma unroll
+                for (int q = 0; q < C; ++q) {
+                    ar[q] = fma(cr, y[q], ar[q]);
+                    if (t != S) ai[q] = fma(ci, y[q], ai[q]);
+                }
+                if constexpr (PACKED) {
+                    if (t != S) ar[0] = fma(-ci, y[1], ar[0]);
+                    ai[0] = fma(cr, y[1], ai[0]);
+                }
+            }
+            const double2 rot = ph.phase[j0 + k];
+#pragma unroll
+            for (int q = 0; q < C; ++q)
+                if (q == 0 || on1)
+                    Z[(int64_t)(j0 + k) * ldz + c + q * kT] = make_float2((float)fma(ar[q], rot.x, -ai[q] * rot.y), (float)fma(ar[q], rot.y, ai[q] * rot.x));
+        }
+    }
+}
+
 // s = 0 off the streaming kernel's alignment, s > 7: one coordinate per thread, rows re-read through the caches,
 // fp64 taps and fp64 accumulation throughout (a tap rounded to fp32 is a fixed error of 2^-24 |tap| that
 // the decoder's cancellation amplifies like any other).  half > 0: packed mode (len complex coordinates; the imaginary
@@ -504,11 +608,33 @@ cyc_encode_generic_kernel(const float* __restrict__ G, float2* __restrict__ Z, i
     }
 }
 
+// Outputs per thread of the short kernels, 0: the walking kernels.  warps: what one output row takes.  One output each while that gives
+// an SM no more than 16 warps (n = 45, d = 4096), else four, up to 600 warps of outputs per SM on aligned rows, 300 (most) off the
+// grid, where the others catch up.  Walking / one / four outputs, us, the caller's 3.4 a call included: n = 45, s = 5, d = 4096 22.0 /
+// 3.4 / 3.4, 30,000 22.5 / 5.9 / 6.2, 100,000 22.5 / 15 / 11.4, 200,000 (630 warps) 22.7 / 30 / 21.3; n = 15, s = 2, 60,000 9.3 / 3.8 / 5.9,
+// 200,000 9.5 / 7.8 / 7.1; n = 105, s = 3, 100,000 (550) 40 / 28 / 22.5, 200,000 42 / 59 / 45; packed n = 45, s = 5, 120,000 22 / 18 / 12;
+// off the grid n = 45, s = 5, 30,003 (140) 14.9 / 8.9 / 6.5, 60,003 (290) 15.7 / 16 / 11.3, 100,003 (480) 16.8 / 26 / 17.5.
+int short_outputs(const draco_plan* p, int64_t warps, int64_t most) {
+    const int64_t all = warps * p->n, sms = p->sm_count;
+    return all <= 16 * sms ? 1 : all <= most * sms ? 4 : 0;
+}
+
 template <int S, bool PACKED, bool REALC = true>
 int launch_stream(const draco_plan* p, const float* G, float2* Z, int64_t len, int64_t ldg, int64_t ldz, int64_t half,
                   cudaStream_t st) {
     using Cfg = StreamCfg<S, PACKED>;
     constexpr int kThreads = Cfg::kThreads;
+    constexpr int kStrip = PACKED ? 64 : 128;
+    const int64_t nstrips = (len + kStrip - 1) / kStrip;
+    const int outputs = short_outputs(p, nstrips, 600);
+    if (outputs > 0) {
+#define DRACO_SHORT(J) launch_dependent(cyc_encode_short_kernel<S, PACKED, REALC, J>, dim3((unsigned)((nstrips + kShortWarps - 1) / kShortWarps), (unsigned)((p->n + J - 1) / J)), \
+                                        32 * kShortWarps, 0, st, G, Z, len, ldg, ldz, half, p->n, p->taps, p->taps64, p->phase64)
+        if (outputs == 1) DRACO_SHORT(1); else DRACO_SHORT(4);
+#undef DRACO_SHORT
+        DRACO_CUDA(cudaGetLastError());
+        return DRACO_OK;
+    }
     auto kern = cyc_encode_stream_kernel<S, PACKED, REALC>;
     static bool configured[64] = {};
     int dev = p->device;
@@ -520,8 +646,6 @@ int launch_stream(const draco_plan* p, const float* G, float2* Z, int64_t len, i
     int per_sm = 1;
     DRACO_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kThreads, Cfg::kSmem));
     if (per_sm < 1) per_sm = 1;
-    constexpr int kStrip = PACKED ? 64 : 128;
-    const int64_t nstrips = (len + kStrip - 1) / kStrip;
     const int64_t nblocks = (nstrips + kThreads / 32 - 1) / (kThreads / 32);
     int64_t grid = (int64_t)p->sm_count * per_sm;
     if (grid > nblocks) grid = nblocks;
@@ -555,6 +679,17 @@ template <int S, bool PACKED>
 int launch_fir(const draco_plan* p, const float* G, float2* Z, int64_t len, int64_t ldg, int64_t ldz, int64_t half,
                int64_t d_real, cudaStream_t st) {
     using Cfg = FirCfg<S, PACKED>;
+    constexpr int kPer = Cfg::kThreads * Cfg::C;
+    const int64_t nshort = (len + kPer - 1) / kPer;
+    const int outputs = short_outputs(p, nshort * (Cfg::kThreads / 32), 300);
+    if (outputs > 0) {
+#define DRACO_SHORT(J) launch_dependent(cyc_encode_fir_short_kernel<S, PACKED, J>, dim3((unsigned)nshort, (unsigned)((p->n + J - 1) / J)), Cfg::kThreads, 0, st, G, Z, len, ldg, ldz, \
+                                        half, d_real, p->n, p->taps64, p->phase64)
+        if (outputs == 1) DRACO_SHORT(1); else DRACO_SHORT(4);
+#undef DRACO_SHORT
+        DRACO_CUDA(cudaGetLastError());
+        return DRACO_OK;
+    }
     const int64_t nstrips = (len + Cfg::kTile - 1) / Cfg::kTile;
     int64_t grid = (int64_t)p->sm_count * Cfg::kBlocks;
     if (grid > nstrips) grid = nstrips;

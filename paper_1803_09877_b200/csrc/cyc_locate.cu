@@ -895,9 +895,9 @@ __device__ void decode_vector_body(CycDevice* cd, const uint8_t* fl, const doubl
     const int a = list_flagged(fl, n, vlist, bits);
     if (a > 2 * s) {                                       // fewer than n - 2 s rows left: no b exists
         if (tid < n) cd->b[tid] = make_double2(0.0, 0.0);
-        if (tid == kSolveThreads - 1) {
+        if (tid == 0) {
             info->n_active = 0; info->n_flagged = a; info->status = DRACO_ETOOMANY;
-            info->im_residual_bits = 0ull; info->re_max_bits = 0ull; info->combine = 0;
+            info->im_residual_bits = 0ull; info->re_max_bits = 0ull;
         }
         return;
     }
@@ -992,7 +992,6 @@ __device__ void decode_vector_body(CycDevice* cd, const uint8_t* fl, const doubl
         info->n_flagged = a;
         info->im_residual_bits = 0ull;                     // the recovery kernel's blocks merge their maxima into these
         info->re_max_bits = 0ull;
-        info->combine = n - a;
         if (info->status == DRACO_ETOOMANY) info->status = DRACO_OK;
     }
 }
@@ -1339,10 +1338,13 @@ cyc_solve_kernel(CycDevice* cd, const double2* __restrict__ e_in, const double2*
         decode_vector_body(cd, fl_s, tw, n, s, mod, rsn, info);
         if (sample != nullptr) {                           // u has been written for the sample's V, if that was beyond doubt
             const int differ = __syncthreads_count(tid < n && fl_s[tid] != sample_flags[tid]);
-            if (tid == kSolveThreads - 1 && differ == 0 && sample->status == DRACO_OK) {
-                info->im_residual_bits = sample->im_residual_bits;
-                info->re_max_bits = sample->re_max_bits;
-                info->combine = -1;
+            if (tid == kSolveThreads - 1) {
+                info->combine = info->n_active;
+                if (differ == 0 && sample->status == DRACO_OK) {
+                    info->im_residual_bits = sample->im_residual_bits;
+                    info->re_max_bits = sample->re_max_bits;
+                    info->combine = -1;
+                }
             }
         }
     }

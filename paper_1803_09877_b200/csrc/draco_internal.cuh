@@ -59,7 +59,7 @@ struct DeviceInfo {                   // mirrors draco_info
     double locator_margin;
     unsigned long long im_residual_bits;   // bit patterns of non-negative doubles: they order like integers, so the
     unsigned long long re_max_bits;        // blocks of the recovery kernel merge their maxima with atomicMax
-    int32_t combine;                  // not in draco_info: n_active, or -1: u has been written, the recovery returns at once
+    int32_t combine;                  // not in draco_info, set after a sample: n_active, or -1: u has been written already
 };
 
 }  // namespace draco
