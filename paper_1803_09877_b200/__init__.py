@@ -3,7 +3,7 @@
 decoding for the repetition and cyclic codes.
 
 The work is done by hand-written CUDA kernels behind a C ABI (``include/draco.h``,
-``libdraco.so``); this package is a thin ctypes binding with the same names.
+``libdraco.so``); this package is a thin binding with the same names.
 There is no CPU fallback: the first use of any name below loads ``libdraco.so``
 and raises if it has not been built (``python -m paper_1803_09877_b200.build``).
 The ``build`` submodule itself imports without the library.

@@ -1,4 +1,4 @@
-"""ctypes binding of libdraco.so: argument marshalling only.
+"""Binding of libdraco.so: argument marshalling only, by ctypes, and natively (``csrc/native.cpp``) for the calls of a training loop.
 
 Every function takes raw device pointers (``tensor.data_ptr()``) or torch
 tensors and a CUDA stream handle; PyTorch is used by callers for device memory
@@ -105,6 +105,7 @@ def _find_current_stream():
     first = torch.cuda.current_stream().cuda_stream        # also sets CUDA up
     raw, device = getattr(torch._C, "_cuda_getCurrentRawStream", None), getattr(torch._C, "_cuda_getDevice", None)
     if raw and device:
+        _native.set_current_stream(raw, device)
         _current_stream = lambda: raw(device())
     else:
         _current_stream = lambda: torch.cuda.current_stream().cuda_stream
@@ -120,6 +121,18 @@ def _stream(stream):
     if isinstance(stream, int):
         return stream
     return stream.cuda_stream
+
+
+def _load_native():
+    try:
+        from . import _native as module
+    except ImportError as e:
+        raise DracoError(f"{_PKG}/_native.so cannot be loaded: build it with `python -m paper_1803_09877_b200.build`") from e
+    module.set_functions(_check, _stream)
+    return module
+
+
+_native = _load_native()
 
 
 def _adv_arrays(adv_idx, adv_model, adv_param):
@@ -147,11 +160,13 @@ class Plan:
         h = _vp()
         _check(lib.draco_plan_create(n, s, d, code, C.byref(h)))
         self._h = h
+        self._address = h.value
 
     def close(self):
         if getattr(self, "_h", None):
             lib.draco_plan_destroy(self._h)
             self._h = None
+            self._address = None
 
     __del__ = close
 
@@ -173,19 +188,19 @@ class Plan:
         return a[..., 0] + 1j * a[..., 1]
 
     def encode(self, G, Z, stream=None):
-        return _check(lib.draco_encode(self._h, _ptr(G), _ptr(Z), _stream(stream)))
+        return _native.encode(self._address, G, Z, stream)
 
     def locate(self, R, f, flags, stream=None):
-        return _check(lib.draco_locate(self._h, _ptr(R), _ptr(f), _ptr(flags), _stream(stream)))
+        return _native.locate(self._address, R, f, flags, stream)
 
     def decode(self, R, flags, u, stream=None):
-        return _check(lib.draco_decode(self._h, _ptr(R), _ptr(flags), _ptr(u), _stream(stream)))
+        return _native.decode(self._address, R, flags, u, stream)
 
     def decode_update(self, R, flags, w, scale: float, stream=None):
-        return _check(lib.draco_decode_update(self._h, _ptr(R), _ptr(flags), _ptr(w), scale, _stream(stream)))
+        return _native.decode_update(self._address, R, flags, w, scale, stream)
 
     def locate_decode(self, R, f, flags, u, stream=None):
-        return _check(lib.draco_locate_decode(self._h, _ptr(R), _ptr(f), _ptr(flags), _ptr(u), _stream(stream)))
+        return _native.locate_decode(self._address, R, f, flags, u, stream)
 
     def rep_vote(self, R, u=None, maj=None, flags=None, stream=None):
         return _check(lib.draco_rep_vote(self._h, _ptr(R), _ptr(u), _ptr(maj), _ptr(flags), _stream(stream)))

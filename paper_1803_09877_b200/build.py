@@ -5,6 +5,7 @@ import os
 import shutil
 import subprocess
 import sys
+import sysconfig
 from concurrent.futures import ThreadPoolExecutor
 
 PKG = os.path.dirname(os.path.abspath(__file__))
@@ -13,6 +14,7 @@ CSRC = os.path.join(PKG, "csrc")
 INCLUDE = os.path.join(ROOT, "include")
 OBJ = os.path.join(PKG, "_build")
 LIB = os.path.join(PKG, "libdraco.so")
+NATIVE = os.path.join(PKG, "_native.so")          # the CPython module of the calls that a training loop makes
 
 SOURCES = ["draco_api.cu", "rep_kernels.cu", "cyc_encode.cu", "cyc_locate.cu", "cyc_onepass.cu", "cyc_recover.cu", "harness_kernels.cu"]
 NVCC_FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
@@ -59,6 +61,10 @@ def build(force: bool = False, verbose: bool = False) -> str:
     objs = [os.path.join(OBJ, s.replace(".cu", ".o")) for s in SOURCES]
     if force or jobs or _stale(LIB, objs):
         run([nvcc, "-shared", "-o", LIB] + objs + ["-lcudart"])
+    src = os.path.join(CSRC, "native.cpp")
+    if force or _stale(NATIVE, [src, headers[0]]):
+        run([nvcc, "-shared", "-O3", "-std=c++17", "-Xcompiler", "-fPIC", "-I", INCLUDE, "-I", sysconfig.get_paths()["include"], src,
+             "-o", NATIVE, "-L", PKG, "-Xlinker", "-l:libdraco.so", "-Xlinker", "-rpath=$ORIGIN"])
     return LIB
 
 
