@@ -139,11 +139,12 @@ namespace {
 // longer than a launch.
 constexpr int64_t kSplitBytes = (int64_t)2 << 20;
 // Received matrices from this size on are located and decoded with one read: what the read saves has to pay for a run of the locator
-// on the sample, about 25 us.  Packed vectors need twice the fp64 operations per byte for the sum, and half as many coordinates
-// share the additions over the lanes: two reads / one, us: n = 45, s = 5, d = 500 k 83 / 85, 800 k 115 / 108, 1.5 M 193 / 147; n = 15,
-// s = 2, 1 M 59 / 67, 2 M 96 / 89, 4 M 160 / 126; n = 105, s = 2, 200 k 93 / 139, 400 k 147 / 132; packed n = 45, 2 M 126 / 133, 4 M
-// 233 / 192; and 60.2 M 6150 / 3490, packed 3180 / 2150.
-constexpr int64_t kOnePassBytes = (int64_t)256 << 20, kOnePassBytesPacked = (int64_t)512 << 20;
+// on the sample, 25 us at s <= 5, up to 60 at s = 7 with fewer than s adversaries (the singular-value iteration) and hundreds beyond,
+// where two reads stay.  Two reads / one, us: n = 45, s = 5, d = 935,000 (337 MB) 125 / 120, 1.5 M (540 MB) 193 / 147, 60.2 M 6150 / 3490; n = 9,
+// s = 3, 4.7 M (338 MB) 111 / 115, 10.5 M (753 MB) 251 / 198; n = 15, s = 2, 4 M (480 MB) 160 / 126; n = 105, s = 2, 400,000 (336 MB) 147 / 134, 800,000
+// 245 / 212; packed n = 45, s = 5, 2 M (360 MB) 126 / 133, 3 M (540 MB) 192 / 157, 60.2 M 3180 / 2150; but n = 45, s = 7, three adversaries,
+// 935,000 157 / 190.
+int64_t one_read_bytes(int s) { return s <= 5 ? (int64_t)512 << 20 : s <= 7 ? (int64_t)1 << 30 : INT64_MAX; }
 }
 
 extern "C" {
@@ -302,7 +303,7 @@ int draco_locate_decode(draco_plan* plan, const void* R, const float* f, uint8_t
     // projection, then syndromes / solve / support / decode vector in one launch, then the recovery
     if (!f || !aligned16(f)) return DRACO_EINVAL;
     const int64_t len = vec_len(plan);
-    const bool once = 8 * plan->n * len >= (is_packed(plan) ? kOnePassBytesPacked : kOnePassBytes);      // the projection and, most probably, the recovery in one
+    const bool once = 8 * plan->n * len >= one_read_bytes(plan->s);      // the projection and, most probably, the recovery in one
     int rc;
     if (once) {
         rc = launch_cyc_sample(plan, (const float2*)R, f, len, len, st);

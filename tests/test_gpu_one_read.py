@@ -6,8 +6,8 @@ import torch
 pytestmark = pytest.mark.gpu
 
 # just above the size from which on one read is tried; rows on and off the 16-byte grid, ragged last chunks, few and many rows
-SHAPES = [("CYC", 15, 2, 2_240_000), ("CYC", 15, 2, 2_240_003), ("CYC", 3, 1, 11_300_130), ("CYC", 45, 5, 746_002), ("CYC", 45, 3, 746_001),
-          ("CYC", 105, 2, 320_300), ("CYC", 128, 1, 263_001), ("CYC_PACKED", 15, 2, 8_960_008), ("CYC_PACKED", 45, 3, 2_984_003),
+SHAPES = [("CYC", 15, 2, 4_480_000), ("CYC", 15, 2, 4_480_003), ("CYC", 3, 1, 22_400_130), ("CYC", 45, 5, 1_492_002), ("CYC", 45, 3, 1_492_001),
+          ("CYC", 105, 2, 640_300), ("CYC", 128, 1, 525_001), ("CYC", 16, 7, 8_400_002), ("CYC_PACKED", 15, 2, 8_960_008), ("CYC_PACKED", 45, 3, 2_984_003),
           ("CYC_PACKED", 45, 3, 2_984_130)]
 
 
@@ -67,7 +67,7 @@ def test_one_read_is_the_separate_calls(code, n, s, d, attack):
 
 
 def test_one_read_replays_from_a_graph_with_other_adversaries():
-    code, n, s, d = "CYC", 15, 2, 2_240_000
+    code, n, s, d = "CYC", 15, 2, 4_480_000
     dr, plan, G, Z, f, _, v = _setup(code, n, s, d, 5)
     flags = torch.zeros(n, dtype=torch.uint8, device="cuda")
     u, R = torch.zeros(d, dtype=torch.float32, device="cuda"), Z.clone()
