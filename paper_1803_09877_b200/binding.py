@@ -1,4 +1,5 @@
-"""Binding of libdraco.so: argument marshalling only, by ctypes, and natively (``csrc/native.cpp``) for the calls of a training loop.
+"""Binding of libdraco.so: argument marshalling only, by ctypes, and natively (``csrc/native.cpp``) for the calls of a training loop
+where that module was built for the running interpreter.
 
 Every function takes raw device pointers (``tensor.data_ptr()``) or torch
 tensors and a CUDA stream handle; PyTorch is used by callers for device memory
@@ -7,7 +8,10 @@ and streams, never for arithmetic on the path.
 from __future__ import annotations
 
 import ctypes as C
+import importlib.util
 import os
+import sysconfig
+import warnings
 
 REP, CYC, CYC_PACKED = 0, 1, 2
 ADV_REVGRAD, ADV_CONST, ADV_GAUSS = 0, 1, 2
@@ -123,11 +127,46 @@ def _stream(stream):
     return stream.cuda_stream
 
 
+class _CtypesCalls:
+    """The calls of csrc/native.cpp through ctypes."""
+
+    @staticmethod
+    def encode(plan, G, Z, stream):
+        return _check(lib.draco_encode(plan, _ptr(G), _ptr(Z), _stream(stream)))
+
+    @staticmethod
+    def locate(plan, R, f, flags, stream):
+        return _check(lib.draco_locate(plan, _ptr(R), _ptr(f), _ptr(flags), _stream(stream)))
+
+    @staticmethod
+    def decode(plan, R, flags, u, stream):
+        return _check(lib.draco_decode(plan, _ptr(R), _ptr(flags), _ptr(u), _stream(stream)))
+
+    @staticmethod
+    def decode_update(plan, R, flags, w, scale, stream):
+        return _check(lib.draco_decode_update(plan, _ptr(R), _ptr(flags), _ptr(w), scale, _stream(stream)))
+
+    @staticmethod
+    def locate_decode(plan, R, f, flags, u, stream):
+        return _check(lib.draco_locate_decode(plan, _ptr(R), _ptr(f), _ptr(flags), _ptr(u), _stream(stream)))
+
+    @staticmethod
+    def set_current_stream(raw, device):
+        pass
+
+
 def _load_native():
+    """The module that was built for this interpreter, by its full name; without it ctypes makes the same calls."""
+    path = os.path.join(_PKG, "_native" + sysconfig.get_config_var("EXT_SUFFIX"))
+    if not os.path.exists(path):
+        return _CtypesCalls
     try:
-        from . import _native as module
+        spec = importlib.util.spec_from_file_location(f"{__package__}._native", path)
+        module = importlib.util.module_from_spec(spec)
+        spec.loader.exec_module(module)
     except ImportError as e:
-        raise DracoError(f"{_PKG}/_native.so cannot be loaded: build it with `python -m paper_1803_09877_b200.build`") from e
+        warnings.warn(f"{path} cannot be loaded ({e}): ctypes makes its calls", RuntimeWarning)
+        return _CtypesCalls
     module.set_functions(_check, _stream)
     return module
 

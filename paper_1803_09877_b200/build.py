@@ -14,7 +14,9 @@ CSRC = os.path.join(PKG, "csrc")
 INCLUDE = os.path.join(ROOT, "include")
 OBJ = os.path.join(PKG, "_build")
 LIB = os.path.join(PKG, "libdraco.so")
-NATIVE = os.path.join(PKG, "_native.so")          # the CPython module of the calls that a training loop makes
+# The CPython module of the calls that a training loop makes, named after the interpreter that it is built for: another one neither
+# loads it nor takes it for up to date.
+NATIVE = os.path.join(PKG, "_native" + sysconfig.get_config_var("EXT_SUFFIX"))
 
 SOURCES = ["draco_api.cu", "rep_kernels.cu", "cyc_encode.cu", "cyc_locate.cu", "cyc_onepass.cu", "cyc_recover.cu", "harness_kernels.cu"]
 NVCC_FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
@@ -62,9 +64,13 @@ def build(force: bool = False, verbose: bool = False) -> str:
     if force or jobs or _stale(LIB, objs):
         run([nvcc, "-shared", "-o", LIB] + objs + ["-lcudart"])
     src = os.path.join(CSRC, "native.cpp")
+    python_include = sysconfig.get_paths()["include"]
     if force or _stale(NATIVE, [src, headers[0]]):
-        run([nvcc, "-shared", "-O3", "-std=c++17", "-Xcompiler", "-fPIC", "-I", INCLUDE, "-I", sysconfig.get_paths()["include"], src,
-             "-o", NATIVE, "-L", PKG, "-Xlinker", "-l:libdraco.so", "-Xlinker", "-rpath=$ORIGIN"])
+        if os.path.exists(os.path.join(python_include, "Python.h")):
+            run([nvcc, "-shared", "-O3", "-std=c++17", "-Xcompiler", "-fPIC", "-I", INCLUDE, "-I", python_include, src,
+                 "-o", NATIVE, "-L", PKG, "-Xlinker", "-l:libdraco.so", "-Xlinker", "-rpath=$ORIGIN"])
+        else:
+            sys.stderr.write(f"no Python.h in {python_include}: {os.path.basename(NATIVE)} is not built, ctypes makes its calls\n")
     return LIB
 
 
