@@ -180,7 +180,8 @@ int draco_decode_update(draco_plan* plan, const void* R, const uint8_t* flags, f
  * reduction of the block partials) when the projection ran on more than 64 blocks.  Received matrices of 512 MB and
  * more (s = 6 and 7: 1 GB; not beyond) are read once instead of twice: the locator first runs on a sample of the columns, one
  * kernel then projects all of R and combines its rows for the V of the sample, and the locator runs on the whole projection.
- * V comes from all coordinates in any case; where the sample's V was another, the recovery reads R again.  f as in draco_locate. */
+ * V comes from all coordinates in any case; where the sample's V was another, the recovery reads R again.  u may share memory with
+ * f (the two reads are then kept).  f as in draco_locate. */
 int draco_locate_decode(draco_plan* plan, const void* R, const float* f, uint8_t* flags, float* u, void* stream);
 
 /* Repetition code with the selections exposed: maj (device [groups][d] fp32, may be NULL) receives

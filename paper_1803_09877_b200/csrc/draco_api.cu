@@ -145,6 +145,11 @@ constexpr int64_t kSplitBytes = (int64_t)2 << 20;
 // 245 / 212; packed n = 45, s = 5, 2 M (360 MB) 126 / 133, 3 M (540 MB) 192 / 157, 60.2 M 3180 / 2150; but n = 45, s = 7, three adversaries,
 // 935,000 157 / 190.
 int64_t one_read_bytes(int s) { return s <= 5 ? (int64_t)512 << 20 : s <= 7 ? (int64_t)1 << 30 : INT64_MAX; }
+
+bool overlap(const void* a, int64_t a_bytes, const void* b, int64_t b_bytes) {
+    const uintptr_t x = reinterpret_cast<uintptr_t>(a), y = reinterpret_cast<uintptr_t>(b);
+    return x < y + (uintptr_t)b_bytes && y < x + (uintptr_t)a_bytes;
+}
 }
 
 extern "C" {
@@ -303,7 +308,11 @@ int draco_locate_decode(draco_plan* plan, const void* R, const float* f, uint8_t
     // projection, then syndromes / solve / support / decode vector in one launch, then the recovery
     if (!f || !aligned16(f)) return DRACO_EINVAL;
     const int64_t len = vec_len(plan);
-    const bool once = 8 * plan->n * len >= one_read_bytes(plan->s);      // the projection and, most probably, the recovery in one
+    // The projection and, most probably, the recovery in one.  u is then written while f and R are read and before the flags are:
+    // a u that shares memory with one of them is left for the separate recovery, which comes after all three.
+    const int64_t u_bytes = 4 * plan->d, R_bytes = 8 * plan->n * len;
+    const bool once = R_bytes >= one_read_bytes(plan->s) && !overlap(u, u_bytes, f, 4 * len) && !overlap(u, u_bytes, R, R_bytes) &&
+                      !overlap(u, u_bytes, flags, plan->n);
     int rc;
     if (once) {
         rc = launch_cyc_sample(plan, (const float2*)R, f, len, len, st);

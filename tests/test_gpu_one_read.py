@@ -24,6 +24,15 @@ def _setup(code, n, s, d, seed):
     return dr, plan, G, Z, f, nodes, v
 
 
+def _separately(dr, plan, Z, f):
+    """flags, u, info and b of the separate calls on a plan of their own."""
+    other = dr.Plan(plan.n, plan.s, plan.d, plan.code)
+    flags, u = torch.empty(plan.n, dtype=torch.uint8, device="cuda"), torch.empty(plan.d, dtype=torch.float32, device="cuda")
+    other.locate(Z, f, flags)
+    other.decode(Z, flags, u)
+    return flags, u, other.info(), other.cyc_decode_vector()
+
+
 def _same(u, u2):
     """Both sum in fp64 and round once: an entry may fall on either side of a rounding boundary, 2^-23 of it."""
     return bool(((u - u2).abs() <= 2.0 ** -23 * u2.abs() + 1e-12 * u2.abs().max()).all())
@@ -88,3 +97,22 @@ def test_one_read_replays_from_a_graph_with_other_adversaries():
         torch.cuda.synchronize()
         assert torch.nonzero(flags).flatten().tolist() == nodes
         assert float((u.double() - sums).abs().max() / sums.abs().max()) <= 1e-5
+
+
+@pytest.mark.parametrize("shift", [0, 64, 1000, -64])
+@pytest.mark.parametrize("code,n,s,d", [("CYC", 15, 2, 4_480_000), ("CYC_PACKED", 45, 3, 2_984_130)])
+def test_sum_may_take_the_place_of_the_projection_vector(code, n, s, d, shift):
+    """u in f's memory: every coordinate of f has to be read before the first of u is written."""
+    dr, plan, G, Z, f, nodes, v = _setup(code, n, s, d, 3 * n + s)
+    plan.corrupt(Z, nodes, [dr.ADV_CONST] * s, [1e4] * s)
+    flags = torch.zeros(n, dtype=torch.uint8, device="cuda")
+    flags2, u2, want, _ = _separately(dr, plan, Z, f)
+    buf = torch.empty(v + d + 2000, dtype=torch.float32, device="cuda")
+    buf[1000:1000 + v] = f
+    u = buf[1000 + shift:1000 + shift + d]
+    plan.locate_decode(Z, buf[1000:1000 + v], flags, u)
+    info = plan.info()
+    assert torch.nonzero(flags).flatten().tolist() == nodes and torch.equal(flags, flags2)
+    # the projection is that of f as it was given: the same kernel, the same bits
+    assert (info["max_syndrome"], info["scale"], info["locator_margin"]) == (want["max_syndrome"], want["scale"], want["locator_margin"])
+    assert torch.equal(u, u2)
