@@ -227,6 +227,10 @@ int draco_cyc_project_noalloc(int n, int64_t d, const void* R, const float* f, d
 /* The decode vector b of the last cyclic decode (host [n][2] doubles); synchronises the stream. */
 int draco_cyc_decode_vector(draco_plan* plan, double* b_host /*host*/, void* stream);
 
+/* How often a cyclic plan's last draco_locate_decode read all of R: 1 where the sample's V stood, else 2 (0: none yet).
+ * Synchronises the stream. */
+int draco_cyc_reads(draco_plan* plan, int* reads /*host*/, void* stream);
+
 /* Copies the device-side results of the last calls to host memory; synchronises the stream. */
 int draco_get_info(draco_plan* plan, draco_info* info /*host*/, void* stream);
 

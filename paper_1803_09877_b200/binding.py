@@ -67,6 +67,7 @@ _SIGS = {
     "draco_cyc_locate_from_projection": ([_vp, _vp, _vp, _vp], _i),
     "draco_cyc_project_noalloc": ([_i, _i64, _vp, _vp, _vp, _vp], _i),
     "draco_cyc_decode_vector": ([_vp, C.POINTER(C.c_double), _vp], _i),
+    "draco_cyc_reads": ([_vp, C.POINTER(_i), _vp], _i),
     "draco_get_info": ([_vp, C.POINTER(DracoInfo), _vp], _i),
     "draco_pipeline_host": ([_vp, _vp, _vp, C.POINTER(_i), C.POINTER(_i), C.POINTER(_f), _i, _u64, _vp, _vp, _vp,
                              C.POINTER(DracoInfo)], _i),
@@ -256,6 +257,11 @@ class Plan:
         _check(lib.draco_cyc_decode_vector(self._h, buf, _stream(stream)))
         a = np.frombuffer(buf, dtype=np.float64).reshape(self.n, 2)
         return a[:, 0] + 1j * a[:, 1]
+
+    def cyc_reads(self, stream=None) -> int:
+        reads = _i()
+        _check(lib.draco_cyc_reads(self._h, C.byref(reads), _stream(stream)))
+        return reads.value
 
     def info(self, stream=None) -> dict:
         out = DracoInfo()

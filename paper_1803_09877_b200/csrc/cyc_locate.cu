@@ -1336,11 +1336,11 @@ cyc_solve_kernel(CycDevice* cd, const double2* __restrict__ e_in, const double2*
     if (with_b) {                                          // the decode vector for the V just found, same launch
         __syncthreads();
         decode_vector_body(cd, fl_s, tw, n, s, mod, rsn, info);
-        if (sample != nullptr) {                           // u has been written for the sample's V, if that was beyond doubt
+        if (sample != nullptr) {                           // u has been written for the sample's V, if there was a decode vector
             const int differ = __syncthreads_count(tid < n && fl_s[tid] != sample_flags[tid]);
             if (tid == kSolveThreads - 1) {
                 info->combine = info->n_active;
-                if (differ == 0 && sample->status == DRACO_OK) {
+                if (differ == 0 && sample->status != DRACO_ETOOMANY) {
                     info->im_residual_bits = sample->im_residual_bits;
                     info->re_max_bits = sample->re_max_bits;
                     info->combine = -1;

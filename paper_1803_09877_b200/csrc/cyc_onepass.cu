@@ -6,8 +6,9 @@
 // whole projection (e, q) and the sum that the sample's decode vector gives.  The locator runs again on the whole projection: V
 // comes from all coordinates, as ever.  Where it is the sample's V, the sum is the one that the recovery would have formed and the
 // recovery kernel returns at once; where it is not (an adversary that leaves the sampled columns alone), the recovery overwrites it
-// with the sum for the right V, at the cost of the second read that was to be saved.  A sample whose own locator is in doubt (status
-// other than DRACO_OK) is not acted on: the kernel then only projects.
+// with the sum for the right V, at the cost of the second read that was to be saved.  A sample in doubt (DRACO_EUNSURE: adversaries
+// side by side from s = 5 on) is acted on like any other: only the comparison of V with V' says whether the sum stands.  Where the
+// sample has more than 2 s nodes flagged there is no decode vector and the kernel only projects.
 //
 // Bound by HBM: 8 n + 4 bytes read and 4 written per coordinate (packed: per complex coordinate, 8 written).  Locate and decode, two
 // reads / one: n = 45, s = 5, d = 60.2 M 6150 -> 3490 us (6.3 TB/s; with back-to-back passes 6300 -> 3640), packed 3180 -> 2150; d =
@@ -109,7 +110,7 @@ cyc_onepass_kernel(const float2* __restrict__ R, const float* __restrict__ f, in
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     Sums* const acc_all = reinterpret_cast<Sums*>(smem + kWarps * kRing);
     Sums* const acc = acc_all + warp * n;
-    const bool go = sample->status == DRACO_OK;
+    const bool go = sample->status != DRACO_ETOOMANY;
     for (int j = threadIdx.x; j < n; j += kThreads) {
         bs[j] = cd->b[j];
         use[j] = go && !flags[j];

@@ -313,6 +313,7 @@ int draco_locate_decode(draco_plan* plan, const void* R, const float* f, uint8_t
     const int64_t u_bytes = 4 * plan->d, R_bytes = 8 * plan->n * len;
     const bool once = R_bytes >= one_read_bytes(plan->s) && !overlap(u, u_bytes, f, 4 * len) && !overlap(u, u_bytes, R, R_bytes) &&
                       !overlap(u, u_bytes, flags, plan->n);
+    plan->reads = once ? 1 : 2;
     int rc;
     if (once) {
         rc = launch_cyc_sample(plan, (const float2*)R, f, len, len, st);
@@ -330,6 +331,18 @@ int draco_cyc_decode_vector(draco_plan* plan, double* b_host, void* stream) {
     cudaStream_t st = (cudaStream_t)stream;
     DRACO_CUDA(cudaMemcpyAsync(b_host, plan->cyc_dev->b, sizeof(double2) * plan->n, cudaMemcpyDeviceToHost, st));
     DRACO_CUDA(cudaStreamSynchronize(st));
+    return DRACO_OK;
+}
+
+int draco_cyc_reads(draco_plan* plan, int* reads, void* stream) {
+    if (!plan || !is_cyc(plan) || !reads) return DRACO_EINVAL;
+    *reads = plan->reads;
+    if (plan->reads != 1) return DRACO_OK;
+    cudaStream_t st = (cudaStream_t)stream;
+    int32_t combine;
+    DRACO_CUDA(cudaMemcpyAsync(&combine, &plan->info_dev->combine, sizeof(combine), cudaMemcpyDeviceToHost, st));
+    DRACO_CUDA(cudaStreamSynchronize(st));
+    if (combine >= 0) *reads = 2;
     return DRACO_OK;
 }
 

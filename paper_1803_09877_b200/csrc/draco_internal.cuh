@@ -84,6 +84,7 @@ struct draco_plan {
     double2* partial_dev;             // [project_grid][n]
     int project_grid;                 // capacity of partial_dev in blocks
     int project_used;                 // blocks whose partials the plan's last projection (all its chunks) filled
+    int reads;                        // of R by the last draco_locate_decode: 0 none yet, 2, or 1: one, if `combine` is negative
     uint8_t* flags_dev;               // [2 kMaxN] internal flags, and those of the sample
     uint32_t* mask_dev;               // repetition: the vote's scratch, zero between calls
     // host-buffer pipeline (allocated on its first call)
