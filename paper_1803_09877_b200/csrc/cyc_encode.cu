@@ -37,6 +37,8 @@
 // 5.79 ms, five fp64 taps 6.02 ms.  The real centre tap (one fp64 operation per coordinate less) took the unpacked encoder from
 // 6.21 to 6.13 ms at s = 5 and from 7.39 to 7.27 ms at s = 7.  In a loop of launches the power cap lowers the clock: unpacked,
 // s = 5, 5.6 ms at 1965 MHz, 6.3 at 1665; packed 5.0 and 5.4 at 1820.
+#include <math.h>
+
 #include "draco_internal.cuh"
 
 namespace draco {
@@ -608,15 +610,46 @@ cyc_encode_generic_kernel(const float* __restrict__ G, float2* __restrict__ Z, i
     }
 }
 
-// Outputs per thread of the short kernels, 0: the walking kernels.  warps: what one output row takes.  One output each while that gives
-// an SM no more than 16 warps (n = 45, d = 4096), else four, up to 600 warps of outputs per SM on aligned rows, 300 (most) off the
-// grid, where the others catch up.  Walking / one / four outputs, us, the caller's 3.4 a call included: n = 45, s = 5, d = 4096 22.0 /
-// 3.4 / 3.4, 30,000 22.5 / 5.9 / 6.2, 100,000 22.5 / 15 / 11.4, 200,000 (630 warps) 22.7 / 30 / 21.3; n = 15, s = 2, 60,000 9.3 / 3.8 / 5.9,
-// 200,000 9.5 / 7.8 / 7.1; n = 105, s = 3, 100,000 (550) 40 / 28 / 22.5, 200,000 42 / 59 / 45; packed n = 45, s = 5, 120,000 22 / 18 / 12;
-// off the grid n = 45, s = 5, 30,003 (140) 14.9 / 8.9 / 6.5, 60,003 (290) 15.7 / 16 / 11.3, 100,003 (480) 16.8 / 26 / 17.5.
-int short_outputs(const draco_plan* p, int64_t warps, int64_t most) {
-    const int64_t all = warps * p->n, sms = p->sm_count;
-    return all <= 16 * sms ? 1 : all <= most * sms ? 4 : 0;
+// Outputs per thread of the short kernels, 0: the walking kernels.  warps: what one output row takes.  The short kernels' time grows
+// with the warps of outputs per SM (`each`) and with s, whatever n is; a walk takes its n + 2 s steps, however short the vector.  One
+// output each while that gives an SM no more than 16 warps.  Beyond, four outputs each do a third to half of the work, but are not below
+// 6 us from 34 (s = 5) to 68 warps on, where one output each is ahead up to 110 - 10 s warps.  Walking / one / four outputs, us, the
+// caller's 2.6 a call included: n = 45, s = 5, 34 warps 22 / 3.6 / 3.7, 68 22.5 / 5.7 / 6.3, 203 22.6 / 13 / 10, 405 22.7 / 26 / 18, 581 43 / 39 / 26; n = 5,
+// s = 1, 68 4.6 / 4.2 / 5.9, 300 10.2 / 13 / 9.8; n = 9, s = 3, 68 6.1 / 5.0 / 6.7.  Up to 600 warps, but the walk where
+//   * it has only one row (nothing is read twice; n = 1, 7.7 M 13.0 / 16.7 / 16.6, packed 12.1 / 16.6 / 16.5);
+//   * packed vectors with s = 3, 4 (all fp64: every output repeats its rows' conversions) have few rows: n = 9, s = 3, 581 22.9 / 27 / 24.5,
+//     n = 17, s = 4, 405 18.2 / 24 / 21 (n = 45, s = 3, 581 33 / 28 / 24);
+//   * all its strips are under way at once (12 an SM) and the outputs are many beside its steps (s >= 3, from 9 (n + 2 s) on).
+int short_outputs(const draco_plan* p, int64_t warps, bool packed) {
+    const int64_t sms = p->sm_count, n = p->n, s = p->s, all = warps * n;
+    const auto each_up_to = [&](int64_t most) { return all <= most * sms; };
+    if (each_up_to(16)) return 1;
+    if (!each_up_to(600)) return 0;
+    if (n == 1) return each_up_to(packed ? 100 : 140) ? 1 : 0;
+    if (s == 0) return 4;
+    if (each_up_to(110 - 10 * s)) return 1;
+    if (packed && (s == 3 || s == 4) && n <= 20 && !each_up_to(300)) return 0;
+    if (s >= 3 && warps <= 12 * sms && !each_up_to(9 * (n + 2 * s))) return 0;
+    return 4;
+}
+// The same off the 16-byte grid, up to 300 warps of outputs per SM; blocks, resident: what the walk takes of its blocks, and how many an
+// SM holds.  Up to 60 warps (s = 1: 80) the short kernels are ahead, one output each from s = 4 on (n = 45, s = 5, 51 warps, walking / one / four
+// 8.1 / 4.3 / 6.6; s = 1 7.3 / 2.9 / 2.9, the caller's 2.9 included).  Beyond, four outputs are compared with the walk by what either
+// was measured to take in us: n = 9, s = 4, 100 warps 4.6 / 6.0 / 6.3, 291 8.3 / 14 / 10.6; n = 21, s = 5, 203 9.6 / 12 / 8.7, 291 9.7 / 17 / 11.6; n = 45,
+// s = 5, 291 15.8 / 17 / 11.3.
+int short_outputs_fir(const draco_plan* p, int64_t warps, int64_t blocks, int resident, bool packed) {
+    const int64_t sms = p->sm_count, all = warps * p->n;
+    const double each = (double)all / (double)sms, s = p->s, steps = p->n + 2 * p->s;
+    if (each <= 16.0) return 1;
+    if (each > 300.0) return 0;
+    if (each <= 60.0) return p->s >= 4 ? 1 : 4;
+    if (p->s == 1 && each <= 80.0) return 4;
+    const double rounds = (double)((blocks + sms * resident - 1) / (sms * resident));
+    const double step = packed ? (p->s <= 2 ? 0.40 : p->s == 3 ? 0.33 : 0.29) : (p->s <= 2 ? 0.36 : 0.27);
+    const double walk = fmax(3.6, step * steps) * (1.0 + (packed ? 1.0 : 0.6) * (rounds - 1.0));
+    const double four = packed ? fmax(4.3 + 0.45 * s, each * (0.0135 + 0.0048 * s))
+                               : fmax(p->s > 1 ? 4.7 + 0.45 * s : 4.7, each * (0.016 + 0.0045 * s));
+    return walk < four ? 0 : 4;
 }
 
 template <int S, bool PACKED, bool REALC = true>
@@ -626,7 +659,7 @@ int launch_stream(const draco_plan* p, const float* G, float2* Z, int64_t len, i
     constexpr int kThreads = Cfg::kThreads;
     constexpr int kStrip = PACKED ? 64 : 128;
     const int64_t nstrips = (len + kStrip - 1) / kStrip;
-    const int outputs = short_outputs(p, nstrips, 600);
+    const int outputs = short_outputs(p, nstrips, PACKED);
     if (outputs > 0) {
 #define DRACO_SHORT(J) launch_dependent(cyc_encode_short_kernel<S, PACKED, REALC, J>, dim3((unsigned)((nstrips + kShortWarps - 1) / kShortWarps), (unsigned)((p->n + J - 1) / J)), \
                                         32 * kShortWarps, 0, st, G, Z, len, ldg, ldz, half, p->n, p->taps, p->taps64, p->phase64)
@@ -681,7 +714,8 @@ int launch_fir(const draco_plan* p, const float* G, float2* Z, int64_t len, int6
     using Cfg = FirCfg<S, PACKED>;
     constexpr int kPer = Cfg::kThreads * Cfg::C;
     const int64_t nshort = (len + kPer - 1) / kPer;
-    const int outputs = short_outputs(p, nshort * (Cfg::kThreads / 32), 300);
+    const int64_t nstrips = (len + Cfg::kTile - 1) / Cfg::kTile;
+    const int outputs = short_outputs_fir(p, nshort * (Cfg::kThreads / 32), nstrips, Cfg::kBlocks, PACKED);
     if (outputs > 0) {
 #define DRACO_SHORT(J) launch_dependent(cyc_encode_fir_short_kernel<S, PACKED, J>, dim3((unsigned)nshort, (unsigned)((p->n + J - 1) / J)), Cfg::kThreads, 0, st, G, Z, len, ldg, ldz, \
                                         half, d_real, p->n, p->taps64, p->phase64)
@@ -690,7 +724,6 @@ int launch_fir(const draco_plan* p, const float* G, float2* Z, int64_t len, int6
         DRACO_CUDA(cudaGetLastError());
         return DRACO_OK;
     }
-    const int64_t nstrips = (len + Cfg::kTile - 1) / Cfg::kTile;
     int64_t grid = (int64_t)p->sm_count * Cfg::kBlocks;
     if (grid > nstrips) grid = nstrips;
     launch_dependent(cyc_encode_fir_kernel<S, PACKED>, (int)grid, Cfg::kThreads, 0, st, G, Z, len, ldg, ldz, half, d_real,
