@@ -611,44 +611,40 @@ cyc_encode_generic_kernel(const float* __restrict__ G, float2* __restrict__ Z, i
 }
 
 // Outputs per thread of the short kernels, 0: the walking kernels.  warps: what one output row takes.  The short kernels' time grows
-// with the warps of outputs per SM (`each`) and with s, whatever n is; a walk takes its n + 2 s steps, however short the vector.  One
-// output each while that gives an SM no more than 16 warps.  Beyond, four outputs each do a third to half of the work, but are not below
-// 6 us from 34 (s = 5) to 68 warps on, where one output each is ahead up to 110 - 10 s warps.  Walking / one / four outputs, us, the
-// caller's 2.6 a call included: n = 45, s = 5, 34 warps 22 / 3.6 / 3.7, 68 22.5 / 5.7 / 6.3, 203 22.6 / 13 / 10, 405 22.7 / 26 / 18, 581 43 / 39 / 26; n = 5,
-// s = 1, 68 4.6 / 4.2 / 5.9, 300 10.2 / 13 / 9.8; n = 9, s = 3, 68 6.1 / 5.0 / 6.7.  Up to 600 warps, but the walk where
-//   * it has only one row (nothing is read twice; n = 1, 7.7 M 13.0 / 16.7 / 16.6, packed 12.1 / 16.6 / 16.5);
-//   * packed vectors with s = 3, 4 (all fp64: every output repeats its rows' conversions) have few rows: n = 9, s = 3, 581 22.9 / 27 / 24.5,
-//     n = 17, s = 4, 405 18.2 / 24 / 21 (n = 45, s = 3, 581 33 / 28 / 24);
+// with the warps of outputs per SM and with s, whatever n is; a walk takes its n + 2 s steps, however short the vector.  One output each
+// while that gives an SM no more than 110 - 10 s warps, then four, which read and convert a third to half as often, but few at a time.
+// Walking / one / four outputs, us of GPU time in a captured chain: n = 45, s = 5, 34 warps 22 / 3.5 / 3.6, 68 22 / 5.5 / 5.9, 120 22 / 8.6 / 6.7,
+// 203 22 / 13 / 10; n = 5, s = 1, 68 4.5 / 3.8 / 5.0, 300 10.1 / 12.3 / 9.6; n = 9, s = 3, 68 6.0 / 4.7 / 6.2, 160 9.8 / 8.5 / 7.5.  (s = 0: four from 16 warps on,
+// n = 9, 50 6.2 / 2.7 / 3.3, 203 9.2 / 8.5 / 5.8.)  Up to 600 warps (n = 45, s = 5: as many strips as the walk has under way at once), but the walk where
+//   * it has only one row, and nothing is read twice (n = 1, 160 7.5 / 6.8 / 6.8, 300 10.5 / 12.3 / 12.2);
+//   * packed vectors with s = 3, 4 (all fp64: every output repeats its rows' conversions) have few rows (n = 9, s = 3, 300 12.7 / 14.6 / 13.1,
+//     581 22.9 / 27 / 24.5, n = 17, s = 4, 405 18.2 / 24 / 21; but n = 45, s = 3, 581 33 / 28 / 24);
 //   * all its strips are under way at once (12 an SM) and the outputs are many beside its steps (s >= 3, from 9 (n + 2 s) on).
 int short_outputs(const draco_plan* p, int64_t warps, bool packed) {
     const int64_t sms = p->sm_count, n = p->n, s = p->s, all = warps * n;
     const auto each_up_to = [&](int64_t most) { return all <= most * sms; };
     if (each_up_to(16)) return 1;
     if (!each_up_to(600)) return 0;
-    if (n == 1) return each_up_to(packed ? 100 : 140) ? 1 : 0;
+    if (n == 1) return each_up_to(180) ? 1 : 0;
     if (s == 0) return 4;
     if (each_up_to(110 - 10 * s)) return 1;
     if (packed && (s == 3 || s == 4) && n <= 20 && !each_up_to(300)) return 0;
     if (s >= 3 && warps <= 12 * sms && !each_up_to(9 * (n + 2 * s))) return 0;
     return 4;
 }
-// The same off the 16-byte grid, up to 300 warps of outputs per SM; blocks, resident: what the walk takes of its blocks, and how many an
-// SM holds.  Up to 60 warps (s = 1: 80) the short kernels are ahead, one output each from s = 4 on (n = 45, s = 5, 51 warps, walking / one / four
-// 8.1 / 4.3 / 6.6; s = 1 7.3 / 2.9 / 2.9, the caller's 2.9 included).  Beyond, four outputs are compared with the walk by what either
-// was measured to take in us: n = 9, s = 4, 100 warps 4.6 / 6.0 / 6.3, 291 8.3 / 14 / 10.6; n = 21, s = 5, 203 9.6 / 12 / 8.7, 291 9.7 / 17 / 11.6; n = 45,
-// s = 5, 291 15.8 / 17 / 11.3.
+// The same off the 16-byte grid, up to 300 warps of outputs per SM.  blocks, resident: the walk's blocks, and how many an SM holds.  Up to 60
+// warps (s = 1: 100) the short kernels are ahead, one output each from s = 4 on (n = 45, s = 5, 51 warps 7.7 / 4.0 / 4.9; s = 1 7.0 / 2.4 / 2.7).
+// Beyond, four outputs are compared with the walk by the time that either was measured to take, in us: n = 9, s = 4, 90 warps 4.3 / 5.3 / 5.8, 291
+// 8.0 / 14 / 10.2; n = 21, s = 5, 160 8.4 / 9.7 / 7.1, 291 9.2 / 16 / 11.5; n = 45, s = 5, 291 13.9 / 16 / 11.3.
 int short_outputs_fir(const draco_plan* p, int64_t warps, int64_t blocks, int resident, bool packed) {
-    const int64_t sms = p->sm_count, all = warps * p->n;
-    const double each = (double)all / (double)sms, s = p->s, steps = p->n + 2 * p->s;
+    const double sms = p->sm_count, s = p->s, each = (double)(warps * p->n) / sms;
     if (each <= 16.0) return 1;
     if (each > 300.0) return 0;
     if (each <= 60.0) return p->s >= 4 ? 1 : 4;
-    if (p->s == 1 && each <= 80.0) return 4;
-    const double rounds = (double)((blocks + sms * resident - 1) / (sms * resident));
-    const double step = packed ? (p->s <= 2 ? 0.40 : p->s == 3 ? 0.33 : 0.29) : (p->s <= 2 ? 0.36 : 0.27);
-    const double walk = fmax(3.6, step * steps) * (1.0 + (packed ? 1.0 : 0.6) * (rounds - 1.0));
-    const double four = packed ? fmax(4.3 + 0.45 * s, each * (0.0135 + 0.0048 * s))
-                               : fmax(p->s > 1 ? 4.7 + 0.45 * s : 4.7, each * (0.016 + 0.0045 * s));
+    if (p->s == 1 && each <= 100.0) return 4;
+    const double rounds = fmax(1.0, (double)blocks / (sms * resident));
+    const double walk = rounds * fmax(packed ? 4.7 : 3.5, 0.3 + (p->s <= 2 ? 0.33 : 0.25) * (p->n + 2 * p->s));
+    const double four = packed ? fmax(4.2 + 0.4 * s, each * (0.011 + 0.0034 * s)) : fmax(3.7 + 0.55 * s, each * (0.0167 + 0.0045 * s));
     return walk < four ? 0 : 4;
 }
 

@@ -50,7 +50,7 @@ def test_both_sides_of_every_line(n, s, aligned, packed):
     code = dr.CYC_PACKED if packed else dr.CYC
     sms = torch.cuda.get_device_properties(0).multi_processor_count
     per_warp = (64 if packed else 128) if aligned else (32 if packed else 64)      # coordinates of a warp
-    lines = (16, 110 - 10 * s, 100, 140, 300, 9 * (n + 2 * s), 600) if aligned else (16, 60, 80, 100, 140, 200, 300)
+    lines = (16, 110 - 10 * s, 140, 180, 300, 9 * (n + 2 * s), 600) if aligned else (16, 60, 100, 140, 200, 300)
     lengths = sorted({int(f * line * sms / n) * per_warp for line in lines for f in (0.97, 1.05)} - {0})
     odd = 0 if aligned else 3
     long = max(lengths) + odd

@@ -110,10 +110,11 @@ def test_sum_may_take_the_place_of_the_projection_vector(code, n, s, d, shift):
 
 
 @pytest.mark.parametrize("code,n,s,d,step", [("CYC", 33, 5, 2_033_700, 1), ("CYC", 105, 3, 640_300, 7), ("CYC", 45, 5, 1_492_002, 5),
-                                             ("CYC", 45, 5, 1_492_001, 11), ("CYC_PACKED", 45, 5, 2_984_130, 11)])
+                                             ("CYC", 45, 5, 1_492_001, 1), ("CYC_PACKED", 45, 5, 2_984_130, 11)])
 def test_samples_in_doubt(code, n, s, d, step):
     """Adversaries side by side: the first pass's margin may be below 10, V may hold an honest neighbour, and the sample's V may be
-    another.  Whichever it is, u, b and flags are those of the separate calls; at 33 nodes the passes nearly always find the same V."""
+    another.  Whichever it is, u, b and flags are those of the separate calls; at 33 nodes the passes nearly always find the same V, at 45,
+    where every sample is in doubt, in two placements of three (d odd; with doubtful samples passed over, in one of 45)."""
     dr, plan, G, Z, f, _, v = _setup(code, n, s, d, n + s)
     R, doubts, once, count = torch.empty_like(Z), 0, 0, 0
     for first in range(0, n, step):
@@ -129,7 +130,7 @@ def test_samples_in_doubt(code, n, s, d, step):
         doubts += info["locator_margin"] < 10.0
         once += reads == 1
         count += 1
-    assert doubts > 0 and (n != 33 or once > 0.8 * count)
+    assert doubts > 0 and once >= {33: 0.9, 45: 0.5}[n] * count if step == 1 else doubts > 0
 
 
 @pytest.mark.parametrize("code,n,s,d", [("CYC", 15, 2, 4_480_000), ("CYC", 45, 3, 1_492_001), ("CYC_PACKED", 45, 3, 2_984_130)])
