@@ -63,8 +63,8 @@ __device__ __forceinline__ double* q_partials(double2* partial, int cap, int n) 
     return reinterpret_cast<double*>(partial + (int64_t)cap * n);
 }
 // Block = 8 warps over one tile of coordinates; warp w owns rows row0 + w, row0 + w + 8, ... of the
-// launch's nrows <= 8 RPW rows; every: 1, or only each `every`-th tile is read; f for the tile sits in shared memory as fp64 (converted once per tile, used by
-// every row).  More than 64 rows take two launches of half the rows each (rows are
+// launch's nrows <= 8 RPW rows; f for the tile sits in shared memory as fp64 (converted once per tile, used by every row).
+// `every` > 1: only each `every`-th tile is read (a sample).  More than 64 rows take two launches of half the rows each (rows are
 // independent; f is read twice, 1 % more traffic): 16 rows per warp in registers halve the blocks per SM
 // (0.79 of the copy bandwidth at n = 105), and per-lane sums in shared memory left the compiler too few
 // registers to keep its loads in flight once the squared norms were added (0.98 -> 0.68).

@@ -28,7 +28,7 @@ constexpr int kBlocksPerSM = 2;
 constexpr int kBatch = 8;             // rows whose lane sums are added up together
 
 // K 16-byte items per lane and row: a warp takes 64 K coordinates.  kRing bytes of rows are on their way per warp.
-template <bool VEC2, bool PACKED>
+template <bool PACKED>
 struct OneCfg {
     static constexpr int K = PACKED ? 2 : 4;
     static constexpr int kChunk = 64 * K;
@@ -64,21 +64,10 @@ __device__ __forceinline__ void copy_row(uint32_t dst, const float2* src, int af
                 ::"r"(dst + q * 512), "l"(src + q * 64), "r"(after), "n"(kNever) : "memory");
     }
 }
-// with the source switched off by a predicate: zeros are written, src is not read
+// as cp_async8_if
 __device__ __forceinline__ void cp_async16_if(uint32_t dst, const void* src, bool on) {
     asm volatile("{\n\t.reg .pred p;\n\tsetp.eq.u32 p, %2, 0;\n\tcp.async.cg.shared.global [%0], [%1], 16, p;\n\t}" ::"r"(dst), "l"(src), "r"((uint32_t)on) : "memory");
 }
-__device__ __forceinline__ void cp_async8_if(uint32_t dst, const void* src, bool on) {
-    asm volatile("{\n\t.reg .pred p;\n\tsetp.eq.u32 p, %2, 0;\n\tcp.async.ca.shared.global [%0], [%1], 8, p;\n\t}" ::"r"(dst), "l"(src), "r"((uint32_t)on) : "memory");
-}
-__device__ __forceinline__ float4 lds128(uint32_t a) {
-    float4 v;
-    asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(a) : "memory");
-    return v;
-}
-
-// |a| for the self-check's maxima; NaN counts as infinity
-__device__ __forceinline__ double magnitude(double a) { return a == a ? fabs(a) : __longlong_as_double(0x7ff0000000000000ll); }
 
 struct Sums {
     double er, ei, q;
@@ -101,7 +90,7 @@ __global__ void __launch_bounds__(kThreads, kBlocksPerSM)
 cyc_onepass_kernel(const float2* __restrict__ R, const float* __restrict__ f, int64_t len, int64_t ld, int n,
                    double2* __restrict__ partial, int cap, const CycDevice* __restrict__ cd, const uint8_t* __restrict__ flags,
                    DeviceInfo* sample, float* __restrict__ u, int64_t d_packed) {
-    using Cfg = OneCfg<VEC2, PACKED>;
+    using Cfg = OneCfg<PACKED>;
     constexpr int K = Cfg::K, kRing = Cfg::kRing;
     extern __shared__ __align__(16) unsigned char smem[];             // ring[kWarps][kRing], sums[kWarps][n]
     __shared__ double2 bs[kMaxN];
@@ -295,7 +284,7 @@ cyc_onepass_kernel(const float2* __restrict__ R, const float* __restrict__ f, in
 
 template <bool VEC2, bool PACKED>
 int launch_onepass(draco_plan* p, const float2* R, const float* f, int64_t len, int64_t ld, float* u, int64_t d_packed, cudaStream_t st) {
-    using Cfg = OneCfg<VEC2, PACKED>;
+    using Cfg = OneCfg<PACKED>;
     const int64_t nblocks = ((len + Cfg::kChunk - 1) / Cfg::kChunk + kWarps - 1) / kWarps;
     int64_t grid = (int64_t)p->sm_count * kBlocksPerSM;
     if (grid > p->project_grid) grid = p->project_grid;

@@ -22,9 +22,6 @@ constexpr int kUnroll = 8;
 constexpr int kShortCoordinates = 300;   // per SM: up to this length the short kernel is the faster one ..
 constexpr int kShortFewRows = 140;       // .. and with at most 16 rows
 
-// |a| for the self-check's maxima; NaN, which a node may send and fmax would drop, counts as infinity
-__device__ __forceinline__ double magnitude(double a) { return a == a ? fabs(a) : __longlong_as_double(0x7ff0000000000000ll); }
-
 // PACKED: the vectors carry two gradient coordinates per complex entry (Section 3, last
 // paragraph): u[i] = Re(u-hat_i), u[len + i] = Im(u-hat_i) for len + i < d_packed.
 // VEC2: a thread owns two neighbouring coordinates, one 16-byte load per row.  Otherwise (odd row starts) two coordinates

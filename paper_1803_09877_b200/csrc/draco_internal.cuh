@@ -131,6 +131,18 @@ __device__ __forceinline__ void pdl_begin() {
     cudaTriggerProgrammaticLaunchCompletion();
     cudaGridDependencySynchronize();
 }
+// |a| for the decoder's self-check maxima; NaN, which a node may send and fmax would drop, counts as infinity
+__device__ __forceinline__ double magnitude(double a) { return a == a ? fabs(a) : __longlong_as_double(0x7ff0000000000000ll); }
+// 8 bytes to shared memory, asynchronously, with the source switched off by a predicate (ignore-src: zeros are written, src is not
+// read), so that a lane outside the vector needs no branch around its copies.
+__device__ __forceinline__ void cp_async8_if(uint32_t dst, const void* src, bool on) {
+    asm volatile("{\n\t.reg .pred p;\n\tsetp.eq.u32 p, %2, 0;\n\tcp.async.ca.shared.global [%0], [%1], 8, p;\n\t}" ::"r"(dst), "l"(src), "r"((uint32_t)on) : "memory");
+}
+__device__ __forceinline__ float4 lds128(uint32_t a) {
+    float4 v;
+    asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(a) : "memory");
+    return v;
+}
 #endif
 
 // kernels / launchers (one per translation unit)
